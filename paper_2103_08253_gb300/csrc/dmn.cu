@@ -132,6 +132,7 @@ TreeDev tree_dev(const Tree& t) {
   d.kid = t.d_tab ? t.d_tab + 4 * t.Lc + 3 * t.N : nullptr;
   d.hcid = t.d_tab ? t.d_tab + 4 * t.Lc + 5 * t.N : nullptr;
   d.kslot = t.d_tab ? t.d_tab + 4 * t.Lc + 5 * t.N + ((1 << t.K) - 1) : nullptr;
+  d.lslot = t.d_tab ? d.kslot + 2 * t.N : nullptr;
   return d;
 }
 
@@ -358,7 +359,17 @@ __global__ void k_tree_scatter(int64_t n, const int32_t* __restrict__ tid, int n
   if (b >= 0) perm[base + __popc(peers & ((1u << lane) - 1u))] = i;
 }
 
-// per point: normals and the macro strain in the principal frame
+// Small calls spread a point over several threads of k_prepare and k_final: enough threads for 1024 per
+// SM (a warp keeps 32 points side by side, so that the field-major arrays stay coalesced).  One thread
+// per point leaves most SMs idle: at 4096 points of depth 8 (128 warps on 152 SMs) each of the two
+// kernels took 0.61-0.63 ms, 15 times its share of the FP64 rate; split it takes 0.13 ms.  `most`: the
+// largest useful split.
+int64_t point_split(int64_t n, int n_sm, int64_t most) {
+  return std::max<int64_t>(1, std::min<int64_t>(most, (int64_t)1024 * n_sm / std::max<int64_t>(n, 1)));
+}
+
+// per point: normals and the macro strain in the principal frame.  blockIdx.y: the share of the
+// laminates (point_split); the first share also writes the strain.
 __global__ void k_prepare(Forest F, int64_t n, const int32_t* __restrict__ tid, const int64_t* __restrict__ perm,
                           const double* __restrict__ lam, const double* __restrict__ Q, const double* __restrict__ En,
                           const double* __restrict__ dE, double* __restrict__ nbuf, int N_max) {
@@ -368,7 +379,8 @@ __global__ void k_prepare(Forest F, int64_t n, const int32_t* __restrict__ tid, 
   int tr;
   point_of(perm, tid, F.n, i, p, tr);
   if (tr >= F.n) return;
-  point_normals(F.t[tr], lam[2 * p], lam[2 * p + 1], nbuf + p, (size_t)n);
+  point_normals(F.t[tr], lam[2 * p], lam[2 * p + 1], nbuf + p, (size_t)n, blockIdx.y, gridDim.y);
+  if (blockIdx.y) return;
   double E[6];
   local_strain(Q + 9 * p, En + 6 * p, dE + 6 * p, E);
 #pragma unroll
@@ -749,6 +761,8 @@ struct FinalParams {
   const double* nbuf;
 };
 
+// Without the sweep a point may be split over gridDim.y = 2^s threads (final_split), each of which takes
+// the leaves below one position of level s + 1; the first also rotates stress and tangent.
 template <bool SWEEP, bool CMP>
 __global__ void __launch_bounds__(128) k_final(FinalParams P) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -758,6 +772,8 @@ __global__ void __launch_bounds__(128) k_final(FinalParams P) {
   point_of(P.perm, P.tid, P.F.n, i, pt, tr);
   if (tr >= P.F.n) return;  // unknown tree: reported by the Newton kernel
   const TreeDev& t = P.F.t[tr];
+  const int part = SWEEP ? 0 : blockIdx.y, split = SWEEP ? 0 : min(31 - __clz((int)gridDim.y), t.K - 1);
+  if (part >> split) return;   // a shallower tree has fewer parts
   const int st = P.status[pt];
   double Eloc[6];
 #pragma unroll
@@ -769,7 +785,9 @@ __global__ void __launch_bounds__(128) k_final(FinalParams P) {
   A.a_out = A.a;
   A.paper = true;
   A.z = P.state_in + pt; A.zs = (size_t)P.n;
-  if (st == DMN_STATUS_NONFINITE) {
+  if (part > 0) {
+    // another thread's
+  } else if (st == DMN_STATUS_NONFINITE) {
     const double qnan = __longlong_as_double(0x7ff8000000000000LL);
     for (int I = 0; I < 6; ++I) P.stress[6 * pt + I] = qnan;
     for (int I = 0; I < 36; ++I) P.tangent[36 * pt + I] = qnan;
@@ -788,8 +806,17 @@ __global__ void __launch_bounds__(128) k_final(FinalParams P) {
     for (int k = 0; k < 21; ++k) C[k] = P.tangent[36 * pt + k];
     write_stress_tangent<double>(P.Q + 9 * pt, sb, C, P.stress + 6 * pt, P.tangent + 36 * pt);
   }
-  if (CMP) write_leaf_states_c(t, Eloc, A, P.state_out + pt, (size_t)P.n, st == DMN_STATUS_NONFINITE);
+  if (!SWEEP && split) write_leaf_states_part(t, Eloc, A, P.state_out + pt, (size_t)P.n, st == DMN_STATUS_NONFINITE, split, part);
+  else if (CMP) write_leaf_states_c(t, Eloc, A, P.state_out + pt, (size_t)P.n, st == DMN_STATUS_NONFINITE);
   else write_leaf_states(t, Eloc, A, P.state_out + pt, (size_t)P.n, st == DMN_STATUS_NONFINITE);
+}
+
+// threads per point of k_final without the sweep: a power of two, at most 32 (each thread walks from the
+// root to its part, s laminates it shares with others)
+unsigned final_split(int64_t n, int n_sm) {
+  unsigned y = 1;
+  while (2 * y <= 32 && 2 * y <= point_split(n, n_sm, 32)) y *= 2;
+  return y;
 }
 
 // ---------------------------------------------------------------------------
@@ -1078,7 +1105,8 @@ struct CmpTree {
   std::vector<double> p, q, c;   // p, q [N][M]; c = c1 [N], c2 [N], sc [N], leaf weights [L], 1 / (c1 c2) [N]
   std::vector<float> cf;         // c1f [N], c2f [N], c12f [N], scf [N], 1 / (c1 c2) [N]
   std::vector<int> tab;          // lf [Lc] (4 ints each), pre [N], post [N], paper index [N], children [2 N],
-                                 // the laminate at each heap position [2^K - 1], leaf children's state slots [2 N]
+                                 // the laminate at each heap position [2^K - 1], leaf children's state slots [2 N],
+                                 // the state slot of each leaf [2^K]
 };
 
 void build_compressed(const dmn_tree_desc& d, const bool inelastic[2], CmpTree& B) {
@@ -1173,6 +1201,7 @@ void build_compressed(const dmn_tree_desc& d, const bool inelastic[2], CmpTree& 
         if (x > N) kslot[2 * cid[h] + side] = slot_of[x - N - 1];
       }
   B.tab.insert(B.tab.end(), kslot.begin(), kslot.end());
+  B.tab.insert(B.tab.end(), slot_of.begin(), slot_of.end());
 }
 
 bool has_zero_weight(const dmn_tree_desc& d) {
@@ -1336,7 +1365,8 @@ int update_on(dmn_handle* h, WorkSet& w, int64_t n, int64_t n_call, const int32_
     k_tree_scatter<<<g1, 128, 0, s>>>(n, tree_id, F.n, w.counter + 10, w.perm);
     perm = w.perm;
   }
-  k_prepare<<<g1, 128, 0, s>>>(F, n, tree_id, perm, lam, Q, E_n, dE, w.nbuf, NM);
+  const dim3 gp(g1, (unsigned)point_split(n, h->n_sm, NM));
+  k_prepare<<<gp, 128, 0, s>>>(F, n, tree_id, perm, lam, Q, E_n, dE, w.nbuf, NM);
   if (ev) cudaEventRecord(ev[1], s);
   const unsigned grid = (unsigned)(h->n_sm * h->opt.ctas_per_sm);
   const bool mixed = h->opt.precision != DMN_PREC_F64;
@@ -1379,6 +1409,7 @@ int update_on(dmn_handle* h, WorkSet& w, int64_t n, int64_t n_call, const int32_
     else launch_newton<float, false>(P, ls, minb, grid, block, s);
   }
   if (ev) cudaEventRecord(ev[3], s);
+  const dim3 gf(g1, final_split(n, h->n_sm));
   FinalParams FP{F, n, NM, tree_id, perm, Q, state_in, state_out, stress, tangent, status, w.nbuf};
   if (sweep && warp) {   // the FP64 sweep in the warp organisation (counter [20]), then k_final rotates
     NewtonParams<double> SP{F, n, h->nslots, NM, tree_id, perm, state_in, state_out, stress, tangent, iters, status,
@@ -1387,14 +1418,14 @@ int update_on(dmn_handle* h, WorkSet& w, int64_t n, int64_t n_call, const int32_
     const int swl = h->opt.warp_lanes ? h->opt.warp_lanes : (n_call <= 16 * (int64_t)h->n_sm ? 32 : 8);
     if (h->cmp) launch_sweep_warp<true>(SP, swl, wgrid, w.scr_w, s);
     else launch_sweep_warp<false>(SP, swl, wgrid, w.scr_w, s);
-    if (h->cmp) k_final<false, true><<<g1, 128, 0, s>>>(FP);
-    else k_final<false, false><<<g1, 128, 0, s>>>(FP);
+    if (h->cmp) k_final<false, true><<<gf, 128, 0, s>>>(FP);
+    else k_final<false, false><<<gf, 128, 0, s>>>(FP);
   } else if (sweep) {
     if (h->cmp) k_final<true, true><<<g1, 128, 0, s>>>(FP);
     else k_final<true, false><<<g1, 128, 0, s>>>(FP);
   } else {
-    if (h->cmp) k_final<false, true><<<g1, 128, 0, s>>>(FP);
-    else k_final<false, false><<<g1, 128, 0, s>>>(FP);
+    if (h->cmp) k_final<false, true><<<gf, 128, 0, s>>>(FP);
+    else k_final<false, false><<<gf, 128, 0, s>>>(FP);
   }
   if (ev) cudaEventRecord(ev[4], s);
   e = cudaGetLastError();

@@ -87,6 +87,7 @@ struct TreeDev {
   const int* kid;    // [2 N] children of each laminate: >= 0 a laminate, -1 - phase a leaf
   const int* hcid;   // [2^K - 1] the laminate standing at each heap position, -1 for none (compressed trees)
   const int* kslot;  // [2 N] the state slot of each child that is a leaf (-1: elastic, or a laminate child)
+  const int* lslot;  // [2^K] the state slot of each leaf (-1: elastic, or of weight zero)
 };
 
 // fields of TreeDev::lf .w
@@ -1111,6 +1112,70 @@ __device__ inline void write_leaf_states(const TreeDev& t, const double Eloc[6],
       load_z(t, P, leaf, side, z);
       leaf_iso<double>(t.ph[side], side ? eR : eL, z, sig, nullptr, zn, nullptr);
       const int slot = t.z_both ? leaf : (leaf >> 1);
+      double* b = zout + (size_t)(6 * slot) * zos;
+#pragma unroll
+      for (int c = 0; c < 6; ++c) b[c * zos] = nan_out ? __longlong_as_double(0x7ff8000000000000LL) : zn[c];
+    }
+  }
+}
+
+// The part of write_leaf_states (heap trees) or write_leaf_states_c (compressed ones) below position
+// `part` of level s + 1, s = 1 .. K - 1: the strain is carried from the root to that position (the same
+// operations as in the whole walk, so the states are the same), then depth first through the subtree.
+// Compressed trees are walked by heap positions: one that holds no laminate hands its strain on.
+__device__ inline void write_leaf_states_part(const TreeDev& t, const double Eloc[6], const PointArrays& P,
+                                              double* zout, size_t zos, bool nan_out, int s, int part) {
+  const int K = t.K;
+  double epsR[KMAX + 1][6], e[6], eL[6], eR[6];
+  auto split = [&](int lvl, int at) {   // strains of the children of position `at` of level lvl
+    const int pos = (1 << (lvl - 1)) + at - 1;
+    const int node = t.hcid ? __ldg(t.hcid + pos) : pos;
+    if (node < 0) {
+#pragma unroll
+      for (int I = 0; I < 6; ++I) eL[I] = eR[I] = e[I];
+      return;
+    }
+    const double nd[3] = {P.nrm[(3 * node) * P.ns], P.nrm[(3 * node + 1) * P.ns], P.nrm[(3 * node + 2) * P.ns]};
+    const double c1 = __ldg(t.c1 + node), c2 = __ldg(t.c2 + node);
+    const double* ap = P.a + (size_t)(3 * (t.hcid ? node : jump_index(P, K, lvl, node))) * P.as;
+    const double a[3] = {ap[0], ap[P.as], ap[2 * P.as]};
+    const double ndr[3] = {nd[0] * RS2, nd[1] * RS2, nd[2] * RS2};
+    double Na[6];
+    N_apply<double>(nd, ndr, a, Na);
+#pragma unroll
+    for (int I = 0; I < 6; ++I) { eL[I] = e[I] - c2 * Na[I]; eR[I] = e[I] + c1 * Na[I]; }
+  };
+#pragma unroll
+  for (int I = 0; I < 6; ++I) e[I] = Eloc[I];
+  for (int lvl = 1; lvl <= s; ++lvl) {
+    split(lvl, part >> (s - lvl + 1));
+    const bool right = part >> (s - lvl) & 1;
+#pragma unroll
+    for (int I = 0; I < 6; ++I) e[I] = right ? eR[I] : eL[I];
+  }
+  const int nb = 1 << (K - 1 - s), m0 = part * nb;
+  for (int x = 0; x < nb; ++x) {
+    const int m = m0 + x, top = x == 0 ? s + 1 : K - __ffs(x) + 1;
+    if (x) {
+#pragma unroll
+      for (int I = 0; I < 6; ++I) e[I] = epsR[top][I];
+    }
+    for (int lvl = top; lvl <= K; ++lvl) {
+      split(lvl, m >> (K - lvl));
+      if (lvl < K) {
+#pragma unroll
+        for (int I = 0; I < 6; ++I) { epsR[lvl + 1][I] = eR[I]; e[I] = eL[I]; }
+      }
+    }
+#pragma unroll
+    for (int side = 0; side < 2; ++side) {
+      if (t.ph[side].kind == 0) continue;
+      const int leaf = 2 * m + side;
+      const int slot = t.lslot ? __ldg(t.lslot + leaf) : t.z_both ? leaf : (leaf >> 1);
+      if (slot < 0) continue;
+      double z[6], zn[6], sig[6];
+      load_z_slot(P, slot, z);
+      leaf_iso<double>(t.ph[side], side ? eR : eL, z, sig, nullptr, zn, nullptr);
       double* b = zout + (size_t)(6 * slot) * zos;
 #pragma unroll
       for (int c = 0; c < 6; ++c) b[c * zos] = nan_out ? __longlong_as_double(0x7ff8000000000000LL) : zn[c];
