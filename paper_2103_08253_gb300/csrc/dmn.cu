@@ -70,6 +70,8 @@ struct WorkSet {
   int64_t nslots_s = 0;         // slots of the first stage's kernel
   double* scr_w = nullptr;      // small calls, the warp organisation: a block of scratch per group of lanes
   int64_t nwarps_w = 0;
+  char* scr_b = nullptr;        // the CTA organisation of the FP64 form: block_scratch_bytes per CTA
+  int64_t* list = nullptr;      // its points left to the all-FP64 kernels
   double* nbuf = nullptr;       // per point: normals [3N] + local macro strain [6], field-major
   int64_t* perm = nullptr;      // points sorted by tree (several trees)
   int64_t nbuf_cap = 0;
@@ -88,6 +90,7 @@ struct HostPipe {
 struct dmn_handle {
   std::vector<Tree> trees;
   int N_max = 0;                // laminates of the deepest tree
+  int K_max = 0;                // its depth
   int64_t S_max = 0;            // state fields of the largest tree
   dmn_options opt;
   int device = 0, n_sm = 0;
@@ -133,6 +136,7 @@ TreeDev tree_dev(const Tree& t) {
   d.hcid = t.d_tab ? t.d_tab + 4 * t.Lc + 5 * t.N : nullptr;
   d.kslot = t.d_tab ? t.d_tab + 4 * t.Lc + 5 * t.N + ((1 << t.K) - 1) : nullptr;
   d.lslot = t.d_tab ? d.kslot + 2 * t.N : nullptr;
+  d.hdir = t.d_tab ? d.lslot + t.L : nullptr;
   return d;
 }
 
@@ -467,6 +471,7 @@ __global__ void __launch_bounds__(128, MINB) k_newton(NewtonParams<T> P) {
   Sub<T> root_acc;   // line search: results at the accepted iterate
   double Eloc[6];
   unsigned long long npass = 0;
+  const int64_t nw = (int64_t)n_work(P.n, P.n_list);
   // the extrapolated start failed: continue from the stored jumps a^n, as a new point would
   auto restart = [&](const TreeDev& t) {
     const int nzf = 6 * t.nz;
@@ -492,7 +497,7 @@ __global__ void __launch_bounds__(128, MINB) k_newton(NewtonParams<T> P) {
       base = __shfl_sync(0xffffffffu, base, leader);
       if (need) {
         const int64_t i = (int64_t)(base + __popc(mask & ((1u << lane) - 1u)));
-        if (i >= P.n) {
+        if (i >= nw) {
           pt = P.n;
         } else {
           point_of(P.perm, P.tid, P.F.n, i, pt, tr);
@@ -759,6 +764,7 @@ struct FinalParams {
   double *state_out, *stress, *tangent;
   const int32_t* status;
   const double* nbuf;
+  const unsigned long long* n_list = nullptr;  // the points are perm[0 .. *n_list) instead of all n
 };
 
 // Without the sweep a point may be split over gridDim.y = 2^s threads (final_split), each of which takes
@@ -766,11 +772,12 @@ struct FinalParams {
 template <bool SWEEP, bool CMP>
 __global__ void __launch_bounds__(128) k_final(FinalParams P) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= P.n) return;
+  if (i >= (int64_t)n_work(P.n, P.n_list)) return;
   int64_t pt;
   int tr;
   point_of(P.perm, P.tid, P.F.n, i, pt, tr);
   if (tr >= P.F.n) return;  // unknown tree: reported by the Newton kernel
+  if (P.status[pt] == STATUS_RETRY) return;
   const TreeDev& t = P.F.t[tr];
   const int part = SWEEP ? 0 : blockIdx.y, split = SWEEP ? 0 : min(31 - __clz((int)gridDim.y), t.K - 1);
   if (part >> split) return;   // a shallower tree has fewer parts
@@ -1106,7 +1113,7 @@ struct CmpTree {
   std::vector<float> cf;         // c1f [N], c2f [N], c12f [N], scf [N], 1 / (c1 c2) [N]
   std::vector<int> tab;          // lf [Lc] (4 ints each), pre [N], post [N], paper index [N], children [2 N],
                                  // the laminate at each heap position [2^K - 1], leaf children's state slots [2 N],
-                                 // the state slot of each leaf [2^K]
+                                 // the state slot of each leaf [2^K], what each heap position does [2^K - 1]
 };
 
 void build_compressed(const dmn_tree_desc& d, const bool inelastic[2], CmpTree& B) {
@@ -1202,6 +1209,8 @@ void build_compressed(const dmn_tree_desc& d, const bool inelastic[2], CmpTree& 
       }
   B.tab.insert(B.tab.end(), kslot.begin(), kslot.end());
   B.tab.insert(B.tab.end(), slot_of.begin(), slot_of.end());
+  for (int h = 1; h <= N; ++h)
+    B.tab.push_back(cid[h] >= 0 ? 0 : !(W[h] > 0.0) ? 3 : W[2 * h] > 0.0 ? 1 : 2);
 }
 
 bool has_zero_weight(const dmn_tree_desc& d) {
@@ -1251,6 +1260,20 @@ int warp_lanes_for(const dmn_handle* h, int64_t n) {
   return h->opt.precision == DMN_PREC_F64 ? 8 : 16;
 }
 
+// The CTA organisation (csrc/dmn_block.cu) runs the FP64 form's Newton iteration from the paper's start, for
+// trees of depth 3 or more (its subtrees), whatever the call's size.
+bool block_on(const dmn_handle* h) {
+  if (h->opt.precision != DMN_PREC_F64 || h->opt.predictor || first_stage_on(h->opt)) return false;
+  for (const Tree& t : h->trees)
+    if (t.K < 3 || t.N < 1) return false;
+  return true;
+}
+int block_leaf_slots(const dmn_handle* h) {
+  for (const Tree& t : h->trees)
+    if (t.z_both) return 8;
+  return 4;
+}
+
 // Per-slot scratch and counters of one work set (per-point buffers come with the first update).
 cudaError_t alloc_ws(const dmn_handle* h, WorkSet& w) {
   // per slot: normals + one or two jump buffers (FP64); one or two g, H buffers + FP32 normals
@@ -1262,6 +1285,8 @@ cudaError_t alloc_ws(const dmn_handle* h, WorkSet& w) {
     w.nslots_s = (int64_t)h->n_sm * h->opt.stage_ctas_per_sm * 128;
     e = cudaMalloc(&w.scr_s, sizeof(float) * (size_t)(27 * h->N_max) * w.nslots_s);
   }
+  if (e == cudaSuccess && block_on(h))
+    e = cudaMalloc(&w.scr_b, block_scratch_bytes(block_leaf_slots(h)) * (size_t)(h->n_sm * BLOCK_CTAS_PER_SM));
   if (e == cudaSuccess && warp_possible(h)) {
     // one slot per group of the smallest size the handle may use
     w.nwarps_w = (int64_t)h->n_sm * WARP_CTAS_PER_SM * 128 / (h->opt.warp_lanes ? h->opt.warp_lanes : WARP_MIN_LANES);
@@ -1274,6 +1299,7 @@ cudaError_t alloc_ws(const dmn_handle* h, WorkSet& w) {
 }
 
 void free_ws(WorkSet& w) {
+  cudaFree(w.scr_b); cudaFree(w.list);
   cudaFree(w.scr_d); cudaFree(w.scr_t); cudaFree(w.scr_s); cudaFree(w.scr_w); cudaFree(w.counter); cudaFree(w.nbuf);
   cudaFree(w.perm);
   w = WorkSet();
@@ -1330,11 +1356,12 @@ int update_on(dmn_handle* h, WorkSet& w, int64_t n, int64_t n_call, const int32_
   if (n > w.nbuf_cap) {
     e = cudaStreamSynchronize(s);
     if (e == cudaSuccess) {
-      cudaFree(w.nbuf); cudaFree(w.perm);
-      w.nbuf = nullptr; w.perm = nullptr; w.nbuf_cap = 0;
+      cudaFree(w.nbuf); cudaFree(w.perm); cudaFree(w.list);
+      w.nbuf = nullptr; w.perm = nullptr; w.list = nullptr; w.nbuf_cap = 0;
     }
     if (e == cudaSuccess) e = cudaMalloc(&w.nbuf, sizeof(double) * (size_t)(3 * NM + 6) * n);
     if (e == cudaSuccess) e = cudaMalloc(&w.perm, sizeof(int64_t) * (size_t)n);
+    if (e == cudaSuccess && w.scr_b) e = cudaMalloc(&w.list, sizeof(int64_t) * (size_t)n);
     if (e != cudaSuccess) return cuda_fail(h, e, "dmn_update: per-point buffer");
     w.nbuf_cap = n;
   }
@@ -1355,7 +1382,8 @@ int update_on(dmn_handle* h, WorkSet& w, int64_t n, int64_t n_call, const int32_
     ev = h->events[h->events_used++].data();
     cudaEventRecord(ev[0], s);
   }
-  // counters: [0] work, [1..9] points per tree, [10..18] cursors, [19] first stage, [20] warp sweep
+  // counters: [0] work, [1..9] points per tree, [10..18] cursors, [19] first stage, [20] warp sweep,
+  // [21..29] the CTA organisation
   e = cudaMemsetAsync(w.counter, 0, sizeof(unsigned long long) * 32, s);
   if (e != cudaSuccess) return cuda_fail(h, e, "dmn_update: counter reset");
   const int64_t* perm = nullptr;
@@ -1374,7 +1402,7 @@ int update_on(dmn_handle* h, WorkSet& w, int64_t n, int64_t n_call, const int32_
   const int threads_per_sm = h->opt.block * h->opt.ctas_per_sm;
   const int minb = threads_per_sm > 384 ? 4 : threads_per_sm > 256 ? 3 : 2;
   const bool ls = h->opt.line_search != 0;
-  const int block = h->opt.block;
+  const int cta = h->opt.block;
   const bool warp = warp_on(h, n_call) && w.scr_w;
   const bool stage = first_stage_on(h->opt) && !warp;   // a small batch goes straight to the warp kernel
   const unsigned wgrid = (unsigned)(h->n_sm * WARP_CTAS_PER_SM);
@@ -1390,42 +1418,66 @@ int update_on(dmn_handle* h, WorkSet& w, int64_t n, int64_t n_call, const int32_
     else launch_stage<false>(SP, h->opt.stage_ctas_per_sm, sgrid, s);
   }
   if (ev) cudaEventRecord(ev[2], s);
-  if (!mixed) {
-    NewtonParams<double> P{F, n, h->nslots, NM, tree_id, perm, state_in, state_out, stress, tangent, iters, status,
-                           w.nbuf, w.scr_d, (double*)w.scr_t, w.counter, h->opt.tol, h->opt.max_iter, 1,
-                           h->opt.predictor, dE, stage ? state_out : nullptr, passes ? passes + 1 : nullptr,
-                           stage ? 1 : 0};
+  const bool block = w.scr_b != nullptr;
+  const dim3 gf(g1, final_split(n, h->n_sm));
+  FinalParams FP{F, n, NM, tree_id, perm, Q, state_in, state_out, stress, tangent, status, w.nbuf};
+  NewtonParams<double> DP{F, n, h->nslots, NM, tree_id, perm, state_in, state_out, stress, tangent, iters, status,
+                          w.nbuf, w.scr_d, (double*)w.scr_t, w.counter, h->opt.tol, h->opt.max_iter, 1,
+                          h->opt.predictor, dE, stage ? state_out : nullptr, passes ? passes + 1 : nullptr,
+                          stage ? 1 : 0};
+  auto newton_f64 = [&](const NewtonParams<double>& P) {
     if (warp && h->cmp) launch_warp<double, true>(P, ls, lanes, wgrid, w.scr_w, s);
     else if (warp) launch_warp<double, false>(P, ls, lanes, wgrid, w.scr_w, s);
-    else if (h->cmp) launch_newton<double, true>(P, ls, minb, grid, block, s);
-    else launch_newton<double, false>(P, ls, minb, grid, block, s);
+    else if (h->cmp) launch_newton<double, true>(P, ls, minb, grid, cta, s);
+    else launch_newton<double, false>(P, ls, minb, grid, cta, s);
+  };
+  auto final_pass = [&](const FinalParams& P, bool with_sweep) {
+    if (with_sweep && h->cmp) k_final<true, true><<<g1, 128, 0, s>>>(P);
+    else if (with_sweep) k_final<true, false><<<g1, 128, 0, s>>>(P);
+    else if (h->cmp) k_final<false, true><<<gf, 128, 0, s>>>(P);
+    else k_final<false, false><<<gf, 128, 0, s>>>(P);
+  };
+  // the FP64 sweep for stress and tangent: in the warp organisation (counter [20]; k_final then rotates) or
+  // one thread per point.  Even at 216 points per SM.
+  auto sweep_pass = [&](bool in_warps) {
+    if (in_warps) {
+      NewtonParams<double> SP = DP;
+      SP.counter = w.counter + 20;
+      const int swl = h->opt.warp_lanes ? h->opt.warp_lanes : (n_call <= 16 * (int64_t)h->n_sm ? 32 : 8);
+      if (h->cmp) launch_sweep_warp<true>(SP, swl, wgrid, w.scr_w, s);
+      else launch_sweep_warp<false>(SP, swl, wgrid, w.scr_w, s);
+    }
+    final_pass(FP, !in_warps);
+  };
+  if (block) {
+    BlockParams P{F, n, NM, block_leaf_slots(h), tree_id, perm, state_in, state_out, stress, tangent, iters, status,
+                  w.nbuf, w.scr_b, w.counter, w.list, h->opt.tol, h->opt.max_iter, passes ? passes + 1 : nullptr};
+    const int64_t ctas = div_up(n, BLOCK_THREADS >> (h->K_max - 3));
+    launch_block(P, ls, h->cmp, (unsigned)std::min<int64_t>(ctas, (int64_t)h->n_sm * BLOCK_CTAS_PER_SM), s);
+  } else if (!mixed) {
+    newton_f64(DP);
   } else {
     NewtonParams<float> P{F, n, h->nslots, NM, tree_id, perm, state_in, state_out, stress, tangent, iters, status,
                           w.nbuf, w.scr_d, (float*)w.scr_t, w.counter, h->opt.tol, h->opt.max_iter, sweep ? 0 : 1,
                           h->opt.predictor, dE, stage ? state_out : nullptr, passes ? passes + 1 : nullptr, 0};
     if (warp && h->cmp) launch_warp<float, true>(P, ls, lanes, wgrid, w.scr_w, s);
     else if (warp) launch_warp<float, false>(P, ls, lanes, wgrid, w.scr_w, s);
-    else if (h->cmp) launch_newton<float, true>(P, ls, minb, grid, block, s);
-    else launch_newton<float, false>(P, ls, minb, grid, block, s);
+    else if (h->cmp) launch_newton<float, true>(P, ls, minb, grid, cta, s);
+    else launch_newton<float, false>(P, ls, minb, grid, cta, s);
   }
   if (ev) cudaEventRecord(ev[3], s);
-  const dim3 gf(g1, final_split(n, h->n_sm));
-  FinalParams FP{F, n, NM, tree_id, perm, Q, state_in, state_out, stress, tangent, status, w.nbuf};
-  if (sweep && warp) {   // the FP64 sweep in the warp organisation (counter [20]), then k_final rotates
-    NewtonParams<double> SP{F, n, h->nslots, NM, tree_id, perm, state_in, state_out, stress, tangent, iters, status,
-                            w.nbuf, w.scr_d, (double*)w.scr_t, w.counter + 20, h->opt.tol, h->opt.max_iter, 1, 0,
-                            dE, nullptr, nullptr, 0};
-    const int swl = h->opt.warp_lanes ? h->opt.warp_lanes : (n_call <= 16 * (int64_t)h->n_sm ? 32 : 8);
-    if (h->cmp) launch_sweep_warp<true>(SP, swl, wgrid, w.scr_w, s);
-    else launch_sweep_warp<false>(SP, swl, wgrid, w.scr_w, s);
-    if (h->cmp) k_final<false, true><<<gf, 128, 0, s>>>(FP);
-    else k_final<false, false><<<gf, 128, 0, s>>>(FP);
+  if (block) {
+    sweep_pass(w.scr_w && n_call <= 216 * (int64_t)h->n_sm);
+    // the points it left: the all-FP64 iteration from their start, in the organisation of the call's size
+    NewtonParams<double> P = DP;
+    P.perm = FP.perm = w.list;
+    P.n_list = FP.n_list = w.counter + 29;
+    newton_f64(P);
+    final_pass(FP, false);
   } else if (sweep) {
-    if (h->cmp) k_final<true, true><<<g1, 128, 0, s>>>(FP);
-    else k_final<true, false><<<g1, 128, 0, s>>>(FP);
+    sweep_pass(warp);
   } else {
-    if (h->cmp) k_final<false, true><<<gf, 128, 0, s>>>(FP);
-    else k_final<false, false><<<gf, 128, 0, s>>>(FP);
+    final_pass(FP, false);
   }
   if (ev) cudaEventRecord(ev[4], s);
   e = cudaGetLastError();
@@ -1594,6 +1646,7 @@ int dmn_create(const dmn_tree_desc* trees, int32_t n_trees, const dmn_options* o
   h->trees = tv;
   h->cmp = cmp;
   h->N_max = std::max(N_max, 1);
+  for (const Tree& t : tv) h->K_max = std::max(h->K_max, t.K);
   h->S_max = S_max;
   h->opt = o;
   cudaError_t e = cudaGetDevice(&h->device);

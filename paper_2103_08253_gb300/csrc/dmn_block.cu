@@ -1,0 +1,792 @@
+// The CTA organisation of the FP64 Newton iteration: k_newton_block and its launch.
+//
+// Newton's method of Sec. 3.2 with the FP64 step obtained by iterative refinement.  GB300 runs FP64 at
+// 1/64 of its FP32 rate, and 152 k of the 183 kflop of an FP64 pass (depth 8) are the condensation that
+// only serves to solve J da = -R.  Here each iteration
+//   A  evaluates strains, leaf laws and the residual R in FP64 (and tests the criterion on it),
+//   S  condenses the leaf tangents in FP32 and solves for da1 (relative error some 1e-6),
+//   B  forms R + J da1 in FP64 with the FP64 leaf tangents and solves again in FP32 for da2,
+// and applies da = da1 + da2, whose relative error is the product of the two solves' (1e-11, at most
+// some 1e-10 on the workloads' plastic paths), far below what the quadratic convergence leaves: the
+// iterates are those of the all-FP64 condensation, with its iteration counts.  A and B cost about 23 k
+// and 16 k FP64 instructions, a pass of the all-FP64 kernel 122 k.  The tangent comes from one FP64
+// sweep at the converged jumps, as in the mixed form.
+//
+// A point for which the FP32 solve does not contract (|R + J da1| > REFINE_MAX |R|: tangents near
+// singular, moduli outside the FP32 range), which is not finite, whose line search fails or which has not
+// converged within BLOCK_ITERS corrections is put on a list (status RETRY) and updated from its start by the
+// all-FP64 kernels, so that every call keeps their results and statuses.
+//
+// Organisation.  A CTA of 256 threads holds 256 / S points, S = 2^(K-3) threads per point: thread (s, p)
+// owns the s-th subtree of depth 3 (7 laminates, 8 leaves) of the point in slot p and, for s >= 1, the
+// laminate s of the top K - 3 levels (heap number).  Subtrees run depth first in registers; the top
+// levels run level by level, the strains (down) and results (up) handed over in shared memory.  All
+// per-laminate data is laid out [field][laminate][thread], so that every access is coalesced whatever
+// the tree's depth, with p fastest: a warp's lanes run the same instructions.  The top levels' laminates
+// lie on different warps (laminate h on warp h P / 32), which balances the SM's four FP64 units.
+// Every slot runs its own Newton iteration: a converged point is written out and its slot takes the next
+// one, so uneven iteration counts do not idle the CTA.
+#include <cuda_runtime.h>
+
+#include "../../include/dmn.h"
+#include "dmn_device.cuh"
+#include "dmn_launch.cuh"
+
+namespace dmn {
+
+namespace {
+
+constexpr int BT = BLOCK_THREADS;
+constexpr float REFINE_MAX = 1e-3f;
+constexpr int BLOCK_ITERS = 16;
+
+// scratch fields of a thread, in units of 8 laminates (7 of the subtree, then the top laminate)
+enum { D_A = 0, D_A2 = 3, D_N = 6, D_T = 9, D_END = 12 };                      // FP64
+enum { F_N = 0, F_H = 3, F_K = 21, F_G = 27, F_D = 30, F_END = 33 };           // FP32
+
+// laminate h (heap order, 0-based) of the full tree: its number in the handle's arrays and its fractions.
+// mode 0: a laminate; 1 / 2: passes its left / right side on (the other is weightless); 3: nothing alive
+template <bool CMP>
+struct Lam {
+  int id, mode;
+  double c1, c2;
+  __device__ Lam(const TreeDev& t, int h) {
+    mode = CMP ? __ldg(t.hdir + h) : 0;
+    id = CMP ? __ldg(t.hcid + h) : h;
+    if (!CMP || mode == 0) { c1 = __ldg(t.c1 + id); c2 = __ldg(t.c2 + id); }
+    else { c1 = c2 = 0.0; }
+  }
+};
+
+struct Ctx {
+  double* D;      // this thread's FP64 scratch: field f of laminate j at D[(8 f + j) BT]
+  float* F;       // this thread's FP32 scratch
+  double* z;      // leaf states: z[(6 leaf + c) BT]
+  double* tan;    // leaf tangents mu, c, m: tan[(8 leaf + c) BT]
+  float* tanf;    // their FP32 copies
+  __device__ double& d(int f, int j) const { return D[(8 * f + j) * BT]; }
+  __device__ float& f(int f, int j) const { return F[(8 * f + j) * BT]; }
+};
+
+__device__ __forceinline__ void load3(const Ctx& c, int f, int j, double v[3]) {
+#pragma unroll
+  for (int k = 0; k < 3; ++k) v[k] = c.d(f + k, j);
+}
+
+// The FP32 step of laminate j: g + H de; hands the corrections to the children (dL, dR).
+template <bool CMP>
+__device__ __forceinline__ void step32(const TreeDev& t, const Ctx& c, const Lam<CMP>& q, int j, const float de[6],
+                                       float da[3], float dL[6], float dR[6]) {
+  const float n[3] = {c.f(F_N, j), c.f(F_N + 1, j), c.f(F_N + 2, j)};
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    float v = c.f(F_G + k, j);
+#pragma unroll
+    for (int I = 0; I < 6; ++I) v += c.f(F_H + 6 * k + I, j) * de[I];
+    da[k] = v;
+  }
+  if (dL) {
+    const float c1 = __ldg(t.c1f + q.id), c2 = __ldg(t.c2f + q.id);
+    const float nr[3] = {n[0] * (float)RS2, n[1] * (float)RS2, n[2] * (float)RS2};
+    float Nd[6];
+    N_apply<float>(n, nr, da, Nd);
+#pragma unroll
+    for (int I = 0; I < 6; ++I) { dL[I] = de[I] - c2 * Nd[I]; dR[I] = de[I] + c1 * Nd[I]; }
+  }
+}
+
+// A, downwards: the jumps of laminate j corrected (apply) and the children's strains.
+// B, downwards: the step da1 stored and its strains.  de: the FP32 correction handed down.
+template <bool CMP, bool LS, bool PHASE_B>
+__device__ __forceinline__ void down(const TreeDev& t, const Ctx& c, int h, int j, int a_in, int a_out, bool apply,
+                                     double step, const double e[6], const float de[6], double eL[6], double eR[6],
+                                     float* dL, float* dR) {
+  const Lam<CMP> q(t, h);
+  if (CMP && q.mode) {
+#pragma unroll
+    for (int I = 0; I < 6; ++I) { eL[I] = eR[I] = e[I]; if (dL) dL[I] = dR[I] = de[I]; }
+    return;
+  }
+  double nd[3], a[3];
+  load3(c, D_N, j, nd);
+  if (PHASE_B) {
+    float da[3];
+    step32<CMP>(t, c, q, j, de, da, dL, dR);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) { c.f(F_D + k, j) = da[k]; a[k] = widen(da[k]); }
+  } else {
+    load3(c, a_in, j, a);
+    if (apply) {
+      float da[3];
+      step32<CMP>(t, c, q, j, de, da, dL, dR);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const double s = widen(c.f(F_D + k, j)) + widen(da[k]);
+        a[k] = LS ? a[k] + step * s : a[k] + s;
+        c.d(a_out + k, j) = a[k];
+      }
+    } else {
+#pragma unroll
+      for (int I = 0; I < 6; ++I) if (dL) dL[I] = dR[I] = 0.f;
+      if (LS) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) c.d(a_out + k, j) = a[k];
+      }
+    }
+  }
+  const double ndr[3] = {nd[0] * RS2, nd[1] * RS2, nd[2] * RS2};
+  double Na[6];
+  N_apply<double>(nd, ndr, a, Na);
+#pragma unroll
+  for (int I = 0; I < 6; ++I) { eL[I] = e[I] - q.c2 * Na[I]; eR[I] = e[I] + q.c1 * Na[I]; }
+}
+
+// A, upwards: residual of laminate j (t = N^T (s_R - s_L), stored) and the average stress.
+template <bool CMP>
+__device__ __forceinline__ void up_a(const TreeDev& t, const Ctx& c, int h, int j, const double sL[6],
+                                     const double sR[6], double sb[6], double& r2) {
+  const Lam<CMP> q(t, h);
+  if (CMP && q.mode) {
+#pragma unroll
+    for (int I = 0; I < 6; ++I) sb[I] = q.mode == 2 ? sR[I] : sL[I];
+    return;
+  }
+  double nd[3], u[3];
+  load3(c, D_N, j, nd);
+  residual_share<double>(nd, q.c1, q.c2, __ldg(t.sc + q.id), sL, sR, sb, u, r2);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) c.d(D_T + k, j) = u[k];
+}
+
+// B, upwards: the linearised residual of laminate j after da1, u = N^T (s_R - s_L) + N^T (tau_R - tau_L)
+// in FP64, then the FP32 solve's upward half with the stored H and Kn^-1:
+//   u += N^T (ds_R - ds_L),  g = -Kn^-1 u,  ds = c1 ds_L + c2 ds_R + c1 c2 H^T u.
+// BOT: the children are leaves (ds = 0 there).
+template <bool CMP, bool BOT>
+__device__ __forceinline__ void up_b(const TreeDev& t, const Ctx& c, int h, int j, const double tL[6],
+                                     const double tR[6], const float dsL[6], const float dsR[6], double tb[6],
+                                     float ds[6], float& r2) {
+  const Lam<CMP> q(t, h);
+  if (CMP && q.mode) {
+#pragma unroll
+    for (int I = 0; I < 6; ++I) {
+      tb[I] = q.mode == 2 ? tR[I] : tL[I];
+      ds[I] = BOT ? 0.f : q.mode == 2 ? dsR[I] : dsL[I];
+    }
+    return;
+  }
+  double nd[3], d[6], v[3];
+  load3(c, D_N, j, nd);
+  const double ndr[3] = {nd[0] * RS2, nd[1] * RS2, nd[2] * RS2};
+#pragma unroll
+  for (int I = 0; I < 6; ++I) { d[I] = tR[I] - tL[I]; tb[I] = tL[I] + q.c2 * d[I]; }
+  Nt_apply<double>(nd, ndr, d, v);
+  float u[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) u[k] = narrow_rn(c.d(D_T + k, j) + v[k]);
+  const float sc = __ldg(t.scf + q.id), c2 = __ldg(t.c2f + q.id), c12 = __ldg(t.c12f + q.id);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) r2 += (sc * u[k]) * (sc * u[k]);
+  float dd[6];
+  if (!BOT) {
+    const float n[3] = {c.f(F_N, j), c.f(F_N + 1, j), c.f(F_N + 2, j)};
+    const float nr[3] = {n[0] * (float)RS2, n[1] * (float)RS2, n[2] * (float)RS2};
+    float w[3];
+#pragma unroll
+    for (int I = 0; I < 6; ++I) dd[I] = dsR[I] - dsL[I];
+    Nt_apply<float>(n, nr, dd, w);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) u[k] += w[k];
+  }
+  float K[6];
+#pragma unroll
+  for (int k = 0; k < 6; ++k) K[k] = c.f(F_K + k, j);
+  c.f(F_G, j) = -(K[0] * u[0] + K[1] * u[1] + K[2] * u[2]);
+  c.f(F_G + 1, j) = -(K[1] * u[0] + K[3] * u[1] + K[4] * u[2]);
+  c.f(F_G + 2, j) = -(K[2] * u[0] + K[4] * u[1] + K[5] * u[2]);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) u[k] *= c12;
+#pragma unroll
+  for (int I = 0; I < 6; ++I) {
+    float x = BOT ? 0.f : dsL[I] + c2 * dd[I];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) x += c.f(F_H + 6 * k + I, j) * u[k];
+    ds[I] = x;
+  }
+}
+
+// S, upwards: FP32 condensation of laminate j (Sub without the FP64 stress).
+struct Sub32 {
+  float ds[6], C[21];
+};
+
+__device__ __forceinline__ void solve32(const Ctx& c, int j, float c12, const float Ki[3][3], const float B[6][3],
+                                        const float u[3], float ds[6], float C[21]) {
+  float H[3][6], g[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+#pragma unroll
+    for (int I = 0; I < 6; ++I) H[k][I] = -(Ki[k][0] * B[I][0] + Ki[k][1] * B[I][1] + Ki[k][2] * B[I][2]);
+    g[k] = -(Ki[k][0] * u[0] + Ki[k][1] * u[1] + Ki[k][2] * u[2]);
+  }
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+#pragma unroll
+    for (int I = 0; I < 6; ++I) c.f(F_H + 6 * k + I, j) = H[k][I];
+    c.f(F_G + k, j) = g[k];
+  }
+  c.f(F_K, j) = Ki[0][0]; c.f(F_K + 1, j) = Ki[0][1]; c.f(F_K + 2, j) = Ki[0][2];
+  c.f(F_K + 3, j) = Ki[1][1]; c.f(F_K + 4, j) = Ki[1][2]; c.f(F_K + 5, j) = Ki[2][2];
+#pragma unroll
+  for (int I = 0; I < 6; ++I) {
+    const float b[3] = {c12 * B[I][0], c12 * B[I][1], c12 * B[I][2]};
+    ds[I] += b[0] * g[0] + b[1] * g[1] + b[2] * g[2];
+#pragma unroll
+    for (int J = I; J < 6; ++J) C[sidx(I, J)] += b[0] * H[0][J] + b[1] * H[1][J] + b[2] * H[2][J];
+  }
+}
+
+template <bool CMP>
+__device__ __forceinline__ void condense32(const TreeDev& t, const Ctx& c, int h, int j, const Sub32& L, const Sub32& R,
+                                           Sub32& o) {
+  const Lam<CMP> q(t, h);
+  if (CMP && q.mode) {
+    if (q.mode == 2) o = R; else o = L;
+    return;
+  }
+  const float c2 = __ldg(t.c2f + q.id), c12 = __ldg(t.c12f + q.id);
+  const float n[3] = {c.f(F_N, j), c.f(F_N + 1, j), c.f(F_N + 2, j)};
+  const float nr[3] = {n[0] * (float)RS2, n[1] * (float)RS2, n[2] * (float)RS2};
+  float dC[21], Ch[21], X[6][3], B[6][3], u[3], w[3], dd[6];
+#pragma unroll
+  for (int k = 0; k < 21; ++k) { dC[k] = R.C[k] - L.C[k]; Ch[k] = R.C[k] - c2 * dC[k]; }
+  SN_apply<float>(Ch, n, nr, X);
+  float Ki[3][3];
+  {
+    const float k00 = n[0] * X[0][0] + nr[2] * X[4][0] + nr[1] * X[5][0];
+    const float k10 = n[1] * X[1][0] + nr[2] * X[3][0] + nr[0] * X[5][0];
+    const float k20 = n[2] * X[2][0] + nr[1] * X[3][0] + nr[0] * X[4][0];
+    const float k11 = n[1] * X[1][1] + nr[2] * X[3][1] + nr[0] * X[5][1];
+    const float k21 = n[2] * X[2][1] + nr[1] * X[3][1] + nr[0] * X[4][1];
+    const float k22 = n[2] * X[2][2] + nr[1] * X[3][2] + nr[0] * X[4][2];
+    inv3_sym<float>(k00, k10, k20, k11, k21, k22, Ki);
+  }
+  SN_apply<float>(dC, n, nr, B);
+#pragma unroll
+  for (int I = 0; I < 6; ++I) dd[I] = R.ds[I] - L.ds[I];
+  Nt_apply<float>(n, nr, dd, w);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) u[k] = narrow_rn(c.d(D_T + k, j)) + w[k];
+#pragma unroll
+  for (int I = 0; I < 6; ++I) o.ds[I] = L.ds[I] + c2 * dd[I];
+#pragma unroll
+  for (int k = 0; k < 21; ++k) o.C[k] = L.C[k] + c2 * dC[k];
+  solve32(c, j, c12, Ki, B, u, o.ds, o.C);
+}
+
+// leaf tangent in FP32: the phase's constants or the stored mu, c, m
+__device__ __forceinline__ void leaf_tan32(const PhaseDev& ph, const float* s, LeafTan<float>& D) {
+  if (ph.kind == 0) {
+    D.lam = ph.lamf; D.mu = ph.Gf; D.c = 0.f;
+#pragma unroll
+    for (int I = 0; I < 6; ++I) D.m[I] = 0.f;
+  } else {
+    D.mu = s[0]; D.c = s[BT];
+    D.lam = ph.f.K - (float)(2.0 / 3.0) * D.mu;
+#pragma unroll
+    for (int I = 0; I < 6; ++I) D.m[I] = s[(2 + I) * BT];
+  }
+}
+
+// the structured condensation of a bottom laminate (condense_bottom); a side passed on keeps its leaf's tangent
+template <bool CMP>
+__device__ __forceinline__ void condense32_bottom(const TreeDev& t, const Ctx& c, int h, int j,
+                                                  const LeafTan<float>& L, const LeafTan<float>& R, bool elL, bool elR,
+                                                  Sub32& o) {
+  const Lam<CMP> q(t, h);
+#pragma unroll
+  for (int I = 0; I < 6; ++I) o.ds[I] = 0.f;
+  float c1, c2;
+  if (CMP && q.mode) { c2 = q.mode == 2 ? 1.f : 0.f; c1 = 1.f - c2; }
+  else { c1 = __ldg(t.c1f + q.id); c2 = __ldg(t.c2f + q.id); }
+  // the average of the two tangents
+  const float lam = c1 * L.lam + c2 * R.lam, mu2 = 2.f * (c1 * L.mu + c2 * R.mu);
+  const float wL = c1 * L.c, wR = c2 * R.c;
+#pragma unroll
+  for (int I = 0; I < 6; ++I) {
+    const float hL = wL * L.m[I], hR = wR * R.m[I];
+#pragma unroll
+    for (int J = I; J < 6; ++J) {
+      float v = I < 3 && J < 3 ? lam : 0.f;
+      if (I == J) v += mu2;
+      if (!elL) v -= hL * L.m[J];
+      if (!elR) v -= hR * R.m[J];
+      o.C[sidx(I, J)] = v;
+    }
+  }
+  if (CMP && q.mode) return;
+  const float c12 = __ldg(t.c12f + q.id);
+  const float n[3] = {c.f(F_N, j), c.f(F_N + 1, j), c.f(F_N + 2, j)};
+  const float nr[3] = {n[0] * (float)RS2, n[1] * (float)RS2, n[2] * (float)RS2};
+  const float a = c2 * L.mu + c1 * R.mu, b = c2 * (L.lam + L.mu) + c1 * (R.lam + R.mu);
+  const float dlam = R.lam - L.lam, dmu2 = 2.f * (R.mu - L.mu), dld = dlam + dmu2;
+  float k[3][3], B[6][3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int l = i; l < 3; ++l) k[i][l] = b * n[i] * n[l] + (i == l ? a : 0.f);
+#pragma unroll
+  for (int I = 0; I < 6; ++I)
+#pragma unroll
+    for (int l = 0; l < 3; ++l)
+      B[I][l] = I < 3 ? (I == l ? dld : dlam) * n[l] : (N_nonzero(I, l) ? dmu2 * N_entry<float>(n, nr, I, l) : 0.f);
+  if (!elL) {
+    float v[3];
+    Nt_apply<float>(n, nr, L.m, v);
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int l = i; l < 3; ++l) k[i][l] -= (c2 * L.c) * v[i] * v[l];
+#pragma unroll
+    for (int I = 0; I < 6; ++I)
+#pragma unroll
+      for (int l = 0; l < 3; ++l) B[I][l] += (L.c * L.m[I]) * v[l];
+  }
+  if (!elR) {
+    float v[3];
+    Nt_apply<float>(n, nr, R.m, v);
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int l = i; l < 3; ++l) k[i][l] -= (c1 * R.c) * v[i] * v[l];
+#pragma unroll
+    for (int I = 0; I < 6; ++I)
+#pragma unroll
+      for (int l = 0; l < 3; ++l) B[I][l] -= (R.c * R.m[I]) * v[l];
+  }
+  float Ki[3][3];
+  inv3_sym<float>(k[0][0], k[0][1], k[0][2], k[1][1], k[1][2], k[2][2], Ki);
+  const float u[3] = {narrow_rn(c.d(D_T, j)), narrow_rn(c.d(D_T + 1, j)), narrow_rn(c.d(D_T + 2, j))};
+  solve32(c, j, c12, Ki, B, u, o.ds, o.C);
+}
+
+// D e of a leaf in FP64 (B): the phase's constants or the stored mu, c, m
+__device__ __forceinline__ void leaf_apply(const PhaseDev& ph, const double* s, const double e[6], double tau[6]) {
+  const double tr = e[0] + e[1] + e[2];
+  if (ph.kind == 0) {
+    const double lt = ph.lam * tr, g2 = 2.0 * ph.G;
+#pragma unroll
+    for (int I = 0; I < 6; ++I) tau[I] = I < 3 ? g2 * e[I] + lt : g2 * e[I];
+    return;
+  }
+  const double mu = s[0];
+  double m[6], me = 0.0;
+#pragma unroll
+  for (int I = 0; I < 6; ++I) { m[I] = s[(2 + I) * BT]; me += m[I] * e[I]; }
+  const double cm = s[BT] * me, g2 = 2.0 * mu, lt = (ph.K - (2.0 / 3.0) * mu) * tr;
+#pragma unroll
+  for (int I = 0; I < 6; ++I) tau[I] = (I < 3 ? g2 * e[I] + lt : g2 * e[I]) - cm * m[I];
+}
+
+}  // namespace
+
+// flags of a slot
+enum { B_ACT = 1, B_NEW = 2, B_FIRST = 4, B_CONT = 8, B_CONV = 16, B_CUR = 32 };
+
+template <bool LS, bool CMP>
+__global__ void __launch_bounds__(BT, 2) k_newton_block(BlockParams P) {
+  __shared__ double sh_e[6][BT];      // strains handed down, stresses handed up, at the leftmost subtree's place
+  __shared__ float sh_c[27][BT];      // FP32 results handed up; its first rows the corrections handed down
+  extern __shared__ double dyn[];
+  double* sh_r = dyn;                 // [BT] partial residual norms
+  long long* sh_pt = (long long*)(dyn + BT);
+  int* sh_fl = (int*)(dyn + 2 * BT);
+  float* sh_st = (float*)(sh_fl + BT);
+  const int tid = threadIdx.x, lane = tid & 31;
+  const size_t n = (size_t)P.n;
+  Ctx c;
+  {
+    char* base = P.scratch + (size_t)blockIdx.x * block_scratch_bytes(P.leaf_slots);
+    double* D = (double*)base;
+    c.D = D + tid;
+    c.z = D + (size_t)8 * D_END * BT + tid;
+    c.tan = c.z + (size_t)6 * P.leaf_slots * BT;
+    float* F = (float*)(D + (size_t)(8 * D_END + 14 * P.leaf_slots) * BT);
+    c.F = F + tid;
+    c.tanf = F + (size_t)8 * F_END * BT + tid;
+  }
+  for (int tr = 0; tr < P.F.n; ++tr) {
+    const TreeDev& t = P.F.t[tr];
+    const int K = t.K, Kt = K - 3, S = 1 << Kt, nP = BT >> Kt, p = tid & (nP - 1), s = tid / nP;
+    // with several trees the points are sorted by tree: this tree's are [begin, end)
+    const unsigned long long end = P.perm ? P.counter[10 + tr] : (tr ? 0ull : (unsigned long long)P.n);
+    const unsigned long long begin = P.perm ? end - P.counter[1 + tr] : 0ull;
+    const int nzf = 6 * t.nz;
+    const bool both = t.z_both;
+    // the thread's top laminate: heap number s on level `lev`, its results at place pos, its right child's at pos + half
+    const int lev = s ? 31 - __clz(s) : -1;
+    const int pos = s ? (((s << (Kt - lev)) - S) * nP + p) : p, half = s ? (S >> (lev + 1)) * nP : 0;
+    const int R1 = S + s;                      // heap number of the thread's subtree
+    auto heap = [&](int j) { return (j == 0 ? R1 : j < 3 ? 2 * R1 + j - 1 : j < 7 ? 4 * R1 + j - 3 : s) - 1; };
+    // a subtree with nothing alive in it is skipped (its results are never used, only kept finite)
+    const bool dead = CMP && __ldg(t.hdir + heap(0)) == 3;
+    // state of slot p, kept by thread p < nP
+    long long pt = -1;
+    int it = 0, halv = 0, np = 0;
+    double rn_acc = 0.0;
+    bool more = tid < nP;
+    if (tid < nP) sh_fl[tid] = 0;
+    for (;;) {
+      if (tid < nP && more && !(sh_fl[tid] & B_ACT)) {
+        for (;;) {
+          const unsigned long long i = begin + atomicAdd(P.counter + 21 + tr, 1ull);
+          if (i >= end) { more = false; break; }
+          int tt;
+          int64_t x;
+          point_of(P.perm, P.tid, P.F.n, (int64_t)i, x, tt);
+          if (tt == tr) {
+            pt = x; it = 0; halv = 0; np = 0; rn_acc = 0.0;
+            sh_pt[tid] = pt; sh_st[tid] = 1.f;
+            sh_fl[tid] = B_ACT | B_NEW | B_FIRST;
+            break;
+          }
+          block_bad_tree(P, x);
+        }
+      }
+      const bool any = tid < nP && (sh_fl[tid] & B_ACT);
+      if (!__syncthreads_or(any)) break;
+      int fl = sh_fl[p];
+      const size_t mypt = (size_t)sh_pt[p];
+      if (fl & B_NEW) {
+        const double* st = P.state_in + mypt;
+        const double* nb = P.nbuf + mypt;
+        for (int j = s ? 7 : 6; j >= 0; --j) {
+          const int h = heap(j);
+          const int id = CMP ? __ldg(t.hcid + h) : h;
+          if (id < 0) continue;
+          const int row = CMP ? id : (1 << K) - 3 * (1 << (31 - __clz(h + 1))) + h + 1;
+#pragma unroll
+          for (int k = 0; k < 3; ++k) {
+            c.d(D_A + k, j) = st[(nzf + 3 * row + k) * n];
+            const double v = nb[(3 * id + k) * n];
+            c.d(D_N + k, j) = v;
+            c.f(F_N + k, j) = narrow_rn(v);
+          }
+        }
+        for (int l = 0; l < 8; ++l) {
+          if (t.ph[l & 1].kind == 0) continue;
+          const int leaf = 8 * s + l, ls = both ? l : l >> 1;
+          const int slot = CMP ? __ldg(t.lslot + leaf) : both ? leaf : leaf >> 1;
+#pragma unroll
+          for (int k = 0; k < 6; ++k) c.z[(6 * ls + k) * BT] = slot >= 0 ? st[(6 * slot + k) * n] : 0.0;
+        }
+      }
+      const bool act = fl & B_ACT, apply = act && !(fl & B_FIRST);
+      const int a_in = LS && (fl & B_CUR) ? D_A2 : D_A, a_out = LS ? (a_in == D_A ? D_A2 : D_A) : D_A;
+      const double step = LS ? (double)sh_st[p] : 1.0;
+      // ---- A: strains down, leaf laws, residual up (FP64)
+      float(*sd)[BT] = sh_c;
+      if (act && s == 0) {
+#pragma unroll
+        for (int I = 0; I < 6; ++I) { sh_e[I][p] = P.nbuf[(3 * P.N_max + I) * n + mypt]; sd[I][p] = 0.f; }
+      }
+      __syncthreads();
+      for (int l = 0; l < Kt; ++l) {
+        if (act && lev == l) {
+          double e[6], eL[6], eR[6];
+          float de[6], dL[6], dR[6];
+#pragma unroll
+          for (int I = 0; I < 6; ++I) { e[I] = sh_e[I][pos]; de[I] = sd[I][pos]; }
+          down<CMP, LS, false>(t, c, s - 1, 7, a_in, a_out, apply, step, e, de, eL, eR, dL, dR);
+#pragma unroll
+          for (int I = 0; I < 6; ++I) {
+            sh_e[I][pos] = eL[I]; sh_e[I][pos + half] = eR[I];
+            sd[I][pos] = dL[I]; sd[I][pos + half] = dR[I];
+          }
+        }
+        __syncthreads();
+      }
+      double r2 = 0.0;
+      if (act && !dead) {
+        double e[6], eL[6], eR[6], fL[6], fR[6], sq[6], sh[6], sb[6];
+        float de[6], dL[6], dR[6], dfL[6], dfR[6];
+#pragma unroll
+        for (int I = 0; I < 6; ++I) { e[I] = sh_e[I][tid]; de[I] = sd[I][tid]; }
+        down<CMP, LS, false>(t, c, heap(0), 0, a_in, a_out, apply, step, e, de, eL, eR, dL, dR);
+#pragma unroll 1
+        for (int q = 0; q < 4; ++q) {
+          if (!(q & 1)) {
+#pragma unroll
+            for (int I = 0; I < 6; ++I) { e[I] = q ? eR[I] : eL[I]; de[I] = q ? dR[I] : dL[I]; }
+            down<CMP, LS, false>(t, c, heap(1 + (q >> 1)), 1 + (q >> 1), a_in, a_out, apply, step, e, de, fL, fR,
+                                 dfL, dfR);
+          }
+          double gL[6], gR[6], z[6], s0[6], s1[6];
+#pragma unroll
+          for (int I = 0; I < 6; ++I) { e[I] = q & 1 ? fR[I] : fL[I]; de[I] = q & 1 ? dfR[I] : dfL[I]; }
+          down<CMP, LS, false>(t, c, heap(3 + q), 3 + q, a_in, a_out, apply, step, e, de, gL, gR, nullptr, nullptr);
+#pragma unroll
+          for (int side = 0; side < 2; ++side) {
+            const int ls = both ? 2 * q + side : q;
+            const bool el = t.ph[side].kind == 0;
+#pragma unroll
+            for (int k = 0; k < 6; ++k) z[k] = el ? 0.0 : c.z[(6 * ls + k) * BT];
+            LeafTan<double> D;
+            leaf_iso<double, double>(t.ph[side], side ? gR : gL, z, side ? s1 : s0, &D, nullptr, nullptr);
+            if (!el) {
+              c.tan[(8 * ls) * BT] = D.mu; c.tan[(8 * ls + 1) * BT] = D.c;
+              c.tanf[(8 * ls) * BT] = narrow_rn(D.mu); c.tanf[(8 * ls + 1) * BT] = narrow_rn(D.c);
+#pragma unroll
+              for (int k = 0; k < 6; ++k) {
+                c.tan[(8 * ls + 2 + k) * BT] = D.m[k];
+                c.tanf[(8 * ls + 2 + k) * BT] = narrow_rn(D.m[k]);
+              }
+            }
+          }
+          up_a<CMP>(t, c, heap(3 + q), 3 + q, s0, s1, sb, r2);
+          if (q & 1) {
+            double o[6];
+            up_a<CMP>(t, c, heap(1 + (q >> 1)), 1 + (q >> 1), sq, sb, o, r2);
+#pragma unroll
+            for (int I = 0; I < 6; ++I) { if (q == 1) sh[I] = o[I]; else sb[I] = o[I]; }
+          } else {
+#pragma unroll
+            for (int I = 0; I < 6; ++I) sq[I] = sb[I];
+          }
+        }
+        up_a<CMP>(t, c, heap(0), 0, sh, sb, e, r2);
+#pragma unroll
+        for (int I = 0; I < 6; ++I) sh_e[I][tid] = e[I];
+      } else if (act) {
+#pragma unroll
+        for (int I = 0; I < 6; ++I) sh_e[I][tid] = 0.0;
+      }
+      __syncthreads();
+      for (int l = Kt - 1; l >= 0; --l) {
+        if (act && lev == l) {
+          double sL[6], sR[6], sb[6];
+#pragma unroll
+          for (int I = 0; I < 6; ++I) { sL[I] = sh_e[I][pos]; sR[I] = sh_e[I][pos + half]; }
+          up_a<CMP>(t, c, s - 1, 7, sL, sR, sb, r2);
+#pragma unroll
+          for (int I = 0; I < 6; ++I) sh_e[I][pos] = sb[I];
+        }
+        __syncthreads();
+      }
+      // sum of the point's shares in a fixed order: the warp's lanes of one slot, then the warps
+      for (int o = 16; o >= nP; o >>= 1) r2 += __shfl_xor_sync(0xffffffffu, r2, o);
+      const int groups = nP < 32 ? BT / 32 : S;
+      if (nP >= 32) sh_r[tid] = r2;
+      else if (lane < nP) sh_r[(tid >> 5) * nP + lane] = r2;
+      __syncthreads();
+      double rn = 0.0;
+      if (tid < nP && (sh_fl[tid] & B_ACT)) {
+        double r = 0.0, sn2 = 0.0;
+        for (int k = 0; k < groups; ++k) r += sh_r[k * nP + tid];
+        rn = sqrt(r);
+#pragma unroll
+        for (int I = 0; I < 6; ++I) sn2 += sh_e[I][tid] * sh_e[I][tid];
+        const double sn = sqrt(sn2);
+        int f = sh_fl[tid] & (B_ACT | B_FIRST | B_CUR);
+        ++np;
+        bool retry = false;
+        const bool ok = !LS || (f & B_FIRST) || rn < rn_acc;
+        if (ok) {
+          if (LS) { f ^= B_CUR; sh_st[tid] = 1.f; halv = 0; }
+          rn_acc = rn;
+          f &= ~B_FIRST;
+          if (!isfinite(rn) || !isfinite(sn)) retry = true;
+          else if (rn <= P.tol * (double)t.N * sn) f |= B_CONV;
+          else if (it >= P.max_iter || it >= BLOCK_ITERS) retry = true;
+          else { ++it; f |= B_CONT; }
+        } else if (++halv > 8) {
+          retry = true;
+        } else {
+          sh_st[tid] *= 0.5f;
+        }
+        if (retry) { block_retry(P, pt); f = 0; }
+        if (f & B_CONV) {
+          P.iters[pt] = it;
+          P.status[pt] = DMN_STATUS_OK;
+          if (P.passes) atomicAdd(P.passes, (unsigned long long)np);
+          f &= ~B_ACT;
+        }
+        sh_fl[tid] = f;
+      }
+      __syncthreads();
+      fl = sh_fl[p];
+      if (fl & B_CONV) {   // the converged jumps, in the state's order
+        const int af = LS && (fl & B_CUR) ? D_A2 : D_A;
+        double* st = P.state_out + mypt;
+        for (int j = s ? 7 : 6; j >= 0; --j) {
+          const int h = heap(j);
+          const int row = CMP ? __ldg(t.hcid + h) : (1 << K) - 3 * (1 << (31 - __clz(h + 1))) + h + 1;
+          if (CMP && row < 0) continue;
+#pragma unroll
+          for (int k = 0; k < 3; ++k) st[(nzf + 3 * row + k) * n] = c.d(af + k, j);
+        }
+      }
+      const bool cont = fl & B_CONT;
+      if (!__syncthreads_or(cont)) {
+        if (tid < nP) sh_fl[tid] &= ~B_CONV;
+        continue;
+      }
+      // ---- S: FP32 condensation up
+      if (cont && !dead) {
+        Sub32 res, pq, ph;
+#pragma unroll 1
+        for (int q = 0; q < 4; ++q) {
+          LeafTan<float> DL, DR;
+          leaf_tan32(t.ph[0], c.tanf + (both ? 16 * q : 8 * q) * BT, DL);
+          leaf_tan32(t.ph[1], c.tanf + (both ? 16 * q + 8 : 8 * q) * BT, DR);
+          condense32_bottom<CMP>(t, c, heap(3 + q), 3 + q, DL, DR, t.ph[0].kind == 0, t.ph[1].kind == 0, res);
+          if (q & 1) {
+            Sub32 o;
+            condense32<CMP>(t, c, heap(1 + (q >> 1)), 1 + (q >> 1), pq, res, o);
+            if (q == 1) ph = o; else res = o;
+          } else {
+            pq = res;
+          }
+        }
+        Sub32 o;
+        condense32<CMP>(t, c, heap(0), 0, ph, res, o);
+#pragma unroll
+        for (int I = 0; I < 6; ++I) sh_c[I][tid] = o.ds[I];
+#pragma unroll
+        for (int k = 0; k < 21; ++k) sh_c[6 + k][tid] = o.C[k];
+      } else if (cont) {
+#pragma unroll
+        for (int k = 0; k < 27; ++k) sh_c[k][tid] = 0.f;
+      }
+      __syncthreads();
+      for (int l = Kt - 1; l >= 0; --l) {
+        if (cont && lev == l) {
+          Sub32 L, R, o;
+#pragma unroll
+          for (int I = 0; I < 6; ++I) { L.ds[I] = sh_c[I][pos]; R.ds[I] = sh_c[I][pos + half]; }
+#pragma unroll
+          for (int k = 0; k < 21; ++k) { L.C[k] = sh_c[6 + k][pos]; R.C[k] = sh_c[6 + k][pos + half]; }
+          condense32<CMP>(t, c, s - 1, 7, L, R, o);
+#pragma unroll
+          for (int I = 0; I < 6; ++I) sh_c[I][pos] = o.ds[I];
+#pragma unroll
+          for (int k = 0; k < 21; ++k) sh_c[6 + k][pos] = o.C[k];
+        }
+        __syncthreads();
+      }
+      // ---- B: da1 down, J da1 up (FP64), second FP32 solve up
+      if (cont && s == 0) {
+#pragma unroll
+        for (int I = 0; I < 6; ++I) { sh_e[I][p] = 0.0; sd[I][p] = 0.f; }
+      }
+      __syncthreads();
+      for (int l = 0; l < Kt; ++l) {
+        if (cont && lev == l) {
+          double e[6], eL[6], eR[6];
+          float de[6], dL[6], dR[6];
+#pragma unroll
+          for (int I = 0; I < 6; ++I) { e[I] = sh_e[I][pos]; de[I] = sd[I][pos]; }
+          down<CMP, LS, true>(t, c, s - 1, 7, 0, 0, true, 1.0, e, de, eL, eR, dL, dR);
+#pragma unroll
+          for (int I = 0; I < 6; ++I) {
+            sh_e[I][pos] = eL[I]; sh_e[I][pos + half] = eR[I];
+            sd[I][pos] = dL[I]; sd[I][pos + half] = dR[I];
+          }
+        }
+        __syncthreads();
+      }
+      float q2 = 0.f;
+      if (cont && !dead) {
+        double e[6], eL[6], eR[6], fL[6], fR[6], tq[6], th[6], tb[6];
+        float de[6], dL[6], dR[6], dfL[6], dfR[6], xq[6], xh[6], xb[6];
+#pragma unroll
+        for (int I = 0; I < 6; ++I) { e[I] = sh_e[I][tid]; de[I] = sd[I][tid]; }
+        down<CMP, LS, true>(t, c, heap(0), 0, 0, 0, true, 1.0, e, de, eL, eR, dL, dR);
+#pragma unroll 1
+        for (int q = 0; q < 4; ++q) {
+          if (!(q & 1)) {
+#pragma unroll
+            for (int I = 0; I < 6; ++I) { e[I] = q ? eR[I] : eL[I]; de[I] = q ? dR[I] : dL[I]; }
+            down<CMP, LS, true>(t, c, heap(1 + (q >> 1)), 1 + (q >> 1), 0, 0, true, 1.0, e, de, fL, fR, dfL, dfR);
+          }
+          double gL[6], gR[6], t0[6], t1[6];
+#pragma unroll
+          for (int I = 0; I < 6; ++I) { e[I] = q & 1 ? fR[I] : fL[I]; de[I] = q & 1 ? dfR[I] : dfL[I]; }
+          down<CMP, LS, true>(t, c, heap(3 + q), 3 + q, 0, 0, true, 1.0, e, de, gL, gR, nullptr, nullptr);
+          leaf_apply(t.ph[0], c.tan + (both ? 16 * q : 8 * q) * BT, gL, t0);
+          leaf_apply(t.ph[1], c.tan + (both ? 16 * q + 8 : 8 * q) * BT, gR, t1);
+          up_b<CMP, true>(t, c, heap(3 + q), 3 + q, t0, t1, nullptr, nullptr, tb, xb, q2);
+          if (q & 1) {
+            double o[6];
+            float x[6];
+            up_b<CMP, false>(t, c, heap(1 + (q >> 1)), 1 + (q >> 1), tq, tb, xq, xb, o, x, q2);
+#pragma unroll
+            for (int I = 0; I < 6; ++I) {
+              if (q == 1) { th[I] = o[I]; xh[I] = x[I]; } else { tb[I] = o[I]; xb[I] = x[I]; }
+            }
+          } else {
+#pragma unroll
+            for (int I = 0; I < 6; ++I) { tq[I] = tb[I]; xq[I] = xb[I]; }
+          }
+        }
+        up_b<CMP, false>(t, c, heap(0), 0, th, tb, xh, xb, e, de, q2);
+#pragma unroll
+        for (int I = 0; I < 6; ++I) { sh_e[I][tid] = e[I]; sd[I][tid] = de[I]; }
+      } else if (cont) {
+#pragma unroll
+        for (int I = 0; I < 6; ++I) { sh_e[I][tid] = 0.0; sd[I][tid] = 0.f; }
+      }
+      __syncthreads();
+      for (int l = Kt - 1; l >= 0; --l) {
+        if (cont && lev == l) {
+          double tL[6], tR[6], tb[6];
+          float xL[6], xR[6], xb[6];
+#pragma unroll
+          for (int I = 0; I < 6; ++I) {
+            tL[I] = sh_e[I][pos]; tR[I] = sh_e[I][pos + half];
+            xL[I] = sd[I][pos]; xR[I] = sd[I][pos + half];
+          }
+          up_b<CMP, false>(t, c, s - 1, 7, tL, tR, xL, xR, tb, xb, q2);
+#pragma unroll
+          for (int I = 0; I < 6; ++I) { sh_e[I][pos] = tb[I]; sd[I][pos] = xb[I]; }
+        }
+        __syncthreads();
+      }
+      for (int o = 16; o >= nP; o >>= 1) q2 += __shfl_xor_sync(0xffffffffu, q2, o);
+      if (nP >= 32) sh_r[tid] = (double)q2;
+      else if (lane < nP) sh_r[(tid >> 5) * nP + lane] = (double)q2;
+      __syncthreads();
+      if (tid < nP) {
+        int f = sh_fl[tid];
+        if (f & B_CONT) {
+          double r = 0.0;
+          for (int k = 0; k < groups; ++k) r += sh_r[k * nP + tid];
+          if (!(r <= (double)REFINE_MAX * REFINE_MAX * rn_acc * rn_acc)) { block_retry(P, pt); f = 0; }
+        }
+        sh_fl[tid] = f & ~(B_CONT | B_CONV);
+      }
+    }
+    __syncthreads();
+  }
+  // points of unknown trees (the last bucket of the sort)
+  if (P.perm) {
+    const unsigned long long end = P.counter[10 + P.F.n], begin = end - P.counter[1 + P.F.n];
+    for (unsigned long long i = begin + blockIdx.x * (unsigned long long)BT + tid; i < end;
+         i += (unsigned long long)gridDim.x * BT)
+      block_bad_tree(P, P.perm[i]);
+  }
+}
+
+template <bool LS, bool CMP>
+static void launch(const BlockParams& P, unsigned grid, cudaStream_t s) {
+  k_newton_block<LS, CMP><<<grid, BT, sizeof(double) * 3 * BT, s>>>(P);
+}
+
+void launch_block(const BlockParams& P, bool ls, bool cmp, unsigned grid, cudaStream_t s) {
+  if (ls && cmp) launch<true, true>(P, grid, s);
+  else if (ls) launch<true, false>(P, grid, s);
+  else if (cmp) launch<false, true>(P, grid, s);
+  else launch<false, false>(P, grid, s);
+}
+
+}  // namespace dmn

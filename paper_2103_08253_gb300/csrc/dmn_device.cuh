@@ -87,6 +87,8 @@ struct TreeDev {
   const int* kid;    // [2 N] children of each laminate: >= 0 a laminate, -1 - phase a leaf
   const int* hcid;   // [2^K - 1] the laminate standing at each heap position, -1 for none (compressed trees)
   const int* kslot;  // [2 N] the state slot of each child that is a leaf (-1: elastic, or a laminate child)
+  const int* hdir;   // [2^K - 1] what each heap position does: 0 holds a laminate, 1 / 2 passes its left / right
+                     // side on, 3 nothing below it is left
   const int* lslot;  // [2^K] the state slot of each leaf (-1: elastic, or of weight zero)
 };
 

@@ -50,7 +50,16 @@ struct NewtonParams {
   int min_corr;       // corrections before the criterion may end the iteration (1 for the FP64 form after
                       // the first stage: one quadratic step from the FP32 iterate, so that the accepted
                       // iterate is as far inside the criterion as in the plain FP64 iteration)
+  const unsigned long long* n_list = nullptr;  // the points are perm[0 .. *n_list) instead of all n
 };
+
+// Status of a point that k_newton_block leaves to the all-FP64 kernels; never returned to a caller.
+constexpr int32_t STATUS_RETRY = -1;
+
+// number of points a launch works through
+__device__ __forceinline__ unsigned long long n_work(int64_t n, const unsigned long long* n_list) {
+  return n_list ? *n_list : (unsigned long long)n;
+}
 
 // Small calls: one point per group of G lanes of a warp (G = 32, 16 or 8; the paper's start; heap
 // trees or compressed ones), the group's lanes sharing each level of the tree (warp_tree_pass).
@@ -78,5 +87,44 @@ void launch_warp(const NewtonParams<T>& P, bool ls, int lanes, unsigned grid, do
 // `scr` holds grid * 128 / lanes slots of warp_slot_doubles<double>(P.N_max) doubles
 template <bool CMP>
 void launch_sweep_warp(const NewtonParams<double>& P, int lanes, unsigned grid, double* scr, cudaStream_t s);
+
+// The CTA organisation of the FP64 form (csrc/dmn_block.cu).  counter: [1..9] points per tree and
+// [10..18] their ends in perm (several trees), [21..28] work counters per tree, [29] points on the list.
+constexpr int BLOCK_THREADS = 256;
+constexpr int BLOCK_CTAS_PER_SM = 2;
+struct BlockParams {
+  Forest F;
+  int64_t n;
+  int N_max, leaf_slots;   // leaf_slots: leaves with a state in a subtree of 8 (4, or 8 with two inelastic phases)
+  const int32_t* tid;
+  const int64_t* perm;
+  const double* state_in;
+  double *state_out, *stress, *tangent;
+  int32_t *iters, *status;
+  const double* nbuf;
+  char* scratch;           // block_scratch_bytes per CTA
+  unsigned long long* counter;
+  int64_t* list;           // points left to the all-FP64 kernels
+  double tol;
+  int max_iter;
+  unsigned long long* passes;
+};
+// per thread, for 8 laminates: jumps (two buffers), normals, residuals (FP64: 12 fields), normals, H, Kn^-1, g,
+// step (FP32: 33 fields); per leaf its state and tangent (FP64: 14) and the tangent in FP32 (8)
+__host__ __device__ inline size_t block_scratch_bytes(int leaf_slots) {
+  return (size_t)BLOCK_THREADS * (sizeof(double) * (8 * 12 + 14 * leaf_slots) + sizeof(float) * (8 * 33 + 8 * leaf_slots));
+}
+__device__ __forceinline__ void block_bad_tree(const BlockParams& P, int64_t pt) {
+  const double qnan = __longlong_as_double(0x7ff8000000000000LL);
+  P.iters[pt] = 0;
+  P.status[pt] = DMN_STATUS_BAD_TREE;
+  for (int I = 0; I < 6; ++I) P.stress[6 * pt + I] = qnan;
+  for (int I = 0; I < 36; ++I) P.tangent[36 * pt + I] = qnan;
+}
+__device__ __forceinline__ void block_retry(const BlockParams& P, int64_t pt) {
+  P.status[pt] = STATUS_RETRY;
+  P.list[atomicAdd(P.counter + 29, 1ull)] = pt;
+}
+void launch_block(const BlockParams& P, bool ls, bool cmp, unsigned grid, cudaStream_t s);
 
 }  // namespace dmn

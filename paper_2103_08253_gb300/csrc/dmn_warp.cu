@@ -47,7 +47,7 @@ __global__ void __launch_bounds__(128) k_newton_warp(NewtonParams<T> P, double* 
       unsigned long long i = 0;
       if (lane == 0) i = atomicAdd(P.counter, 1ull);
       i = __shfl_sync(gmask, i, 0, G);
-      if (i >= (unsigned long long)P.n) return false;
+      if (i >= n_work(P.n, P.n_list)) return false;
       point_of(P.perm, P.tid, P.F.n, (int64_t)i, pt, tr);
       if (tr < P.F.n) break;
       if (lane == 0) {   // unknown tree: report and take the next point
@@ -193,9 +193,9 @@ __global__ void __launch_bounds__(128) k_sweep_warp(NewtonParams<double> P, doub
       unsigned long long i = 0;
       if (lane == 0) i = atomicAdd(P.counter, 1ull);
       i = __shfl_sync(gmask, i, 0, G);
-      if (i >= (unsigned long long)P.n) return false;
+      if (i >= n_work(P.n, P.n_list)) return false;
       point_of(P.perm, P.tid, P.F.n, (int64_t)i, pt, tr);
-      if (tr < P.F.n && P.status[pt] != DMN_STATUS_NONFINITE) break;
+      if (tr < P.F.n && P.status[pt] != DMN_STATUS_NONFINITE && P.status[pt] != STATUS_RETRY) break;
     }
     const TreeDev& t = P.F.t[tr];
     const int nzf = 6 * t.nz;
