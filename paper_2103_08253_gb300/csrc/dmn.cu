@@ -1286,7 +1286,7 @@ cudaError_t alloc_ws(const dmn_handle* h, WorkSet& w) {
     e = cudaMalloc(&w.scr_s, sizeof(float) * (size_t)(27 * h->N_max) * w.nslots_s);
   }
   if (e == cudaSuccess && block_on(h))
-    e = cudaMalloc(&w.scr_b, block_scratch_bytes(block_leaf_slots(h)) * (size_t)(h->n_sm * BLOCK_CTAS_PER_SM));
+    e = cudaMalloc(&w.scr_b, block_scratch_bytes(block_leaf_slots(h), h->opt.line_search != 0) * (size_t)(h->n_sm * BLOCK_CTAS_PER_SM));
   if (e == cudaSuccess && warp_possible(h)) {
     // one slot per group of the smallest size the handle may use
     w.nwarps_w = (int64_t)h->n_sm * WARP_CTAS_PER_SM * 128 / (h->opt.warp_lanes ? h->opt.warp_lanes : WARP_MIN_LANES);
@@ -1453,7 +1453,8 @@ int update_on(dmn_handle* h, WorkSet& w, int64_t n, int64_t n_call, const int32_
     BlockParams P{F, n, NM, block_leaf_slots(h), tree_id, perm, state_in, state_out, stress, tangent, iters, status,
                   w.nbuf, w.scr_b, w.counter, w.list, h->opt.tol, h->opt.max_iter, passes ? passes + 1 : nullptr};
     const int64_t ctas = div_up(n, BLOCK_THREADS >> (h->K_max - 3));
-    launch_block(P, ls, h->cmp, (unsigned)std::min<int64_t>(ctas, (int64_t)h->n_sm * BLOCK_CTAS_PER_SM), s);
+    e = launch_block(P, ls, h->cmp, (unsigned)std::min<int64_t>(ctas, (int64_t)h->n_sm * BLOCK_CTAS_PER_SM), s);
+    if (e != cudaSuccess) return cuda_fail(h, e, "dmn_update: launch");
   } else if (!mixed) {
     newton_f64(DP);
   } else {

@@ -5,11 +5,11 @@
 // only serves to solve J da = -R.  Here each iteration
 //   A  evaluates strains, leaf laws and the residual R in FP64 (and tests the criterion on it),
 //   S  condenses the leaf tangents in FP32 and solves for da1 (relative error some 1e-6),
-//   B  forms R + J da1 in FP64 with the FP64 leaf tangents and solves again in FP32 for da2,
+//   B  forms R + J da1 with pairs of FP32 numbers (about 46 bits) and solves again in FP32 for da2,
 // and applies da = da1 + da2, whose relative error is the product of the two solves' (1e-11, at most
 // some 1e-10 on the workloads' plastic paths), far below what the quadratic convergence leaves: the
-// iterates are those of the all-FP64 condensation, with its iteration counts.  A and B cost about 23 k
-// and 16 k FP64 instructions, a pass of the all-FP64 kernel 122 k.  The tangent comes from one FP64
+// iterates are those of the all-FP64 condensation, with its iteration counts.  A costs about 22 k FP64
+// instructions, a pass of the all-FP64 kernel 122 k; S and B cost none.  The tangent comes from one FP64
 // sweep at the converged jumps, as in the mixed form.
 //
 // A point for which the FP32 solve does not contract (|R + J da1| > REFINE_MAX |R|: tangents near
@@ -41,8 +41,39 @@ constexpr float REFINE_MAX = 1e-3f;
 constexpr int BLOCK_ITERS = 16;
 
 // scratch fields of a thread, in units of 8 laminates (7 of the subtree, then the top laminate)
-enum { D_A = 0, D_A2 = 3, D_N = 6, D_T = 9, D_END = 12 };                      // FP64
-enum { F_N = 0, F_H = 3, F_K = 21, F_G = 27, F_D = 30, F_END = 33 };           // FP32
+enum { D_A = 0, D_N = 3, D_A2 = 6 };                                               // FP64 (D_A2: line search)
+enum { F_H = 0, F_K = 18, F_G = 24, F_D = 27, F_T = 30, F_TL = 33, F_END = 36 };   // FP32
+
+// Pairs of FP32 numbers, value h + l (Dekker 1971: error-free sum and product): a sum costs 8 FP32
+// instructions, a product 4, against 64 cycles of the FP64 unit for a warp's FP64 instruction.
+struct pair {
+  float h, l;
+};
+__device__ __forceinline__ pair add(pair a, pair b) {
+  const float s = __fadd_rn(a.h, b.h), t = __fsub_rn(s, a.h);
+  const float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, t)), __fsub_rn(b.h, t));
+  return {s, __fadd_rn(e, __fadd_rn(a.l, b.l))};
+}
+__device__ __forceinline__ pair neg(pair a) { return {-a.h, -a.l}; }
+__device__ __forceinline__ pair mul(pair a, float b) {
+  const float p = __fmul_rn(a.h, b);
+  return {p, __fmaf_rn(a.l, b, __fmaf_rn(a.h, b, -p))};
+}
+__device__ __forceinline__ pair mul(pair a, pair b) {
+  const float p = __fmul_rn(a.h, b.h);
+  return {p, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, __fmaf_rn(a.h, b.h, -p)))};
+}
+// x as a pair, with integer instructions (as narrow_rn): h the 24 leading bits truncated, l the 29 bits
+// below them.  Magnitudes below FP32's normal range give 0 (l: below 2^-74), above it infinity.
+__device__ __forceinline__ pair split(double x) {
+  const unsigned long long b = bits_of(x);
+  const unsigned hi = (unsigned)(b >> 32), lo = (unsigned)b, sign = hi & 0x80000000u, e = (hi >> 20) & 0x7ffu;
+  unsigned h = ((e - 896u) << 23) + (((hi & 0xfffffu) << 3) | (lo >> 29));
+  if (e <= 896u) h = 0u;
+  if (e >= 1151u) h = 0x7f800000u;
+  const float l = e > 948u && e < 1151u ? __uint2float_rn(lo & 0x1fffffffu) * float_of((e - 948u) << 23) : 0.f;
+  return {float_of(sign | h), float_of(sign | bits_of(l))};
+}
 
 // laminate h (heap order, 0-based) of the full tree: its number in the handle's arrays and its fractions.
 // mode 0: a laminate; 1 / 2: passes its left / right side on (the other is weightless); 3: nothing alive
@@ -62,8 +93,7 @@ struct Ctx {
   double* D;      // this thread's FP64 scratch: field f of laminate j at D[(8 f + j) BT]
   float* F;       // this thread's FP32 scratch
   double* z;      // leaf states: z[(6 leaf + c) BT]
-  double* tan;    // leaf tangents mu, c, m: tan[(8 leaf + c) BT]
-  float* tanf;    // their FP32 copies
+  float* tan;     // leaf tangents mu, c, m as pairs: h at tan[(16 leaf + k) BT], l at tan[(16 leaf + 8 + k) BT]
   __device__ double& d(int f, int j) const { return D[(8 * f + j) * BT]; }
   __device__ float& f(int f, int j) const { return F[(8 * f + j) * BT]; }
 };
@@ -72,12 +102,13 @@ __device__ __forceinline__ void load3(const Ctx& c, int f, int j, double v[3]) {
 #pragma unroll
   for (int k = 0; k < 3; ++k) v[k] = c.d(f + k, j);
 }
+__device__ __forceinline__ void normal32(const Ctx& c, int j, float n[3], float nr[3]) {
+#pragma unroll
+  for (int k = 0; k < 3; ++k) { n[k] = narrow_rn(c.d(D_N + k, j)); nr[k] = n[k] * (float)RS2; }
+}
 
-// The FP32 step of laminate j: g + H de; hands the corrections to the children (dL, dR).
-template <bool CMP>
-__device__ __forceinline__ void step32(const TreeDev& t, const Ctx& c, const Lam<CMP>& q, int j, const float de[6],
-                                       float da[3], float dL[6], float dR[6]) {
-  const float n[3] = {c.f(F_N, j), c.f(F_N + 1, j), c.f(F_N + 2, j)};
+// The FP32 step of laminate j, g + H de.
+__device__ __forceinline__ void step32(const Ctx& c, int j, const float de[6], float da[3]) {
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     float v = c.f(F_G + k, j);
@@ -85,22 +116,14 @@ __device__ __forceinline__ void step32(const TreeDev& t, const Ctx& c, const Lam
     for (int I = 0; I < 6; ++I) v += c.f(F_H + 6 * k + I, j) * de[I];
     da[k] = v;
   }
-  if (dL) {
-    const float c1 = __ldg(t.c1f + q.id), c2 = __ldg(t.c2f + q.id);
-    const float nr[3] = {n[0] * (float)RS2, n[1] * (float)RS2, n[2] * (float)RS2};
-    float Nd[6];
-    N_apply<float>(n, nr, da, Nd);
-#pragma unroll
-    for (int I = 0; I < 6; ++I) { dL[I] = de[I] - c2 * Nd[I]; dR[I] = de[I] + c1 * Nd[I]; }
-  }
 }
 
-// A, downwards: the jumps of laminate j corrected (apply) and the children's strains.
-// B, downwards: the step da1 stored and its strains.  de: the FP32 correction handed down.
-template <bool CMP, bool LS, bool PHASE_B>
-__device__ __forceinline__ void down(const TreeDev& t, const Ctx& c, int h, int j, int a_in, int a_out, bool apply,
-                                     double step, const double e[6], const float de[6], double eL[6], double eR[6],
-                                     float* dL, float* dR) {
+// A, downwards: the jumps of laminate j corrected (apply) and the children's strains.  de: the FP32
+// correction of the second solve handed down (dL, dR: to the children; NULL for leaves).
+template <bool CMP, bool LS>
+__device__ __forceinline__ void down_a(const TreeDev& t, const Ctx& c, int h, int j, int a_in, int a_out, bool apply,
+                                       double step, const double e[6], const float de[6], double eL[6], double eR[6],
+                                       float* dL, float* dR) {
   const Lam<CMP> q(t, h);
   if (CMP && q.mode) {
 #pragma unroll
@@ -109,29 +132,33 @@ __device__ __forceinline__ void down(const TreeDev& t, const Ctx& c, int h, int 
   }
   double nd[3], a[3];
   load3(c, D_N, j, nd);
-  if (PHASE_B) {
+  load3(c, a_in, j, a);
+  if (apply) {
     float da[3];
-    step32<CMP>(t, c, q, j, de, da, dL, dR);
+    step32(c, j, de, da);
+    if (dL) {
+      const float c1 = __ldg(t.c1f + q.id), c2 = __ldg(t.c2f + q.id);
+      const float n[3] = {narrow_rn(nd[0]), narrow_rn(nd[1]), narrow_rn(nd[2])};
+      const float nr[3] = {n[0] * (float)RS2, n[1] * (float)RS2, n[2] * (float)RS2};
+      float Nd[6];
+      N_apply<float>(n, nr, da, Nd);
 #pragma unroll
-    for (int k = 0; k < 3; ++k) { c.f(F_D + k, j) = da[k]; a[k] = widen(da[k]); }
+      for (int I = 0; I < 6; ++I) { dL[I] = de[I] - c2 * Nd[I]; dR[I] = de[I] + c1 * Nd[I]; }
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const double s = widen(c.f(F_D + k, j)) + widen(da[k]);
+      a[k] = LS ? a[k] + step * s : a[k] + s;
+      c.d(a_out + k, j) = a[k];
+    }
   } else {
-    load3(c, a_in, j, a);
-    if (apply) {
-      float da[3];
-      step32<CMP>(t, c, q, j, de, da, dL, dR);
+    if (dL) {
 #pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        const double s = widen(c.f(F_D + k, j)) + widen(da[k]);
-        a[k] = LS ? a[k] + step * s : a[k] + s;
-        c.d(a_out + k, j) = a[k];
-      }
-    } else {
+      for (int I = 0; I < 6; ++I) dL[I] = dR[I] = 0.f;
+    }
+    if (LS) {
 #pragma unroll
-      for (int I = 0; I < 6; ++I) if (dL) dL[I] = dR[I] = 0.f;
-      if (LS) {
-#pragma unroll
-        for (int k = 0; k < 3; ++k) c.d(a_out + k, j) = a[k];
-      }
+      for (int k = 0; k < 3; ++k) c.d(a_out + k, j) = a[k];
     }
   }
   const double ndr[3] = {nd[0] * RS2, nd[1] * RS2, nd[2] * RS2};
@@ -139,6 +166,37 @@ __device__ __forceinline__ void down(const TreeDev& t, const Ctx& c, int h, int 
   N_apply<double>(nd, ndr, a, Na);
 #pragma unroll
   for (int I = 0; I < 6; ++I) { eL[I] = e[I] - q.c2 * Na[I]; eR[I] = e[I] + q.c1 * Na[I]; }
+}
+
+// N(n) x for x in FP32 and N(n)^T v, in pairs
+__device__ __forceinline__ void pair_normal(const Ctx& c, int j, pair n[3], pair nr[3]) {
+#pragma unroll
+  for (int k = 0; k < 3; ++k) { n[k] = split(c.d(D_N + k, j)); nr[k] = mul(n[k], split(RS2)); }
+}
+
+// B, downwards: the step da1 of laminate j stored, and its strains in the children.
+template <bool CMP>
+__device__ __forceinline__ void down_b(const TreeDev& t, const Ctx& c, int h, int j, const pair e[6], pair eL[6],
+                                       pair eR[6]) {
+  const Lam<CMP> q(t, h);
+  if (CMP && q.mode) {
+#pragma unroll
+    for (int I = 0; I < 6; ++I) eL[I] = eR[I] = e[I];
+    return;
+  }
+  float de[6], x[3];
+#pragma unroll
+  for (int I = 0; I < 6; ++I) de[I] = e[I].h;
+  step32(c, j, de, x);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) c.f(F_D + k, j) = x[k];
+  pair n[3], nr[3];
+  pair_normal(c, j, n, nr);
+  const pair Nx[6] = {mul(n[0], x[0]), mul(n[1], x[1]), mul(n[2], x[2]), add(mul(nr[2], x[1]), mul(nr[1], x[2])),
+                      add(mul(nr[2], x[0]), mul(nr[0], x[2])), add(mul(nr[1], x[0]), mul(nr[0], x[1]))};
+  const pair c2 = split(-q.c2);
+#pragma unroll
+  for (int I = 0; I < 6; ++I) { eL[I] = add(e[I], mul(c2, Nx[I])); eR[I] = add(eL[I], Nx[I]); }   // c1 = 1 - c2
 }
 
 // A, upwards: residual of laminate j (t = N^T (s_R - s_L), stored) and the average stress.
@@ -155,17 +213,20 @@ __device__ __forceinline__ void up_a(const TreeDev& t, const Ctx& c, int h, int 
   load3(c, D_N, j, nd);
   residual_share<double>(nd, q.c1, q.c2, __ldg(t.sc + q.id), sL, sR, sb, u, r2);
 #pragma unroll
-  for (int k = 0; k < 3; ++k) c.d(D_T + k, j) = u[k];
+  for (int k = 0; k < 3; ++k) {
+    const pair v = split(u[k]);
+    c.f(F_T + k, j) = v.h;
+    c.f(F_TL + k, j) = v.l;
+  }
 }
 
 // B, upwards: the linearised residual of laminate j after da1, u = N^T (s_R - s_L) + N^T (tau_R - tau_L)
-// in FP64, then the FP32 solve's upward half with the stored H and Kn^-1:
+// in pairs, then the FP32 solve's upward half with the stored H and Kn^-1:
 //   u += N^T (ds_R - ds_L),  g = -Kn^-1 u,  ds = c1 ds_L + c2 ds_R + c1 c2 H^T u.
 // BOT: the children are leaves (ds = 0 there).
 template <bool CMP, bool BOT>
-__device__ __forceinline__ void up_b(const TreeDev& t, const Ctx& c, int h, int j, const double tL[6],
-                                     const double tR[6], const float dsL[6], const float dsR[6], double tb[6],
-                                     float ds[6], float& r2) {
+__device__ __forceinline__ void up_b(const TreeDev& t, const Ctx& c, int h, int j, const pair tL[6], const pair tR[6],
+                                     const float dsL[6], const float dsR[6], pair tb[6], float ds[6], float& r2) {
   const Lam<CMP> q(t, h);
   if (CMP && q.mode) {
 #pragma unroll
@@ -175,26 +236,30 @@ __device__ __forceinline__ void up_b(const TreeDev& t, const Ctx& c, int h, int 
     }
     return;
   }
-  double nd[3], d[6], v[3];
-  load3(c, D_N, j, nd);
-  const double ndr[3] = {nd[0] * RS2, nd[1] * RS2, nd[2] * RS2};
+  pair n[3], nr[3], d[6];
+  pair_normal(c, j, n, nr);
+  const pair p2 = split(q.c2);
 #pragma unroll
-  for (int I = 0; I < 6; ++I) { d[I] = tR[I] - tL[I]; tb[I] = tL[I] + q.c2 * d[I]; }
-  Nt_apply<double>(nd, ndr, d, v);
+  for (int I = 0; I < 6; ++I) { d[I] = add(tR[I], neg(tL[I])); tb[I] = add(tL[I], mul(p2, d[I])); }
+  const pair v[3] = {add(mul(n[0], d[0]), add(mul(nr[2], d[4]), mul(nr[1], d[5]))),
+                     add(mul(n[1], d[1]), add(mul(nr[2], d[3]), mul(nr[0], d[5]))),
+                     add(mul(n[2], d[2]), add(mul(nr[1], d[3]), mul(nr[0], d[4])))};
   float u[3];
 #pragma unroll
-  for (int k = 0; k < 3; ++k) u[k] = narrow_rn(c.d(D_T + k, j) + v[k]);
+  for (int k = 0; k < 3; ++k) {
+    const pair x = add(pair{c.f(F_T + k, j), c.f(F_TL + k, j)}, v[k]);
+    u[k] = x.h + x.l;
+  }
   const float sc = __ldg(t.scf + q.id), c2 = __ldg(t.c2f + q.id), c12 = __ldg(t.c12f + q.id);
 #pragma unroll
   for (int k = 0; k < 3; ++k) r2 += (sc * u[k]) * (sc * u[k]);
   float dd[6];
   if (!BOT) {
-    const float n[3] = {c.f(F_N, j), c.f(F_N + 1, j), c.f(F_N + 2, j)};
-    const float nr[3] = {n[0] * (float)RS2, n[1] * (float)RS2, n[2] * (float)RS2};
+    const float m[3] = {n[0].h, n[1].h, n[2].h}, mr[3] = {nr[0].h, nr[1].h, nr[2].h};
     float w[3];
 #pragma unroll
     for (int I = 0; I < 6; ++I) dd[I] = dsR[I] - dsL[I];
-    Nt_apply<float>(n, nr, dd, w);
+    Nt_apply<float>(m, mr, dd, w);
 #pragma unroll
     for (int k = 0; k < 3; ++k) u[k] += w[k];
   }
@@ -255,8 +320,8 @@ __device__ __forceinline__ void condense32(const TreeDev& t, const Ctx& c, int h
     return;
   }
   const float c2 = __ldg(t.c2f + q.id), c12 = __ldg(t.c12f + q.id);
-  const float n[3] = {c.f(F_N, j), c.f(F_N + 1, j), c.f(F_N + 2, j)};
-  const float nr[3] = {n[0] * (float)RS2, n[1] * (float)RS2, n[2] * (float)RS2};
+  float n[3], nr[3];
+  normal32(c, j, n, nr);
   float dC[21], Ch[21], X[6][3], B[6][3], u[3], w[3], dd[6];
 #pragma unroll
   for (int k = 0; k < 21; ++k) { dC[k] = R.C[k] - L.C[k]; Ch[k] = R.C[k] - c2 * dC[k]; }
@@ -276,7 +341,7 @@ __device__ __forceinline__ void condense32(const TreeDev& t, const Ctx& c, int h
   for (int I = 0; I < 6; ++I) dd[I] = R.ds[I] - L.ds[I];
   Nt_apply<float>(n, nr, dd, w);
 #pragma unroll
-  for (int k = 0; k < 3; ++k) u[k] = narrow_rn(c.d(D_T + k, j)) + w[k];
+  for (int k = 0; k < 3; ++k) u[k] = c.f(F_T + k, j) + w[k];
 #pragma unroll
   for (int I = 0; I < 6; ++I) o.ds[I] = L.ds[I] + c2 * dd[I];
 #pragma unroll
@@ -326,8 +391,8 @@ __device__ __forceinline__ void condense32_bottom(const TreeDev& t, const Ctx& c
   }
   if (CMP && q.mode) return;
   const float c12 = __ldg(t.c12f + q.id);
-  const float n[3] = {c.f(F_N, j), c.f(F_N + 1, j), c.f(F_N + 2, j)};
-  const float nr[3] = {n[0] * (float)RS2, n[1] * (float)RS2, n[2] * (float)RS2};
+  float n[3], nr[3];
+  normal32(c, j, n, nr);
   const float a = c2 * L.mu + c1 * R.mu, b = c2 * (L.lam + L.mu) + c1 * (R.lam + R.mu);
   const float dlam = R.lam - L.lam, dmu2 = 2.f * (R.mu - L.mu), dld = dlam + dmu2;
   float k[3][3], B[6][3];
@@ -366,26 +431,32 @@ __device__ __forceinline__ void condense32_bottom(const TreeDev& t, const Ctx& c
   }
   float Ki[3][3];
   inv3_sym<float>(k[0][0], k[0][1], k[0][2], k[1][1], k[1][2], k[2][2], Ki);
-  const float u[3] = {narrow_rn(c.d(D_T, j)), narrow_rn(c.d(D_T + 1, j)), narrow_rn(c.d(D_T + 2, j))};
+  const float u[3] = {c.f(F_T, j), c.f(F_T + 1, j), c.f(F_T + 2, j)};
   solve32(c, j, c12, Ki, B, u, o.ds, o.C);
 }
 
-// D e of a leaf in FP64 (B): the phase's constants or the stored mu, c, m
-__device__ __forceinline__ void leaf_apply(const PhaseDev& ph, const double* s, const double e[6], double tau[6]) {
-  const double tr = e[0] + e[1] + e[2];
+// D e of a leaf in pairs (B): the phase's constants or the stored mu, c, m
+__device__ __forceinline__ void leaf_apply(const PhaseDev& ph, const float* s, const pair e[6], pair tau[6]) {
+  const pair tr = add(add(e[0], e[1]), e[2]);
   if (ph.kind == 0) {
-    const double lt = ph.lam * tr, g2 = 2.0 * ph.G;
+    const pair lt = mul(split(ph.lam), tr), g2 = split(2.0 * ph.G);
 #pragma unroll
-    for (int I = 0; I < 6; ++I) tau[I] = I < 3 ? g2 * e[I] + lt : g2 * e[I];
+    for (int I = 0; I < 6; ++I) { tau[I] = mul(g2, e[I]); if (I < 3) tau[I] = add(tau[I], lt); }
     return;
   }
-  const double mu = s[0];
-  double m[6], me = 0.0;
+  pair m[6], me;
 #pragma unroll
-  for (int I = 0; I < 6; ++I) { m[I] = s[(2 + I) * BT]; me += m[I] * e[I]; }
-  const double cm = s[BT] * me, g2 = 2.0 * mu, lt = (ph.K - (2.0 / 3.0) * mu) * tr;
+  for (int I = 0; I < 6; ++I) {
+    m[I] = pair{s[(2 + I) * BT], s[(10 + I) * BT]};
+    me = I ? add(me, mul(m[I], e[I])) : mul(m[I], e[I]);
+  }
+  const pair mu = {s[0], s[8 * BT]}, cm = neg(mul(pair{s[BT], s[9 * BT]}, me)), g2 = {2.f * mu.h, 2.f * mu.l};
+  const pair lt = mul(add(split(ph.K), mul(split(-2.0 / 3.0), mu)), tr);
 #pragma unroll
-  for (int I = 0; I < 6; ++I) tau[I] = (I < 3 ? g2 * e[I] + lt : g2 * e[I]) - cm * m[I];
+  for (int I = 0; I < 6; ++I) {
+    tau[I] = add(mul(g2, e[I]), mul(cm, m[I]));
+    if (I < 3) tau[I] = add(tau[I], lt);
+  }
 }
 
 }  // namespace
@@ -393,27 +464,75 @@ __device__ __forceinline__ void leaf_apply(const PhaseDev& ph, const double* s, 
 // flags of a slot
 enum { B_ACT = 1, B_NEW = 2, B_FIRST = 4, B_CONT = 8, B_CONV = 16, B_CUR = 32 };
 
+// Own-column accesses: a thread's vector of 6 in rows 0 .. 5 of a shared array, at column x.
+template <typename T>
+__device__ __forceinline__ void put6(T (*m)[BT], int x, const T v[6]) {
+#pragma unroll
+  for (int I = 0; I < 6; ++I) m[I][x] = v[I];
+}
+template <typename T>
+__device__ __forceinline__ void get6(T (*m)[BT], int x, T v[6]) {
+#pragma unroll
+  for (int I = 0; I < 6; ++I) v[I] = m[I][x];
+}
+__device__ __forceinline__ void put6(float (*m)[BT], int x, const pair v[6]) {
+#pragma unroll
+  for (int I = 0; I < 6; ++I) { m[I][x] = v[I].h; m[6 + I][x] = v[I].l; }
+}
+__device__ __forceinline__ void get6(float (*m)[BT], int x, pair v[6]) {
+#pragma unroll
+  for (int I = 0; I < 6; ++I) v[I] = pair{m[I][x], m[6 + I][x]};
+}
+__device__ __forceinline__ void put27(float (*m)[BT], int x, const Sub32& v) {
+#pragma unroll
+  for (int I = 0; I < 6; ++I) m[I][x] = v.ds[I];
+#pragma unroll
+  for (int k = 0; k < 21; ++k) m[6 + k][x] = v.C[k];
+}
+__device__ __forceinline__ void get27(float (*m)[BT], int x, Sub32& v) {
+#pragma unroll
+  for (int I = 0; I < 6; ++I) v.ds[I] = m[I][x];
+#pragma unroll
+  for (int k = 0; k < 21; ++k) v.C[k] = m[6 + k][x];
+}
+
+// Shared memory: what a level hands to the next, at the column of its leftmost subtree (in place: a
+// laminate's own column is its left child's); between levels a thread's own column keeps what its depth-first
+// walk sets aside, with sh_s for the level below.
+struct BlockShared {
+  double e[6][BT];       // strains down, stresses up (FP64, or pairs in 12 FP32 rows)
+  float c[27][BT];       // FP32 condensation up; rows 0 .. 5 also the FP32 corrections
+  float s[27][BT];       // the bottom walk's set-aside vectors (FP64: the first 12 rows)
+  double r[BT];          // partial residual norms
+  long long pt[BT];
+  int fl[BT];
+  float st[BT];
+};
+
 template <bool LS, bool CMP>
 __global__ void __launch_bounds__(BT, 2) k_newton_block(BlockParams P) {
-  __shared__ double sh_e[6][BT];      // strains handed down, stresses handed up, at the leftmost subtree's place
-  __shared__ float sh_c[27][BT];      // FP32 results handed up; its first rows the corrections handed down
-  extern __shared__ double dyn[];
-  double* sh_r = dyn;                 // [BT] partial residual norms
-  long long* sh_pt = (long long*)(dyn + BT);
-  int* sh_fl = (int*)(dyn + 2 * BT);
-  float* sh_st = (float*)(sh_fl + BT);
+  extern __shared__ __align__(16) char dyn[];
+  BlockShared& M = *reinterpret_cast<BlockShared*>(dyn);
+  double (*const sh_e)[BT] = M.e;
+  float (*const sh_c)[BT] = M.c;
+  double (*const sh_s)[BT] = reinterpret_cast<double (*)[BT]>(M.s);
+  float (*const sh_p)[BT] = reinterpret_cast<float (*)[BT]>(M.e);   // pairs
+  float (*const sh_x)[BT] = M.s + 12;
+  double* const sh_r = M.r;
+  long long* const sh_pt = M.pt;
+  int* const sh_fl = M.fl;
+  float* const sh_st = M.st;
   const int tid = threadIdx.x, lane = tid & 31;
   const size_t n = (size_t)P.n;
   Ctx c;
   {
-    char* base = P.scratch + (size_t)blockIdx.x * block_scratch_bytes(P.leaf_slots);
+    char* base = P.scratch + (size_t)blockIdx.x * block_scratch_bytes(P.leaf_slots, LS);
     double* D = (double*)base;
     c.D = D + tid;
-    c.z = D + (size_t)8 * D_END * BT + tid;
-    c.tan = c.z + (size_t)6 * P.leaf_slots * BT;
-    float* F = (float*)(D + (size_t)(8 * D_END + 14 * P.leaf_slots) * BT);
+    c.z = D + (size_t)8 * (LS ? 9 : 6) * BT + tid;
+    float* F = (float*)(D + (size_t)(8 * (LS ? 9 : 6) + 6 * P.leaf_slots) * BT);
     c.F = F + tid;
-    c.tanf = F + (size_t)8 * F_END * BT + tid;
+    c.tan = F + (size_t)8 * F_END * BT + tid;
   }
   for (int tr = 0; tr < P.F.n; ++tr) {
     const TreeDev& t = P.F.t[tr];
@@ -468,9 +587,7 @@ __global__ void __launch_bounds__(BT, 2) k_newton_block(BlockParams P) {
 #pragma unroll
           for (int k = 0; k < 3; ++k) {
             c.d(D_A + k, j) = st[(nzf + 3 * row + k) * n];
-            const double v = nb[(3 * id + k) * n];
-            c.d(D_N + k, j) = v;
-            c.f(F_N + k, j) = narrow_rn(v);
+            c.d(D_N + k, j) = nb[(3 * id + k) * n];
           }
         }
         for (int l = 0; l < 8; ++l) {
@@ -495,36 +612,37 @@ __global__ void __launch_bounds__(BT, 2) k_newton_block(BlockParams P) {
         if (act && lev == l) {
           double e[6], eL[6], eR[6];
           float de[6], dL[6], dR[6];
-#pragma unroll
-          for (int I = 0; I < 6; ++I) { e[I] = sh_e[I][pos]; de[I] = sd[I][pos]; }
-          down<CMP, LS, false>(t, c, s - 1, 7, a_in, a_out, apply, step, e, de, eL, eR, dL, dR);
-#pragma unroll
-          for (int I = 0; I < 6; ++I) {
-            sh_e[I][pos] = eL[I]; sh_e[I][pos + half] = eR[I];
-            sd[I][pos] = dL[I]; sd[I][pos + half] = dR[I];
-          }
+          get6(sh_e, pos, e);
+          get6(sd, pos, de);
+          down_a<CMP, LS>(t, c, s - 1, 7, a_in, a_out, apply, step, e, de, eL, eR, dL, dR);
+          put6(sh_e, pos, eL); put6(sh_e, pos + half, eR);
+          put6(sd, pos, dL); put6(sd, pos + half, dR);
         }
         __syncthreads();
       }
       double r2 = 0.0;
       if (act && !dead) {
-        double e[6], eL[6], eR[6], fL[6], fR[6], sq[6], sh[6], sb[6];
-        float de[6], dL[6], dR[6], dfL[6], dfR[6];
+        double e[6], eL[6], eR[6], sb[6];
+        float de[6], dL[6], dR[6];
+        get6(sh_e, tid, e);
+        get6(sd, tid, de);
+        down_a<CMP, LS>(t, c, heap(0), 0, a_in, a_out, apply, step, e, de, eL, eR, dL, dR);
+        put6(sh_e, tid, eR);
+        put6(sd, tid, dR);
 #pragma unroll
-        for (int I = 0; I < 6; ++I) { e[I] = sh_e[I][tid]; de[I] = sd[I][tid]; }
-        down<CMP, LS, false>(t, c, heap(0), 0, a_in, a_out, apply, step, e, de, eL, eR, dL, dR);
+        for (int I = 0; I < 6; ++I) { e[I] = eL[I]; de[I] = dL[I]; }
 #pragma unroll 1
         for (int q = 0; q < 4; ++q) {
+          const int mid = 1 + (q >> 1);
           if (!(q & 1)) {
+            down_a<CMP, LS>(t, c, heap(mid), mid, a_in, a_out, apply, step, e, de, eL, eR, dL, dR);
+            put6(sh_s, tid, eR);
+            put6(sh_x, tid, dR);
 #pragma unroll
-            for (int I = 0; I < 6; ++I) { e[I] = q ? eR[I] : eL[I]; de[I] = q ? dR[I] : dL[I]; }
-            down<CMP, LS, false>(t, c, heap(1 + (q >> 1)), 1 + (q >> 1), a_in, a_out, apply, step, e, de, fL, fR,
-                                 dfL, dfR);
+            for (int I = 0; I < 6; ++I) { e[I] = eL[I]; de[I] = dL[I]; }
           }
-          double gL[6], gR[6], z[6], s0[6], s1[6];
-#pragma unroll
-          for (int I = 0; I < 6; ++I) { e[I] = q & 1 ? fR[I] : fL[I]; de[I] = q & 1 ? dfR[I] : dfL[I]; }
-          down<CMP, LS, false>(t, c, heap(3 + q), 3 + q, a_in, a_out, apply, step, e, de, gL, gR, nullptr, nullptr);
+          down_a<CMP, LS>(t, c, heap(3 + q), 3 + q, a_in, a_out, apply, step, e, de, eL, eR, nullptr, nullptr);
+          double z[6], s0[6], s1[6];
 #pragma unroll
           for (int side = 0; side < 2; ++side) {
             const int ls = both ? 2 * q + side : q;
@@ -532,31 +650,40 @@ __global__ void __launch_bounds__(BT, 2) k_newton_block(BlockParams P) {
 #pragma unroll
             for (int k = 0; k < 6; ++k) z[k] = el ? 0.0 : c.z[(6 * ls + k) * BT];
             LeafTan<double> D;
-            leaf_iso<double, double>(t.ph[side], side ? gR : gL, z, side ? s1 : s0, &D, nullptr, nullptr);
+            leaf_iso<double, double>(t.ph[side], side ? eR : eL, z, side ? s1 : s0, &D, nullptr, nullptr);
             if (!el) {
-              c.tan[(8 * ls) * BT] = D.mu; c.tan[(8 * ls + 1) * BT] = D.c;
-              c.tanf[(8 * ls) * BT] = narrow_rn(D.mu); c.tanf[(8 * ls + 1) * BT] = narrow_rn(D.c);
+              float* T = c.tan + 16 * ls * BT;
+              pair v = split(D.mu);
+              T[0] = v.h; T[8 * BT] = v.l;
+              v = split(D.c);
+              T[BT] = v.h; T[9 * BT] = v.l;
 #pragma unroll
               for (int k = 0; k < 6; ++k) {
-                c.tan[(8 * ls + 2 + k) * BT] = D.m[k];
-                c.tanf[(8 * ls + 2 + k) * BT] = narrow_rn(D.m[k]);
+                v = split(D.m[k]);
+                T[(2 + k) * BT] = v.h; T[(10 + k) * BT] = v.l;
               }
             }
           }
           up_a<CMP>(t, c, heap(3 + q), 3 + q, s0, s1, sb, r2);
-          if (q & 1) {
-            double o[6];
-            up_a<CMP>(t, c, heap(1 + (q >> 1)), 1 + (q >> 1), sq, sb, o, r2);
-#pragma unroll
-            for (int I = 0; I < 6; ++I) { if (q == 1) sh[I] = o[I]; else sb[I] = o[I]; }
+          if (!(q & 1)) {
+            get6(sh_s, tid, e);
+            get6(sh_x, tid, de);
+            put6(sh_s, tid, sb);
           } else {
-#pragma unroll
-            for (int I = 0; I < 6; ++I) sq[I] = sb[I];
+            get6(sh_s, tid, s0);
+            up_a<CMP>(t, c, heap(mid), mid, s0, sb, s1, r2);
+            if (q == 1) {
+              get6(sh_e, tid, e);
+              get6(sd, tid, de);
+              put6(sh_e, tid, s1);
+            }
+          }
+          if (q == 3) {
+            get6(sh_e, tid, s0);
+            up_a<CMP>(t, c, heap(0), 0, s0, s1, sb, r2);
+            put6(sh_e, tid, sb);
           }
         }
-        up_a<CMP>(t, c, heap(0), 0, sh, sb, e, r2);
-#pragma unroll
-        for (int I = 0; I < 6; ++I) sh_e[I][tid] = e[I];
       } else if (act) {
 #pragma unroll
         for (int I = 0; I < 6; ++I) sh_e[I][tid] = 0.0;
@@ -565,11 +692,10 @@ __global__ void __launch_bounds__(BT, 2) k_newton_block(BlockParams P) {
       for (int l = Kt - 1; l >= 0; --l) {
         if (act && lev == l) {
           double sL[6], sR[6], sb[6];
-#pragma unroll
-          for (int I = 0; I < 6; ++I) { sL[I] = sh_e[I][pos]; sR[I] = sh_e[I][pos + half]; }
+          get6(sh_e, pos, sL);
+          get6(sh_e, pos + half, sR);
           up_a<CMP>(t, c, s - 1, 7, sL, sR, sb, r2);
-#pragma unroll
-          for (int I = 0; I < 6; ++I) sh_e[I][pos] = sb[I];
+          put6(sh_e, pos, sb);
         }
         __syncthreads();
       }
@@ -633,27 +759,25 @@ __global__ void __launch_bounds__(BT, 2) k_newton_block(BlockParams P) {
       }
       // ---- S: FP32 condensation up
       if (cont && !dead) {
-        Sub32 res, pq, ph;
+        Sub32 res, sib, o;
 #pragma unroll 1
         for (int q = 0; q < 4; ++q) {
+          const int mid = 1 + (q >> 1);
           LeafTan<float> DL, DR;
-          leaf_tan32(t.ph[0], c.tanf + (both ? 16 * q : 8 * q) * BT, DL);
-          leaf_tan32(t.ph[1], c.tanf + (both ? 16 * q + 8 : 8 * q) * BT, DR);
+          leaf_tan32(t.ph[0], c.tan + 16 * (both ? 2 * q : q) * BT, DL);
+          leaf_tan32(t.ph[1], c.tan + 16 * (both ? 2 * q + 1 : q) * BT, DR);
           condense32_bottom<CMP>(t, c, heap(3 + q), 3 + q, DL, DR, t.ph[0].kind == 0, t.ph[1].kind == 0, res);
-          if (q & 1) {
-            Sub32 o;
-            condense32<CMP>(t, c, heap(1 + (q >> 1)), 1 + (q >> 1), pq, res, o);
-            if (q == 1) ph = o; else res = o;
+          if (!(q & 1)) {
+            put27(M.s, tid, res);
           } else {
-            pq = res;
+            get27(M.s, tid, sib);
+            condense32<CMP>(t, c, heap(mid), mid, sib, res, o);
+            if (q == 1) put27(sh_c, tid, o);
           }
         }
-        Sub32 o;
-        condense32<CMP>(t, c, heap(0), 0, ph, res, o);
-#pragma unroll
-        for (int I = 0; I < 6; ++I) sh_c[I][tid] = o.ds[I];
-#pragma unroll
-        for (int k = 0; k < 21; ++k) sh_c[6 + k][tid] = o.C[k];
+        get27(sh_c, tid, sib);
+        condense32<CMP>(t, c, heap(0), 0, sib, o, res);
+        put27(sh_c, tid, res);
       } else if (cont) {
 #pragma unroll
         for (int k = 0; k < 27; ++k) sh_c[k][tid] = 0.f;
@@ -662,93 +786,94 @@ __global__ void __launch_bounds__(BT, 2) k_newton_block(BlockParams P) {
       for (int l = Kt - 1; l >= 0; --l) {
         if (cont && lev == l) {
           Sub32 L, R, o;
-#pragma unroll
-          for (int I = 0; I < 6; ++I) { L.ds[I] = sh_c[I][pos]; R.ds[I] = sh_c[I][pos + half]; }
-#pragma unroll
-          for (int k = 0; k < 21; ++k) { L.C[k] = sh_c[6 + k][pos]; R.C[k] = sh_c[6 + k][pos + half]; }
+          get27(sh_c, pos, L);
+          get27(sh_c, pos + half, R);
           condense32<CMP>(t, c, s - 1, 7, L, R, o);
-#pragma unroll
-          for (int I = 0; I < 6; ++I) sh_c[I][pos] = o.ds[I];
-#pragma unroll
-          for (int k = 0; k < 21; ++k) sh_c[6 + k][pos] = o.C[k];
+          put27(sh_c, pos, o);
         }
         __syncthreads();
       }
-      // ---- B: da1 down, J da1 up (FP64), second FP32 solve up
+      // ---- B: da1 down, J da1 up (pairs), second FP32 solve up
       if (cont && s == 0) {
 #pragma unroll
-        for (int I = 0; I < 6; ++I) { sh_e[I][p] = 0.0; sd[I][p] = 0.f; }
+        for (int I = 0; I < 12; ++I) sh_p[I][p] = 0.f;
       }
       __syncthreads();
       for (int l = 0; l < Kt; ++l) {
         if (cont && lev == l) {
-          double e[6], eL[6], eR[6];
-          float de[6], dL[6], dR[6];
-#pragma unroll
-          for (int I = 0; I < 6; ++I) { e[I] = sh_e[I][pos]; de[I] = sd[I][pos]; }
-          down<CMP, LS, true>(t, c, s - 1, 7, 0, 0, true, 1.0, e, de, eL, eR, dL, dR);
-#pragma unroll
-          for (int I = 0; I < 6; ++I) {
-            sh_e[I][pos] = eL[I]; sh_e[I][pos + half] = eR[I];
-            sd[I][pos] = dL[I]; sd[I][pos + half] = dR[I];
-          }
+          pair e[6], eL[6], eR[6];
+          get6(sh_p, pos, e);
+          down_b<CMP>(t, c, s - 1, 7, e, eL, eR);
+          put6(sh_p, pos, eL); put6(sh_p, pos + half, eR);
         }
         __syncthreads();
       }
       float q2 = 0.f;
       if (cont && !dead) {
-        double e[6], eL[6], eR[6], fL[6], fR[6], tq[6], th[6], tb[6];
-        float de[6], dL[6], dR[6], dfL[6], dfR[6], xq[6], xh[6], xb[6];
+        pair e[6], eL[6], eR[6], t0[6], t1[6];
+        float x0[6], x1[6];
+        get6(sh_p, tid, e);
+        down_b<CMP>(t, c, heap(0), 0, e, eL, eR);
+        put6(sh_p, tid, eR);
 #pragma unroll
-        for (int I = 0; I < 6; ++I) { e[I] = sh_e[I][tid]; de[I] = sd[I][tid]; }
-        down<CMP, LS, true>(t, c, heap(0), 0, 0, 0, true, 1.0, e, de, eL, eR, dL, dR);
+        for (int I = 0; I < 6; ++I) e[I] = eL[I];
 #pragma unroll 1
         for (int q = 0; q < 4; ++q) {
+          const int mid = 1 + (q >> 1);
           if (!(q & 1)) {
+            down_b<CMP>(t, c, heap(mid), mid, e, eL, eR);
+            put6(M.s, tid, eR);
 #pragma unroll
-            for (int I = 0; I < 6; ++I) { e[I] = q ? eR[I] : eL[I]; de[I] = q ? dR[I] : dL[I]; }
-            down<CMP, LS, true>(t, c, heap(1 + (q >> 1)), 1 + (q >> 1), 0, 0, true, 1.0, e, de, fL, fR, dfL, dfR);
+            for (int I = 0; I < 6; ++I) e[I] = eL[I];
           }
-          double gL[6], gR[6], t0[6], t1[6];
-#pragma unroll
-          for (int I = 0; I < 6; ++I) { e[I] = q & 1 ? fR[I] : fL[I]; de[I] = q & 1 ? dfR[I] : dfL[I]; }
-          down<CMP, LS, true>(t, c, heap(3 + q), 3 + q, 0, 0, true, 1.0, e, de, gL, gR, nullptr, nullptr);
-          leaf_apply(t.ph[0], c.tan + (both ? 16 * q : 8 * q) * BT, gL, t0);
-          leaf_apply(t.ph[1], c.tan + (both ? 16 * q + 8 : 8 * q) * BT, gR, t1);
-          up_b<CMP, true>(t, c, heap(3 + q), 3 + q, t0, t1, nullptr, nullptr, tb, xb, q2);
-          if (q & 1) {
-            double o[6];
-            float x[6];
-            up_b<CMP, false>(t, c, heap(1 + (q >> 1)), 1 + (q >> 1), tq, tb, xq, xb, o, x, q2);
-#pragma unroll
-            for (int I = 0; I < 6; ++I) {
-              if (q == 1) { th[I] = o[I]; xh[I] = x[I]; } else { tb[I] = o[I]; xb[I] = x[I]; }
-            }
+          down_b<CMP>(t, c, heap(3 + q), 3 + q, e, eL, eR);
+          leaf_apply(t.ph[0], c.tan + 16 * (both ? 2 * q : q) * BT, eL, t0);
+          leaf_apply(t.ph[1], c.tan + 16 * (both ? 2 * q + 1 : q) * BT, eR, t1);
+          up_b<CMP, true>(t, c, heap(3 + q), 3 + q, t0, t1, nullptr, nullptr, eL, x1, q2);
+          if (!(q & 1)) {
+            get6(M.s, tid, e);
+            put6(M.s, tid, eL);
+            put6(sh_x, tid, x1);
           } else {
+            get6(M.s, tid, t0);
+            get6(sh_x, tid, x0);
+            float y[6];
+            up_b<CMP, false>(t, c, heap(mid), mid, t0, eL, x0, x1, t1, y, q2);
 #pragma unroll
-            for (int I = 0; I < 6; ++I) { tq[I] = tb[I]; xq[I] = xb[I]; }
+            for (int I = 0; I < 6; ++I) x1[I] = y[I];
+            if (q == 1) {
+              get6(sh_p, tid, e);
+              put6(sh_p, tid, t1);
+              put6(sd, tid, x1);
+            }
+          }
+          if (q == 3) {
+            get6(sh_p, tid, t0);
+            get6(sd, tid, x0);
+            float y[6];
+            up_b<CMP, false>(t, c, heap(0), 0, t0, t1, x0, x1, eL, y, q2);
+            put6(sh_p, tid, eL);
+            put6(sd, tid, y);
           }
         }
-        up_b<CMP, false>(t, c, heap(0), 0, th, tb, xh, xb, e, de, q2);
-#pragma unroll
-        for (int I = 0; I < 6; ++I) { sh_e[I][tid] = e[I]; sd[I][tid] = de[I]; }
       } else if (cont) {
 #pragma unroll
-        for (int I = 0; I < 6; ++I) { sh_e[I][tid] = 0.0; sd[I][tid] = 0.f; }
+        for (int I = 0; I < 12; ++I) sh_p[I][tid] = 0.f;
+#pragma unroll
+        for (int I = 0; I < 6; ++I) sd[I][tid] = 0.f;
       }
       __syncthreads();
       for (int l = Kt - 1; l >= 0; --l) {
         if (cont && lev == l) {
-          double tL[6], tR[6], tb[6];
+          pair tL[6], tR[6], tb[6];
           float xL[6], xR[6], xb[6];
-#pragma unroll
-          for (int I = 0; I < 6; ++I) {
-            tL[I] = sh_e[I][pos]; tR[I] = sh_e[I][pos + half];
-            xL[I] = sd[I][pos]; xR[I] = sd[I][pos + half];
-          }
+          get6(sh_p, pos, tL);
+          get6(sh_p, pos + half, tR);
+          get6(sd, pos, xL);
+          get6(sd, pos + half, xR);
           up_b<CMP, false>(t, c, s - 1, 7, tL, tR, xL, xR, tb, xb, q2);
-#pragma unroll
-          for (int I = 0; I < 6; ++I) { sh_e[I][pos] = tb[I]; sd[I][pos] = xb[I]; }
+          put6(sh_p, pos, tb);
+          put6(sd, pos, xb);
         }
         __syncthreads();
       }
@@ -778,15 +903,19 @@ __global__ void __launch_bounds__(BT, 2) k_newton_block(BlockParams P) {
 }
 
 template <bool LS, bool CMP>
-static void launch(const BlockParams& P, unsigned grid, cudaStream_t s) {
-  k_newton_block<LS, CMP><<<grid, BT, sizeof(double) * 3 * BT, s>>>(P);
+static cudaError_t launch(const BlockParams& P, unsigned grid, cudaStream_t s) {
+  const cudaError_t e = cudaFuncSetAttribute(k_newton_block<LS, CMP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)sizeof(BlockShared));
+  if (e != cudaSuccess) return e;
+  k_newton_block<LS, CMP><<<grid, BT, sizeof(BlockShared), s>>>(P);
+  return cudaSuccess;
 }
 
-void launch_block(const BlockParams& P, bool ls, bool cmp, unsigned grid, cudaStream_t s) {
-  if (ls && cmp) launch<true, true>(P, grid, s);
-  else if (ls) launch<true, false>(P, grid, s);
-  else if (cmp) launch<false, true>(P, grid, s);
-  else launch<false, false>(P, grid, s);
+cudaError_t launch_block(const BlockParams& P, bool ls, bool cmp, unsigned grid, cudaStream_t s) {
+  if (ls && cmp) return launch<true, true>(P, grid, s);
+  if (ls) return launch<true, false>(P, grid, s);
+  if (cmp) return launch<false, true>(P, grid, s);
+  return launch<false, false>(P, grid, s);
 }
 
 }  // namespace dmn

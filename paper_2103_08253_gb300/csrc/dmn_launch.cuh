@@ -109,10 +109,11 @@ struct BlockParams {
   int max_iter;
   unsigned long long* passes;
 };
-// per thread, for 8 laminates: jumps (two buffers), normals, residuals (FP64: 12 fields), normals, H, Kn^-1, g,
-// step (FP32: 33 fields); per leaf its state and tangent (FP64: 14) and the tangent in FP32 (8)
-__host__ __device__ inline size_t block_scratch_bytes(int leaf_slots) {
-  return (size_t)BLOCK_THREADS * (sizeof(double) * (8 * 12 + 14 * leaf_slots) + sizeof(float) * (8 * 33 + 8 * leaf_slots));
+// per thread, for 8 laminates: jumps (two buffers with the line search) and normals (FP64), H, Kn^-1, g, step
+// and residual (FP32: 36 fields); per leaf its state (FP64: 6) and tangent (FP32: 16)
+__host__ __device__ inline size_t block_scratch_bytes(int leaf_slots, bool line_search) {
+  return (size_t)BLOCK_THREADS * (sizeof(double) * (8 * (line_search ? 9 : 6) + 6 * leaf_slots) +
+                                  sizeof(float) * (8 * 36 + 16 * leaf_slots));
 }
 __device__ __forceinline__ void block_bad_tree(const BlockParams& P, int64_t pt) {
   const double qnan = __longlong_as_double(0x7ff8000000000000LL);
@@ -125,6 +126,6 @@ __device__ __forceinline__ void block_retry(const BlockParams& P, int64_t pt) {
   P.status[pt] = STATUS_RETRY;
   P.list[atomicAdd(P.counter + 29, 1ull)] = pt;
 }
-void launch_block(const BlockParams& P, bool ls, bool cmp, unsigned grid, cudaStream_t s);
+cudaError_t launch_block(const BlockParams& P, bool ls, bool cmp, unsigned grid, cudaStream_t s);
 
 }  // namespace dmn
