@@ -765,6 +765,7 @@ struct FinalParams {
   const int32_t* status;
   const double* nbuf;
   const unsigned long long* n_list = nullptr;  // the points are perm[0 .. *n_list) instead of all n
+  int states_only = 0;     // stress and tangent are done (k_sweep_block)
 };
 
 // Without the sweep a point may be split over gridDim.y = 2^s threads (final_split), each of which takes
@@ -792,8 +793,8 @@ __global__ void __launch_bounds__(128) k_final(FinalParams P) {
   A.a_out = A.a;
   A.paper = true;
   A.z = P.state_in + pt; A.zs = (size_t)P.n;
-  if (part > 0) {
-    // another thread's
+  if (part > 0 || P.states_only) {
+    // another thread's or kernel's
   } else if (st == DMN_STATUS_NONFINITE) {
     const double qnan = __longlong_as_double(0x7ff8000000000000LL);
     for (int I = 0; I < 6; ++I) P.stress[6 * pt + I] = qnan;
@@ -1260,13 +1261,15 @@ int warp_lanes_for(const dmn_handle* h, int64_t n) {
   return h->opt.precision == DMN_PREC_F64 ? 8 : 16;
 }
 
-// The CTA organisation (csrc/dmn_block.cu) runs the FP64 form's Newton iteration from the paper's start, for
-// trees of depth 3 or more (its subtrees), whatever the call's size.
-bool block_on(const dmn_handle* h) {
-  if (h->opt.precision != DMN_PREC_F64 || h->opt.predictor || first_stage_on(h->opt)) return false;
+// The CTA organisation (csrc/dmn_block.cu) takes trees of depth 3 or more (its subtrees), whatever the call's
+// size: the FP64 form's Newton iteration from the paper's start, and every FP64 sweep.
+bool block_trees(const dmn_handle* h) {
   for (const Tree& t : h->trees)
     if (t.K < 3 || t.N < 1) return false;
   return true;
+}
+bool block_on(const dmn_handle* h) {
+  return h->opt.precision == DMN_PREC_F64 && !h->opt.predictor && !first_stage_on(h->opt) && block_trees(h);
 }
 int block_leaf_slots(const dmn_handle* h) {
   for (const Tree& t : h->trees)
@@ -1290,9 +1293,8 @@ cudaError_t alloc_ws(const dmn_handle* h, WorkSet& w) {
   if (e == cudaSuccess && warp_possible(h)) {
     // one slot per group of the smallest size the handle may use
     w.nwarps_w = (int64_t)h->n_sm * WARP_CTAS_PER_SM * 128 / (h->opt.warp_lanes ? h->opt.warp_lanes : WARP_MIN_LANES);
-    // FP64 slots where an FP64 pass runs in them (the FP64 form's Newton, the mixed form's final sweep)
-    const size_t per = h->opt.precision == DMN_PREC_MIXED_F32_TANGENT ? warp_slot_doubles<float>(h->N_max)
-                                                                     : warp_slot_doubles<double>(h->N_max);
+    const size_t per = h->opt.precision != DMN_PREC_F64 ? warp_slot_doubles<float>(h->N_max)
+                                                        : warp_slot_doubles<double>(h->N_max);
     e = cudaMalloc(&w.scr_w, sizeof(double) * per * (size_t)w.nwarps_w);
   }
   return e;
@@ -1382,7 +1384,7 @@ int update_on(dmn_handle* h, WorkSet& w, int64_t n, int64_t n_call, const int32_
     ev = h->events[h->events_used++].data();
     cudaEventRecord(ev[0], s);
   }
-  // counters: [0] work, [1..9] points per tree, [10..18] cursors, [19] first stage, [20] warp sweep,
+  // counters: [0] work, [1..9] points per tree, [10..18] cursors, [19] first stage,
   // [21..29] the CTA organisation
   e = cudaMemsetAsync(w.counter, 0, sizeof(unsigned long long) * 32, s);
   if (e != cudaSuccess) return cuda_fail(h, e, "dmn_update: counter reset");
@@ -1406,7 +1408,8 @@ int update_on(dmn_handle* h, WorkSet& w, int64_t n, int64_t n_call, const int32_
   const bool warp = warp_on(h, n_call) && w.scr_w;
   const bool stage = first_stage_on(h->opt) && !warp;   // a small batch goes straight to the warp kernel
   const unsigned wgrid = (unsigned)(h->n_sm * WARP_CTAS_PER_SM);
-  const int lanes = warp ? warp_lanes_for(h, n_call) : 32;
+  const bool block = w.scr_b != nullptr;
+  const int lanes = warp && !block ? warp_lanes_for(h, n_call) : 32;
   unsigned long long* passes = h->profiling ? h->d_passes : nullptr;
   if (stage) {   // counter [19]: the first stage's work counter
     // its corrections count against max_iter: the FP64-residual iteration keeps at least one
@@ -1418,7 +1421,6 @@ int update_on(dmn_handle* h, WorkSet& w, int64_t n, int64_t n_call, const int32_
     else launch_stage<false>(SP, h->opt.stage_ctas_per_sm, sgrid, s);
   }
   if (ev) cudaEventRecord(ev[2], s);
-  const bool block = w.scr_b != nullptr;
   const dim3 gf(g1, final_split(n, h->n_sm));
   FinalParams FP{F, n, NM, tree_id, perm, Q, state_in, state_out, stress, tangent, status, w.nbuf};
   NewtonParams<double> DP{F, n, h->nslots, NM, tree_id, perm, state_in, state_out, stress, tangent, iters, status,
@@ -1437,17 +1439,11 @@ int update_on(dmn_handle* h, WorkSet& w, int64_t n, int64_t n_call, const int32_
     else if (h->cmp) k_final<false, true><<<gf, 128, 0, s>>>(P);
     else k_final<false, false><<<gf, 128, 0, s>>>(P);
   };
-  // the FP64 sweep for stress and tangent: in the warp organisation (counter [20]; k_final then rotates) or
-  // one thread per point.  Even at 216 points per SM.
-  auto sweep_pass = [&](bool in_warps) {
-    if (in_warps) {
-      NewtonParams<double> SP = DP;
-      SP.counter = w.counter + 20;
-      const int swl = h->opt.warp_lanes ? h->opt.warp_lanes : (n_call <= 16 * (int64_t)h->n_sm ? 32 : 8);
-      if (h->cmp) launch_sweep_warp<true>(SP, swl, wgrid, w.scr_w, s);
-      else launch_sweep_warp<false>(SP, swl, wgrid, w.scr_w, s);
-    }
-    final_pass(FP, !in_warps);
+  // the FP64 sweep for stress, tangent and, in the FP64 form, the leaf states
+  auto sweep_pass = [&](bool states) -> cudaError_t {
+    SweepParams P{F, n, NM, tree_id, perm, Q, state_in, state_out, stress, tangent, status, w.nbuf, w.counter};
+    const int64_t ctas = div_up(n, SWEEP_THREADS >> (h->K_max - 3)) + (int64_t)h->trees.size();
+    return launch_sweep_block(P, h->cmp, states, (unsigned)std::min<int64_t>(ctas, (int64_t)h->n_sm * SWEEP_CTAS_PER_SM), s);
   };
   if (block) {
     BlockParams P{F, n, NM, block_leaf_slots(h), tree_id, perm, state_in, state_out, stress, tangent, iters, status,
@@ -1468,15 +1464,22 @@ int update_on(dmn_handle* h, WorkSet& w, int64_t n, int64_t n_call, const int32_
   }
   if (ev) cudaEventRecord(ev[3], s);
   if (block) {
-    sweep_pass(w.scr_w && n_call <= 216 * (int64_t)h->n_sm);
-    // the points it left: the all-FP64 iteration from their start, in the organisation of the call's size
+    e = sweep_pass(true);
+    if (e != cudaSuccess) return cuda_fail(h, e, "dmn_update: launch");
+    // the points it left: the all-FP64 iteration from their start, in the organisation of the call's size (few
+    // points: a warp each)
     NewtonParams<double> P = DP;
     P.perm = FP.perm = w.list;
     P.n_list = FP.n_list = w.counter + 29;
     newton_f64(P);
     final_pass(FP, false);
+  } else if (sweep && block_trees(h)) {
+    e = sweep_pass(false);
+    if (e != cudaSuccess) return cuda_fail(h, e, "dmn_update: launch");
+    FP.states_only = 1;
+    final_pass(FP, false);
   } else if (sweep) {
-    sweep_pass(warp);
+    final_pass(FP, true);
   } else {
     final_pass(FP, false);
   }

@@ -13,8 +13,8 @@
 // sweep at the converged jumps, as in the mixed form.
 //
 // A point for which the FP32 solve does not contract (|R + J da1| > REFINE_MAX |R|: tangents near
-// singular, moduli outside the FP32 range), which is not finite, whose line search fails or which has not
-// converged within BLOCK_ITERS corrections is put on a list (status RETRY) and updated from its start by the
+// singular, moduli outside the FP32 range), which is not finite or which has not converged within BLOCK_ITERS
+// corrections is put on a list (status RETRY) and updated from its start by the
 // all-FP64 kernels, so that every call keeps their results and statuses.
 //
 // Organisation.  A CTA of 256 threads holds 256 / S points, S = 2^(K-3) threads per point: thread (s, p)
@@ -462,7 +462,7 @@ __device__ __forceinline__ void leaf_apply(const PhaseDev& ph, const float* s, c
 }  // namespace
 
 // flags of a slot
-enum { B_ACT = 1, B_NEW = 2, B_FIRST = 4, B_CONT = 8, B_CONV = 16, B_CUR = 32 };
+enum { B_ACT = 1, B_FIRST = 4, B_CONT = 8, B_CONV = 16, B_CUR = 32 };
 
 // Own-column accesses: a thread's vector of 6 in rows 0 .. 5 of a shared array, at column x.
 template <typename T>
@@ -507,10 +507,30 @@ struct BlockShared {
   long long pt[BT];
   int fl[BT];
   float st[BT];
+  int n_in, n_out;       // slots that take a point in / hand one out in this round
+  short in[BT], out[BT];
 };
 
+// Laminate h (0-based) of the full tree of depth Kt + 3 lies with subtree thread s as its laminate j.
+__device__ __forceinline__ void owner(int h, int Kt, int& s, int& j) {
+  const int h1 = h + 1, d = 31 - __clz(h1) - Kt, S = 1 << Kt;
+  if (d < 0) { s = h1; j = 7; }
+  else { s = (h1 >> d) - S; j = (1 << d) - 1 + (h1 & ((1 << d) - 1)); }
+}
+
+// The two CTAs of an SM alternate between the FP64 phase A and the FP32 phases S and B.  Started together
+// they run in step, both in A or both out of it, and the FP64 units idle half of the time; started half a
+// round apart they stay apart (100003 points: 35.7 ms always, against 35.8 to 43 ms).  The launch's second
+// half of the CTAs lands beside the first; the wait is bounded.
+__device__ __forceinline__ void stagger() {
+  constexpr long long HALF_ROUND = 150000;   // cycles
+  if (gridDim.x < 2 || 2 * blockIdx.x < gridDim.x) return;
+  const long long t0 = clock64();
+  for (int k = 0; k < 2000 && clock64() - t0 < HALF_ROUND; ++k) __nanosleep(100);
+}
+
 template <bool LS, bool CMP>
-__global__ void __launch_bounds__(BT, 2) k_newton_block(BlockParams P) {
+__global__ void __launch_bounds__(BT, BLOCK_CTAS_PER_SM) k_newton_block(BlockParams P) {
   extern __shared__ __align__(16) char dyn[];
   BlockShared& M = *reinterpret_cast<BlockShared*>(dyn);
   double (*const sh_e)[BT] = M.e;
@@ -525,9 +545,12 @@ __global__ void __launch_bounds__(BT, 2) k_newton_block(BlockParams P) {
   const int tid = threadIdx.x, lane = tid & 31;
   const size_t n = (size_t)P.n;
   Ctx c;
+  double *D0, *z0;
   {
     char* base = P.scratch + (size_t)blockIdx.x * block_scratch_bytes(P.leaf_slots, LS);
     double* D = (double*)base;
+    D0 = D;
+    z0 = D + (size_t)8 * (LS ? 9 : 6) * BT;
     c.D = D + tid;
     c.z = D + (size_t)8 * (LS ? 9 : 6) * BT + tid;
     float* F = (float*)(D + (size_t)(8 * (LS ? 9 : 6) + 6 * P.leaf_slots) * BT);
@@ -549,12 +572,15 @@ __global__ void __launch_bounds__(BT, 2) k_newton_block(BlockParams P) {
     auto heap = [&](int j) { return (j == 0 ? R1 : j < 3 ? 2 * R1 + j - 1 : j < 7 ? 4 * R1 + j - 3 : s) - 1; };
     // a subtree with nothing alive in it is skipped (its results are never used, only kept finite)
     const bool dead = CMP && __ldg(t.hdir + heap(0)) == 3;
+    if (tr == 0) stagger();
     // state of slot p, kept by thread p < nP
     long long pt = -1;
     int it = 0, halv = 0, np = 0;
     double rn_acc = 0.0;
     bool more = tid < nP;
     if (tid < nP) sh_fl[tid] = 0;
+    if (tid == 0) M.n_in = 0;
+    __syncthreads();
     for (;;) {
       if (tid < nP && more && !(sh_fl[tid] & B_ACT)) {
         for (;;) {
@@ -566,7 +592,8 @@ __global__ void __launch_bounds__(BT, 2) k_newton_block(BlockParams P) {
           if (tt == tr) {
             pt = x; it = 0; halv = 0; np = 0; rn_acc = 0.0;
             sh_pt[tid] = pt; sh_st[tid] = 1.f;
-            sh_fl[tid] = B_ACT | B_NEW | B_FIRST;
+            sh_fl[tid] = B_ACT | B_FIRST;
+            M.in[atomicAdd(&M.n_in, 1)] = (short)tid;
             break;
           }
           block_bad_tree(P, x);
@@ -576,28 +603,33 @@ __global__ void __launch_bounds__(BT, 2) k_newton_block(BlockParams P) {
       if (!__syncthreads_or(any)) break;
       int fl = sh_fl[p];
       const size_t mypt = (size_t)sh_pt[p];
-      if (fl & B_NEW) {
-        const double* st = P.state_in + mypt;
-        const double* nb = P.nbuf + mypt;
-        for (int j = s ? 7 : 6; j >= 0; --j) {
-          const int h = heap(j);
-          const int id = CMP ? __ldg(t.hcid + h) : h;
-          if (id < 0) continue;
+      // the CTA's threads load the new points together, a laminate and a leaf each: independent loads, where
+      // the slot's own S threads would wait for one after another (a quarter of a round; now a twentieth)
+      for (int i = tid; i < M.n_in << K; i += BT) {
+        const int x = M.in[i >> K], h = i & (t.L - 1);
+        const size_t q = (size_t)sh_pt[x];
+        const int id = h == t.L - 1 ? -1 : CMP ? __ldg(t.hcid + h) : h;
+        if (id >= 0) {
           const int row = CMP ? id : (1 << K) - 3 * (1 << (31 - __clz(h + 1))) + h + 1;
+          int os, oj;
+          owner(h, Kt, os, oj);
+          double* w = D0 + oj * BT + os * nP + x;
 #pragma unroll
           for (int k = 0; k < 3; ++k) {
-            c.d(D_A + k, j) = st[(nzf + 3 * row + k) * n];
-            c.d(D_N + k, j) = nb[(3 * id + k) * n];
+            w[8 * (D_A + k) * BT] = __ldg(P.state_in + (nzf + 3 * row + k) * n + q);
+            w[8 * (D_N + k) * BT] = __ldg(P.nbuf + (3 * id + k) * n + q);
           }
         }
-        for (int l = 0; l < 8; ++l) {
-          if (t.ph[l & 1].kind == 0) continue;
-          const int leaf = 8 * s + l, ls = both ? l : l >> 1;
+        const int leaf = h;   // as many leaves as laminates and one
+        if (t.ph[leaf & 1].kind != 0) {
           const int slot = CMP ? __ldg(t.lslot + leaf) : both ? leaf : leaf >> 1;
+          const int l = leaf & 7;
+          double* w = z0 + (6 * (both ? l : l >> 1)) * BT + (leaf >> 3) * nP + x;
 #pragma unroll
-          for (int k = 0; k < 6; ++k) c.z[(6 * ls + k) * BT] = slot >= 0 ? st[(6 * slot + k) * n] : 0.0;
+          for (int k = 0; k < 6; ++k) w[k * BT] = slot >= 0 ? __ldg(P.state_in + (6 * slot + k) * n + q) : 0.0;
         }
       }
+      if (tid == 0) M.n_out = 0;
       const bool act = fl & B_ACT, apply = act && !(fl & B_FIRST);
       const int a_in = LS && (fl & B_CUR) ? D_A2 : D_A, a_out = LS ? (a_in == D_A ? D_A2 : D_A) : D_A;
       const double step = LS ? (double)sh_st[p] : 1.0;
@@ -716,41 +748,47 @@ __global__ void __launch_bounds__(BT, 2) k_newton_block(BlockParams P) {
         int f = sh_fl[tid] & (B_ACT | B_FIRST | B_CUR);
         ++np;
         bool retry = false;
+        int st = -1;   // the point's status once it is done
         const bool ok = !LS || (f & B_FIRST) || rn < rn_acc;
         if (ok) {
           if (LS) { f ^= B_CUR; sh_st[tid] = 1.f; halv = 0; }
           rn_acc = rn;
           f &= ~B_FIRST;
           if (!isfinite(rn) || !isfinite(sn)) retry = true;
-          else if (rn <= P.tol * (double)t.N * sn) f |= B_CONV;
-          else if (it >= P.max_iter || it >= BLOCK_ITERS) retry = true;
+          else if (rn <= P.tol * (double)t.N * sn) st = DMN_STATUS_OK;
+          else if (it >= P.max_iter) st = DMN_STATUS_MAXITER;
+          else if (it >= BLOCK_ITERS) retry = true;
           else { ++it; f |= B_CONT; }
         } else if (++halv > 8) {
-          retry = true;
+          st = DMN_STATUS_LINESEARCH;   // no halving lowered the residual: the accepted iterate stands
+          ++it;
         } else {
           sh_st[tid] *= 0.5f;
         }
         if (retry) { block_retry(P, pt); f = 0; }
-        if (f & B_CONV) {
+        if (st >= 0) {
+          f |= B_CONV;
           P.iters[pt] = it;
-          P.status[pt] = DMN_STATUS_OK;
+          P.status[pt] = st;
           if (P.passes) atomicAdd(P.passes, (unsigned long long)np);
+          M.out[atomicAdd(&M.n_out, 1)] = (short)tid;
           f &= ~B_ACT;
         }
         sh_fl[tid] = f;
       }
       __syncthreads();
       fl = sh_fl[p];
-      if (fl & B_CONV) {   // the converged jumps, in the state's order
-        const int af = LS && (fl & B_CUR) ? D_A2 : D_A;
-        double* st = P.state_out + mypt;
-        for (int j = s ? 7 : 6; j >= 0; --j) {
-          const int h = heap(j);
-          const int row = CMP ? __ldg(t.hcid + h) : (1 << K) - 3 * (1 << (31 - __clz(h + 1))) + h + 1;
-          if (CMP && row < 0) continue;
+      if (tid == 0) M.n_in = 0;
+      for (int i = tid; i < M.n_out << K; i += BT) {   // the converged jumps, in the state's order
+        const int x = M.out[i >> K], h = i & (t.L - 1);
+        const int row = h == t.L - 1 ? -1 : CMP ? __ldg(t.hcid + h) : (1 << K) - 3 * (1 << (31 - __clz(h + 1))) + h + 1;
+        if (row < 0) continue;
+        int os, oj;
+        owner(h, Kt, os, oj);
+        const double* w = D0 + 8 * (LS && (sh_fl[x] & B_CUR) ? D_A2 : D_A) * BT + oj * BT + os * nP + x;
+        double* st = P.state_out + (nzf + 3 * row) * n + (size_t)sh_pt[x];
 #pragma unroll
-          for (int k = 0; k < 3; ++k) st[(nzf + 3 * row + k) * n] = c.d(af + k, j);
-        }
+        for (int k = 0; k < 3; ++k) st[k * n] = w[8 * k * BT];
       }
       const bool cont = fl & B_CONT;
       if (!__syncthreads_or(cont)) {
@@ -900,6 +938,381 @@ __global__ void __launch_bounds__(BT, 2) k_newton_block(BlockParams P) {
          i += (unsigned long long)gridDim.x * BT)
       block_bad_tree(P, P.perm[i]);
   }
+}
+
+// ---------------------------------------------------------------------------
+// The FP64 sweep at the converged jumps in the same organisation: stress, algorithmic tangent and leaf states
+// of every point (the FP64 form after k_newton_block, the mixed form after its Newton kernel).  One pass:
+// strains down, leaf laws (which give the FP64 form's new leaf states too), condensation up, rotation.  It
+// replaces one sweep per thread, whose last wave and per-thread stacks cost 20 % at 10^5 points, or 8 lanes per
+// point.  The FP64 pipe bounds it, so its algebra is the shortest form
+// found: tangents in Voigt components (C_IJ / (w_I w_J), w = sqrt 2 in the shear rows), in which N(n) has the
+// bare components of n; Kn as quadratic forms in n instead of N^T (C N); and, without a Newton step to store,
+// Kn = L D L^T and C -= c1 c2 (B L^-T) D^-1 (B L^-T)^T in place of the inverse and H.  88 k FP64 instructions
+// per point at depth 8 instead of 107 k.
+constexpr int ST = SWEEP_THREADS;
+
+struct Sub64 {
+  double sb[6], C[21];
+};
+
+// C -= c12 B Kn^-1 B^T for Kn symmetric positive definite
+__device__ __forceinline__ void downdate(double k00, double k01, double k02, double k11, double k12, double k22,
+                                         double B[6][3], double c12, double C[21]) {
+  const double i0 = 1.0 / k00, l10 = k01 * i0, l20 = k02 * i0;
+  const double d1 = k11 - l10 * k01, s12 = k12 - l10 * k02, s22 = k22 - l20 * k02;
+  const double t = s22 * d1 - s12 * s12, r = 1.0 / (d1 * t);   // t = d1 d2: one division for 1 / d1 and 1 / d2
+  const double i1 = r * t, i2 = d1 * (r * d1), l21 = s12 * i1;
+  const double w0 = -c12 * i0, w1 = -c12 * i1, w2 = -c12 * i2;
+#pragma unroll
+  for (int I = 0; I < 6; ++I) {
+    B[I][1] -= l10 * B[I][0];
+    B[I][2] -= l20 * B[I][0] + l21 * B[I][1];
+  }
+#pragma unroll
+  for (int I = 0; I < 6; ++I) {
+    const double z0 = w0 * B[I][0], z1 = w1 * B[I][1], z2 = w2 * B[I][2];
+#pragma unroll
+    for (int J = I; J < 6; ++J) {
+      double v = C[sidx(I, J)];
+      v += z0 * B[J][0];
+      v += z1 * B[J][1];
+      v += z2 * B[J][2];
+      C[sidx(I, J)] = v;
+    }
+  }
+}
+
+// laminate with normal n: L and R condensed into o (Voigt tangents)
+__device__ __forceinline__ void condense64(const double n[3], double c2, double c12, const Sub64& L, const Sub64& R,
+                                           Sub64& o) {
+#pragma unroll
+  for (int I = 0; I < 6; ++I) o.sb[I] = L.sb[I] + c2 * (R.sb[I] - L.sb[I]);
+  double dC[21], H[21], B[6][3];
+#pragma unroll
+  for (int k = 0; k < 21; ++k) { dC[k] = R.C[k] - L.C[k]; H[k] = R.C[k] - c2 * dC[k]; o.C[k] = L.C[k] + c2 * dC[k]; }
+  const double x = n[0], y = n[1], z = n[2], xx = x * x, yy = y * y, zz = z * z, xy = x * y, xz = x * z, yz = y * z;
+  const double xy2 = 2.0 * xy, xz2 = 2.0 * xz, yz2 = 2.0 * yz;
+#define C_(i, j) H[sidx(i, j)]
+  const double k00 = C_(0, 0) * xx + C_(5, 5) * yy + C_(4, 4) * zz + C_(0, 5) * xy2 + C_(0, 4) * xz2 + C_(4, 5) * yz2;
+  const double k11 = C_(5, 5) * xx + C_(1, 1) * yy + C_(3, 3) * zz + C_(1, 5) * xy2 + C_(3, 5) * xz2 + C_(1, 3) * yz2;
+  const double k22 = C_(4, 4) * xx + C_(3, 3) * yy + C_(2, 2) * zz + C_(3, 4) * xy2 + C_(2, 4) * xz2 + C_(2, 3) * yz2;
+  const double k01 = C_(0, 5) * xx + C_(1, 5) * yy + C_(3, 4) * zz + (C_(0, 1) + C_(5, 5)) * xy +
+                     (C_(0, 3) + C_(4, 5)) * xz + (C_(1, 4) + C_(3, 5)) * yz;
+  const double k02 = C_(0, 4) * xx + C_(3, 5) * yy + C_(2, 4) * zz + (C_(0, 3) + C_(4, 5)) * xy +
+                     (C_(0, 2) + C_(4, 4)) * xz + (C_(2, 5) + C_(3, 4)) * yz;
+  const double k12 = C_(4, 5) * xx + C_(1, 3) * yy + C_(2, 3) * zz + (C_(3, 5) + C_(1, 4)) * xy +
+                     (C_(2, 5) + C_(3, 4)) * xz + (C_(1, 2) + C_(3, 3)) * yz;
+#undef C_
+#pragma unroll
+  for (int I = 0; I < 6; ++I) {   // dC N: the columns of N are (x, 0, 0, 0, z, y), (0, y, 0, z, 0, x), (0, 0, z, y, x, 0)
+    B[I][0] = dC[sidx(I, 0)] * x + dC[sidx(I, 4)] * z + dC[sidx(I, 5)] * y;
+    B[I][1] = dC[sidx(I, 1)] * y + dC[sidx(I, 3)] * z + dC[sidx(I, 5)] * x;
+    B[I][2] = dC[sidx(I, 2)] * z + dC[sidx(I, 3)] * y + dC[sidx(I, 4)] * x;
+  }
+  downdate(k00, k01, k02, k11, k12, k22, B, c12, o.C);
+}
+
+// bottom laminate from its leaves' tangents lam 1(x)1 + 2 mu I - c m(x)m (condense_bottom in Voigt components);
+// el: the phase is elastic, c = 0.  c1 + c2 = 1; a passed-on side has fraction 1 and no normal (n = 0, c12 = 0).
+__device__ __forceinline__ void condense64_bottom(const double n[3], double c1, double c2, double c12,
+                                                  const double sL[6], const LeafTan<double>& L, bool elL,
+                                                  const double sR[6], const LeafTan<double>& R, bool elR, Sub64& o) {
+#pragma unroll
+  for (int I = 0; I < 6; ++I) o.sb[I] = sL[I] + c2 * (sR[I] - sL[I]);
+  const double lam = c1 * L.lam + c2 * R.lam, mu = c1 * L.mu + c2 * R.mu;
+#pragma unroll
+  for (int I = 0; I < 6; ++I)
+#pragma unroll
+    for (int J = I; J < 6; ++J) o.C[sidx(I, J)] = J < 3 ? (I == J ? lam + 2.0 * mu : lam) : (I == J ? mu : 0.0);
+  const double a = c2 * L.mu + c1 * R.mu, b = c2 * (L.lam + L.mu) + c1 * (R.lam + R.mu);
+  const double bx = b * n[0], by = b * n[1], bz = b * n[2];
+  double k00 = bx * n[0] + a, k01 = bx * n[1], k02 = bx * n[2], k11 = by * n[1] + a, k12 = by * n[2], k22 = bz * n[2] + a;
+  const double dlam = R.lam - L.lam, dmu = R.mu - L.mu, dld = dlam + 2.0 * dmu;
+  double B[6][3];
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    const double l = dlam * n[j], d = dmu * n[j];
+#pragma unroll
+    for (int I = 0; I < 3; ++I) B[I][j] = I == j ? dld * n[j] : l;
+    // shear rows 23, 13, 12: entry (row, column) is dmu times the other index's component
+    if (j == 0) { B[4][2] = d; B[5][1] = d; }
+    if (j == 1) { B[3][2] = d; B[5][0] = d; }
+    if (j == 2) { B[3][1] = d; B[4][0] = d; }
+  }
+  B[3][0] = 0.0; B[4][1] = 0.0; B[5][2] = 0.0;
+  auto leaf = [&](const LeafTan<double>& D, double frac, double other, double sign) {
+    const double m[6] = {D.m[0], D.m[1], D.m[2], RS2 * D.m[3], RS2 * D.m[4], RS2 * D.m[5]};
+    const double u[3] = {m[0] * n[0] + m[4] * n[2] + m[5] * n[1], m[1] * n[1] + m[3] * n[2] + m[5] * n[0],
+                         m[2] * n[2] + m[3] * n[1] + m[4] * n[0]};
+    const double w = -other * D.c, wx = w * u[0], wy = w * u[1], wz = w * u[2];
+    k00 += wx * u[0]; k01 += wx * u[1]; k02 += wx * u[2]; k11 += wy * u[1]; k12 += wy * u[2]; k22 += wz * u[2];
+#pragma unroll
+    for (int I = 0; I < 6; ++I) {
+      const double cm = D.c * m[I], h = -frac * cm, s = sign * cm;
+#pragma unroll
+      for (int j = 0; j < 3; ++j) B[I][j] += s * u[j];
+#pragma unroll
+      for (int J = I; J < 6; ++J) o.C[sidx(I, J)] += h * m[J];
+    }
+  };
+  if (!elL) leaf(L, c1, c2, 1.0);
+  if (!elR) leaf(R, c2, c1, -1.0);
+  downdate(k00, k01, k02, k11, k12, k22, B, c12, o.C);
+}
+
+struct SweepShared {
+  double e[6][ST], f[6][ST];       // strains handed down; set aside by the bottom walk
+  double c[27][ST], s[27][ST];     // results handed up; set aside
+};
+__device__ __forceinline__ void put27(double (*m)[ST], int x, const Sub64& v) {
+#pragma unroll
+  for (int I = 0; I < 6; ++I) m[I][x] = v.sb[I];
+#pragma unroll
+  for (int k = 0; k < 21; ++k) m[6 + k][x] = v.C[k];
+}
+__device__ __forceinline__ void get27(double (*m)[ST], int x, Sub64& v) {
+#pragma unroll
+  for (int I = 0; I < 6; ++I) v.sb[I] = m[I][x];
+#pragma unroll
+  for (int k = 0; k < 21; ++k) v.C[k] = m[6 + k][x];
+}
+__device__ __forceinline__ void sput6(double (*m)[ST], int x, const double v[6]) {
+#pragma unroll
+  for (int I = 0; I < 6; ++I) m[I][x] = v[I];
+}
+__device__ __forceinline__ void sget6(double (*m)[ST], int x, double v[6]) {
+#pragma unroll
+  for (int I = 0; I < 6; ++I) v[I] = m[I][x];
+}
+
+// STATES: also the leaf states.  The mixed form leaves them to k_final, as its FP32-tangent variant does: the two
+// return the same state bit for bit.
+template <bool CMP, bool STATES>
+__global__ void __launch_bounds__(ST, SWEEP_CTAS_PER_SM) k_sweep_block(SweepParams P) {
+  extern __shared__ __align__(16) char dyn[];
+  SweepShared& M = *reinterpret_cast<SweepShared*>(dyn);
+  const int tid = threadIdx.x;
+  const size_t n = (size_t)P.n;
+  const double qnan = __longlong_as_double(0x7ff8000000000000LL);
+  for (unsigned long long g = blockIdx.x;; g += gridDim.x) {
+    // group g: nP consecutive points of one tree
+    int tr = 0;
+    unsigned long long b = g, begin = 0, end = 0;
+    for (; tr < P.F.n; ++tr) {
+      const int w = ST >> (P.F.t[tr].K - 3);
+      end = P.perm ? P.counter[10 + tr] : (tr ? 0ull : (unsigned long long)P.n);
+      begin = P.perm ? end - P.counter[1 + tr] : 0ull;
+      const unsigned long long groups = (end - begin + w - 1) / w;
+      if (b < groups) break;
+      b -= groups;
+    }
+    if (tr == P.F.n) return;
+    const TreeDev& t = P.F.t[tr];
+    const int K = t.K, Kt = K - 3, S = 1 << Kt, nP = ST >> Kt, p = tid & (nP - 1), s = tid / nP;
+    const int nzf = 6 * t.nz, R1 = S + s, lev = s ? 31 - __clz(s) : -1;
+    const int pos = s ? (((s << (Kt - lev)) - S) * nP + p) : p, half = s ? (S >> (lev + 1)) * nP : 0;
+    const bool both = t.z_both;
+    auto heap = [&](int j) { return (j == 0 ? R1 : j < 3 ? 2 * R1 + j - 1 : 4 * R1 + j - 3) - 1; };
+    const bool dead = CMP && __ldg(t.hdir + heap(0)) == 3;
+    const unsigned long long i = begin + b * nP + p;
+    int64_t pt = 0;
+    int st = STATUS_RETRY;
+    if (i < end) {
+      int tt;
+      point_of(P.perm, P.tid, P.F.n, (int64_t)i, pt, tt);
+      if (tt == tr) st = P.status[pt];
+    }
+    const bool act = st != STATUS_RETRY && st != DMN_STATUS_NONFINITE;
+    const double* zin = P.state_in + pt;
+    double* zout = P.state_out + pt;
+    auto normal = [&](const Lam<CMP>& q, double v[3]) {
+#pragma unroll
+      for (int k = 0; k < 3; ++k) v[k] = P.nbuf[(3 * q.id + k) * n + pt];
+    };
+    auto down = [&](int h, const double e[6], double eL[6], double eR[6]) {
+      const Lam<CMP> q(t, h);
+      if (CMP && q.mode) {
+#pragma unroll
+        for (int I = 0; I < 6; ++I) eL[I] = eR[I] = e[I];
+        return;
+      }
+      const int row = CMP ? q.id : (1 << K) - 3 * (1 << (31 - __clz(h + 1))) + h + 1;
+      double v[3], a[3], Na[6];
+      normal(q, v);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) a[k] = zout[(nzf + 3 * row + k) * n];
+      const double vr[3] = {v[0] * RS2, v[1] * RS2, v[2] * RS2};
+      N_apply<double>(v, vr, a, Na);
+#pragma unroll
+      for (int I = 0; I < 6; ++I) { eL[I] = e[I] - q.c2 * Na[I]; eR[I] = e[I] + q.c1 * Na[I]; }
+    };
+    auto up = [&](int h, const Sub64& L, const Sub64& R, Sub64& o) {
+      const Lam<CMP> q(t, h);
+      if (CMP && q.mode) {
+        if (q.mode == 2) o = R; else o = L;
+        return;
+      }
+      double v[3];
+      normal(q, v);
+      condense64(v, q.c2, q.c1 * q.c2, L, R, o);
+    };
+    if (STATES && st == DMN_STATUS_NONFINITE) {   // NaN outputs and leaf states; the Newton kernel wrote the jumps
+      for (int l = 0; l < 8; ++l) {
+        const int leaf = 8 * s + l;
+        const int slot = t.ph[l & 1].kind == 0 ? -1 : CMP ? __ldg(t.lslot + leaf) : both ? leaf : leaf >> 1;
+        if (slot < 0) continue;
+        for (int k = 0; k < 6; ++k) zout[(6 * slot + k) * n] = qnan;
+      }
+    }
+    if (act && s == 0) {
+#pragma unroll
+      for (int I = 0; I < 6; ++I) M.e[I][p] = P.nbuf[(3 * P.N_max + I) * n + pt];
+    }
+    __syncthreads();
+    for (int l = 0; l < Kt; ++l) {
+      if (act && lev == l) {
+        double e[6], eL[6], eR[6];
+        sget6(M.e, pos, e);
+        down(s - 1, e, eL, eR);
+        sput6(M.e, pos, eL);
+        sput6(M.e, pos + half, eR);
+      }
+      __syncthreads();
+    }
+    if (act && !dead) {
+      double e[6], eL[6], eR[6];
+      Sub64 res, sib, o;
+      sget6(M.e, tid, e);
+      down(heap(0), e, eL, eR);
+      sput6(M.e, tid, eR);
+#pragma unroll
+      for (int I = 0; I < 6; ++I) e[I] = eL[I];
+#pragma unroll 1
+      for (int q = 0; q < 4; ++q) {
+        const int mid = 1 + (q >> 1);
+        if (!(q & 1)) {
+          down(heap(mid), e, eL, eR);
+          sput6(M.f, tid, eR);
+#pragma unroll
+          for (int I = 0; I < 6; ++I) e[I] = eL[I];
+        }
+        const int h = heap(3 + q);
+        down(h, e, eL, eR);
+        LeafTan<double> D[2];
+        double s0[6], s1[6];
+#pragma unroll
+        for (int side = 0; side < 2; ++side) {
+          const int leaf = 8 * s + 2 * q + side;
+          const int slot = t.ph[side].kind == 0 ? -1 : CMP ? __ldg(t.lslot + leaf) : both ? leaf : leaf >> 1;
+          double z[6], zn[6];
+#pragma unroll
+          for (int k = 0; k < 6; ++k) z[k] = slot >= 0 ? zin[(6 * slot + k) * n] : 0.0;
+          leaf_iso<double, double>(t.ph[side], side ? eR : eL, z, side ? s1 : s0, &D[side], STATES ? zn : nullptr, nullptr);
+          if (STATES && slot >= 0) {
+#pragma unroll
+            for (int k = 0; k < 6; ++k) zout[(6 * slot + k) * n] = zn[k];
+          }
+        }
+        {
+          const Lam<CMP> lam(t, h);
+          double v[3] = {0.0, 0.0, 0.0}, c1 = lam.c1, c2 = lam.c2, c12 = lam.c1 * lam.c2;
+          if (CMP && lam.mode) { c2 = lam.mode == 2 ? 1.0 : 0.0; c1 = 1.0 - c2; c12 = 0.0; }
+          else normal(lam, v);
+          condense64_bottom(v, c1, c2, c12, s0, D[0], t.ph[0].kind == 0, s1, D[1], t.ph[1].kind == 0, res);
+          if (CMP && lam.mode) {
+#pragma unroll
+            for (int I = 0; I < 6; ++I) res.sb[I] = lam.mode == 2 ? s1[I] : s0[I];
+          }
+        }
+        if (!(q & 1)) {
+          put27(M.s, tid, res);
+          sget6(M.f, tid, e);
+        } else {
+          get27(M.s, tid, sib);
+          up(heap(mid), sib, res, o);
+          if (q == 1) {
+            put27(M.c, tid, o);
+            sget6(M.e, tid, e);
+          }
+        }
+      }
+      get27(M.c, tid, sib);
+      up(heap(0), sib, o, res);
+      put27(M.c, tid, res);
+    } else if (act) {
+#pragma unroll
+      for (int k = 0; k < 27; ++k) M.c[k][tid] = 0.0;
+    }
+    __syncthreads();
+    for (int l = Kt - 1; l >= 0; --l) {
+      if (act && lev == l) {
+        Sub64 L, R, o;
+        get27(M.c, pos, L);
+        get27(M.c, pos + half, R);
+        up(s - 1, L, R, o);
+        put27(M.c, pos, o);
+      }
+      __syncthreads();
+    }
+    // rotation to the global frame by a thread per entry: R (6 x 6), R C, (R C) R^T
+    const int pi[6] = {0, 1, 2, 1, 0, 0}, pj[6] = {0, 1, 2, 2, 2, 1};
+    constexpr double W2 = 1.41421356237309504880;
+    double* rot = &M.s[0][0];           // [36][nP] R, then [36][nP] R C (in chunks of at most 32 points)
+    const int w = min(nP, 32);
+    for (int p0 = 0; p0 < nP; p0 += w) {
+      for (int x = tid; x < 36 * w; x += ST) {
+        const int pp = x % w, I = x / w / 6, J = x / w % 6;
+        const unsigned long long ii = begin + b * nP + p0 + pp;
+        if (ii >= end) continue;
+        const double* Q = P.Q + 9 * (P.perm ? P.perm[ii] : (int64_t)ii);
+        const double wIJ = (I < 3 ? 1.0 : W2) * (J < 3 ? 1.0 : W2) * 0.5;
+        rot[x] = wIJ * (Q[3 * pi[I] + pi[J]] * Q[3 * pj[I] + pj[J]] + Q[3 * pi[I] + pj[J]] * Q[3 * pj[I] + pi[J]]);
+      }
+      __syncthreads();
+      for (int x = tid; x < 36 * w; x += ST) {
+        const int pp = x % w, I = x / w / 6, J = x / w % 6;
+        double v = 0.0;
+        for (int k = 0; k < 6; ++k) v += rot[(6 * I + k) * w + pp] * (k < 3 ? 1.0 : W2) * M.c[6 + sidx(k, J)][p0 + pp];
+        rot[36 * w + x] = (J < 3 ? 1.0 : W2) * v;
+      }
+      __syncthreads();
+      for (int x = tid; x < 42 * w; x += ST) {
+        const int pp = x % w, y = x / w;
+        const unsigned long long ii = begin + b * nP + p0 + pp;
+        if (ii >= end) continue;
+        int64_t q;
+        int tt;
+        point_of(P.perm, P.tid, P.F.n, (int64_t)ii, q, tt);
+        if (tt != tr) continue;
+        const int qs = P.status[q];
+        if (qs == STATUS_RETRY) continue;
+        double v = 0.0;
+        if (y < 36) {
+          for (int k = 0; k < 6; ++k) v += rot[(36 + 6 * (y / 6) + k) * w + pp] * rot[(6 * (y % 6) + k) * w + pp];
+          P.tangent[36 * q + y] = qs == DMN_STATUS_NONFINITE ? qnan : v;
+        } else {
+          for (int k = 0; k < 6; ++k) v += rot[(6 * (y - 36) + k) * w + pp] * M.c[k][p0 + pp];
+          P.stress[6 * q + y - 36] = qs == DMN_STATUS_NONFINITE ? qnan : v;
+        }
+      }
+      __syncthreads();
+    }
+  }
+}
+
+template <bool CMP, bool STATES>
+static cudaError_t sweep(const SweepParams& P, unsigned grid, cudaStream_t s) {
+  const int bytes = (int)sizeof(SweepShared);
+  const cudaError_t e = cudaFuncSetAttribute(k_sweep_block<CMP, STATES>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e != cudaSuccess) return e;
+  k_sweep_block<CMP, STATES><<<grid, ST, bytes, s>>>(P);
+  return cudaSuccess;
+}
+
+cudaError_t launch_sweep_block(const SweepParams& P, bool cmp, bool states, unsigned grid, cudaStream_t s) {
+  if (cmp) return states ? sweep<true, true>(P, grid, s) : sweep<true, false>(P, grid, s);
+  return states ? sweep<false, true>(P, grid, s) : sweep<false, false>(P, grid, s);
 }
 
 template <bool LS, bool CMP>

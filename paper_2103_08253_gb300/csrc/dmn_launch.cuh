@@ -83,11 +83,6 @@ constexpr int WARP_MIN_LANES = 8;     // the smallest group: the scratch holds 3
 // grid * 128 / lanes slots of warp_slot_doubles<T>(P.N_max) doubles
 template <typename T, bool CMP>
 void launch_warp(const NewtonParams<T>& P, bool ls, int lanes, unsigned grid, double* scr, cudaStream_t s);
-// k_sweep_warp<CMP, lanes>: the mixed form's FP64 final sweep in the warp organisation (csrc/dmn_warp.cu);
-// `scr` holds grid * 128 / lanes slots of warp_slot_doubles<double>(P.N_max) doubles
-template <bool CMP>
-void launch_sweep_warp(const NewtonParams<double>& P, int lanes, unsigned grid, double* scr, cudaStream_t s);
-
 // The CTA organisation of the FP64 form (csrc/dmn_block.cu).  counter: [1..9] points per tree and
 // [10..18] their ends in perm (several trees), [21..28] work counters per tree, [29] points on the list.
 constexpr int BLOCK_THREADS = 256;
@@ -126,6 +121,23 @@ __device__ __forceinline__ void block_retry(const BlockParams& P, int64_t pt) {
   P.status[pt] = STATUS_RETRY;
   P.list[atomicAdd(P.counter + 29, 1ull)] = pt;
 }
+// The FP64 sweep in the same organisation (k_sweep_block): stress, tangent and, on request, leaf states at the
+// jumps in state_out, of every point whose status is not RETRY.  counter: as above, [1..9] and [10..18].
+constexpr int SWEEP_THREADS = 128;
+constexpr int SWEEP_CTAS_PER_SM = 2;
+struct SweepParams {
+  Forest F;
+  int64_t n;
+  int N_max;
+  const int32_t* tid;
+  const int64_t* perm;
+  const double *Q, *state_in;
+  double *state_out, *stress, *tangent;
+  const int32_t* status;
+  const double* nbuf;
+  const unsigned long long* counter;
+};
+cudaError_t launch_sweep_block(const SweepParams& P, bool cmp, bool states, unsigned grid, cudaStream_t s);
 cudaError_t launch_block(const BlockParams& P, bool ls, bool cmp, unsigned grid, cudaStream_t s);
 
 }  // namespace dmn
