@@ -306,7 +306,7 @@ int dmn_set_params(dmn_handle* h, int32_t tree_id, const double* p, const double
  * g_stress NULL, E_n, dE, state_in and state_out may be NULL and g_E (if
  * given) is set to zero.  One tree per handle (tree_id must be NULL).  The
  * first call with a larger n than any earlier call (up to 65536 points per
- * chunk, about 71 KB each at K = 8) allocates work space.  Errors: DMN_ERR_ARG
+ * chunk, about 18 KB each at K = 8, and once 100 MB) allocates work space.  Errors: DMN_ERR_ARG
  * for NULL arrays, both seeds NULL, a tangent seed on a tree with an inelastic
  * phase, n < 0, a non-NULL tree_id or a handle with several trees. */
 int dmn_grad(dmn_handle* h, int64_t n, const int32_t* tree_id, const double* lam, const double* Q, const double* E_n,

@@ -3,7 +3,7 @@
 ``python -m paper_2103_08253_gb300.build`` compiles ``csrc/dmn.cu`` (the DMN
 update: C ABI and the thread-per-point kernels), ``csrc/dmn_warp.cu`` (its warp
 organisation for small calls), ``csrc/dmn_block.cu`` (the FP64 form's Newton
-iteration), ``csrc/fe.cu`` (the hexahedral FE operator and
+iteration and the FP64 sweep), ``csrc/dmn_grad.cu`` (the adjoints), ``csrc/fe.cu`` (the hexahedral FE operator and
 PCG) and ``csrc/peak.cu`` (the measured FMA peaks of the rooflines) with nvcc, in
 parallel, and links them into ``_build/libdmn.so`` next to this file.
 """
@@ -18,8 +18,10 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 SOURCES = [os.path.join(HERE, "csrc", "dmn.cu"), os.path.join(HERE, "csrc", "dmn_warp.cu"),
            os.path.join(HERE, "csrc", "dmn_block.cu"),
+           os.path.join(HERE, "csrc", "dmn_grad.cu"),
            os.path.join(HERE, "csrc", "fe.cu"), os.path.join(HERE, "csrc", "peak.cu")]
 DEPS = SOURCES + [os.path.join(HERE, "csrc", "dmn_device.cuh"), os.path.join(HERE, "csrc", "dmn_launch.cuh"),
+                  os.path.join(HERE, "csrc", "dmn_block.cuh"),
                   os.path.join(ROOT, "include", "dmn.h"),
                   os.path.join(ROOT, "include", "fe.h"), os.path.join(ROOT, "include", "dmn_peak.h")]
 LIB = os.path.join(HERE, "_build", "libdmn.so")

@@ -100,6 +100,7 @@ struct dmn_handle {
   HostPipe hp;
   double* gwork = nullptr;      // dmn_grad per-point work, one chunk
   int64_t gwork_cap = 0;
+  double* gscratch = nullptr;   // and the adjoints' per-CTA scratch (csrc/dmn_grad.cu)
   bool profiling = false;
   std::vector<std::array<cudaEvent_t, 5>> events;  // per timed update: before/after each kernel
   unsigned long long* d_passes = nullptr;          // profiling: tree passes of the first stage and of k_newton
@@ -939,24 +940,25 @@ __global__ void __launch_bounds__(128) k_grad(GradParams P) {
 // Sums the per-point gradients of a chunk into the parameter gradients (added to
 // g_p, g_q, g_w in the paper's ordering): one CTA per parameter, fixed-order
 // reduction, so results are repeatable bit for bit.
-__global__ void __launch_bounds__(256) k_grad_reduce(TreeDev t, int64_t nc, const double* __restrict__ work,
-                                                     double* g_p, double* g_q, double* g_w) {
+// gab, gw, ph: the first fields of the angles' and weights' gradients and of the shape-function values.
+__global__ void __launch_bounds__(256) k_grad_reduce(TreeDev t, int64_t nc, const double* __restrict__ work, int gab,
+                                                     int gw, int ph, double* g_p, double* g_q, double* g_w) {
   const int r = blockIdx.x;
-  const int N = t.N, M = t.M, L = t.L;
+  const int N = t.N, M = t.M;
   const size_t ws = (size_t)nc;
   const double* base;
   const double* fac = nullptr;
   double* out;
   if (r < 2 * N * M) {
     const int which = r / (N * M), rr = r % (N * M), node = rr / M, m = rr % M;
-    base = work + (size_t)(31 * N + which * N + node) * ws;
-    fac = work + (size_t)(33 * N + 2 * L + m) * ws;
+    base = work + (size_t)(gab + which * N + node) * ws;
+    fac = work + (size_t)(ph + m) * ws;
     const int lvl = 32 - __clz(node + 1);
     const int j = t.pidx ? t.pidx[node] : (1 << t.K) - 3 * (1 << (lvl - 1)) + node + 1;
     out = (which ? g_q : g_p) + j * M + m;
   } else {
     const int l = r - 2 * N * M;
-    base = work + (size_t)(33 * N + L + l) * ws;
+    base = work + (size_t)(gw + l) * ws;
     out = g_w + l;
   }
   double s = 0.0;
@@ -1718,6 +1720,7 @@ void dmn_destroy(dmn_handle* h) {
   for (auto& w : h->ws) free_ws(w);
   free_pipe(h->hp);
   cudaFree(h->gwork);
+  cudaFree(h->gscratch);
   cudaFree(h->d_passes);
   delete h;
 }
@@ -1952,7 +1955,9 @@ int dmn_grad(dmn_handle* h, int64_t n, const int32_t* tree_id, const double* lam
     return fail(h, DMN_ERR_ARG, "dmn_grad: NULL array");
   cudaStream_t s = (cudaStream_t)stream;
   const int64_t chunk = std::min<int64_t>(n, 65536);   // few points per chunk leave the adjoint latency-bound
-  const size_t fields = g_tangent ? grad_fields_tangent(T.N, T.L) : grad_fields(T.N, T.L);
+  const bool block = block_trees(h);                   // the CTA organisation, or one thread / warp per point (depth < 3)
+  GradWork G{td, n, 0, chunk, lam, Q, E_n, dE, state_in, state_out, g_stress, g_tangent, g_E, nullptr, nullptr};
+  const size_t fields = block ? (size_t)G.fields() : g_tangent ? grad_fields_tangent(T.N, T.L) : grad_fields(T.N, T.L);
   const int64_t need = (int64_t)(fields * (size_t)chunk);   // doubles
   cudaError_t e;
   if (need > h->gwork_cap) {
@@ -1962,10 +1967,28 @@ int dmn_grad(dmn_handle* h, int64_t n, const int32_t* tree_id, const double* lam
     if (e != cudaSuccess) return cuda_fail(h, e, "dmn_grad: work buffer");
     h->gwork_cap = need;
   }
+  if (block && !h->gscratch) {
+    e = cudaMalloc(&h->gscratch, sizeof(double) * GRAD_SCRATCH_DOUBLES * SWEEP_THREADS * (size_t)(h->n_sm * SWEEP_CTAS_PER_SM));
+    if (e != cudaSuccess) return cuda_fail(h, e, "dmn_grad: work buffer");
+  }
   const int n_params = 2 * T.N * T.M + T.L;
   for (int64_t n0 = 0; n0 < n; n0 += chunk) {
     const int64_t nc = std::min(chunk, n - n0);
     const unsigned grid = (unsigned)div_up(nc, 128);
+    if (block) {
+      G.n0 = n0; G.nc = nc; G.work = h->gwork; G.scratch = h->gscratch;
+      const unsigned ctas = (unsigned)std::min<int64_t>(div_up(nc, SWEEP_THREADS >> (T.K - 3)),
+                                                        (int64_t)h->n_sm * SWEEP_CTAS_PER_SM);
+      e = launch_grad_normals(G, (unsigned)point_split(nc, h->n_sm, T.N), s);
+      for (int tangent = 0; tangent < 2 && e == cudaSuccess; ++tangent) {   // each seed's terms added in turn
+        if (tangent ? !g_tangent : !g_stress) continue;
+        G.g_E = tangent && g_stress ? nullptr : g_E;   // the stress seed's; the tangent seed's is zero
+        e = launch_grad_block(G, h->cmp, tangent != 0, ctas, s);
+        if (e == cudaSuccess) k_grad_reduce<<<n_params, 256, 0, s>>>(td, nc, h->gwork, G.gab(), G.gw(), G.ph(), g_p, g_q, g_w);
+      }
+      if (e != cudaSuccess) return cuda_fail(h, e, "dmn_grad: launch");
+      continue;
+    }
     if (g_stress) {
       GradParams P{td, n, n0, nc, lam, Q, E_n, dE, state_in, state_out, g_stress, g_E, h->gwork};
       if (h->cmp) k_grad<true><<<grid, 128, 0, s>>>(P);
@@ -1977,7 +2000,7 @@ int dmn_grad(dmn_handle* h, int64_t n, const int32_t* tree_id, const double* lam
       if (h->cmp) k_grad_tangent<true><<<wgrid, 128, 0, s>>>(P);
       else k_grad_tangent<false><<<wgrid, 128, 0, s>>>(P);
     }
-    k_grad_reduce<<<n_params, 256, 0, s>>>(td, nc, h->gwork, g_p, g_q, g_w);
+    k_grad_reduce<<<n_params, 256, 0, s>>>(td, nc, h->gwork, 31 * T.N, 33 * T.N + T.L, 33 * T.N + 2 * T.L, g_p, g_q, g_w);
   }
   e = cudaGetLastError();
   return e == cudaSuccess ? DMN_OK : cuda_fail(h, e, "dmn_grad: launch");

@@ -140,4 +140,23 @@ struct SweepParams {
 cudaError_t launch_sweep_block(const SweepParams& P, bool cmp, bool states, unsigned grid, cudaStream_t s);
 cudaError_t launch_block(const BlockParams& P, bool ls, bool cmp, unsigned grid, cudaStream_t s);
 
+// The adjoints in the CTA organisation (csrc/dmn_grad.cu): one chunk of nc points from n0 on.  work, field-major
+// over the chunk: normals [3 N], sin(alpha), cos(beta), sin(beta) [3 N], dL/d alpha [N], dL/d beta [N], dL/dw [L],
+// shape-function values [6].
+constexpr int GRAD_SCRATCH_DOUBLES = 320;   // per thread of a CTA
+struct GradWork {
+  TreeDev t;
+  int64_t n, n0, nc;
+  const double *lam, *Q, *En, *dE, *state_in, *state_out, *g_stress, *g_tangent;
+  double* g_E;
+  double* work;
+  double* scratch;
+  __host__ __device__ int gab() const { return 6 * t.N; }
+  __host__ __device__ int gw() const { return 8 * t.N; }
+  __host__ __device__ int ph() const { return 8 * t.N + t.L; }
+  __host__ __device__ int fields() const { return 8 * t.N + t.L + 6; }
+};
+cudaError_t launch_grad_normals(const GradWork& G, unsigned split, cudaStream_t s);
+cudaError_t launch_grad_block(const GradWork& G, bool cmp, bool tangent, unsigned grid, cudaStream_t s);
+
 }  // namespace dmn
