@@ -11,7 +11,13 @@
 // sums, per node, the entries of its elements in a fixed order (node-to-element
 // lists built at mesh creation): no atomics, and results that do not depend on
 // scheduling.  Reductions for the CG (dot products) likewise use per-block
-// partial sums and one final block in a fixed order.
+// partial sums and one final sum in a fixed order.
+//
+// A CG iteration is three kernels.  At 74 k Gauss points (12 k nodes) every one of them is a few microseconds
+// of latency, so launches count: the search direction p = z + beta p is formed where it is read (the products)
+// and stored by the node sums, which also take p . K p; the scalars alpha and beta are summed from the partial
+// sums by every block that needs them, in the order of the one-block reduction they replace.  46 -> 25 us per
+// iteration (seven kernels before) with the same roundings.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -30,7 +36,7 @@ constexpr int GF = 25;             // fields per Gauss point: 24 gradients + det
 constexpr int TPB = 256;           // threads per block of the operator kernels
 constexpr int RED_BLOCKS = 608;    // partial sums per reduction (<= 1024)
 constexpr double RS2 = 0.70710678118654752440;  // 1 / sqrt(2)
-enum { S_RZ = 0, S_PQ = 1, S_RZN = 2, S_RR = 3, S_BB = 4, S_OUT = 5, N_SCAL = 8 };
+enum { S_RZ = 0 /* r.z of the even, then of the odd iterations */, S_RR = 3, S_OUT = 5, N_SCAL = 8 };
 
 }  // namespace
 
@@ -44,10 +50,10 @@ struct fe_mesh {
   float* G32 = nullptr;        // dev [25][n_gp]: FP32 copy of G (fe_pcg_f32, made on first use)
   float* C32 = nullptr;        // dev [36][n_gp]: FP32 tangents, field-major (fe_pcg_f32)
   float* fe32 = nullptr;       // dev [n_elem][24] FP32 element vectors (fe_pcg_f32)
-  double* part = nullptr;      // dev [2][RED_BLOCKS] partial sums
+  double* part = nullptr;      // dev [3][RED_BLOCKS] partial sums: r.z, r.r, p.q
   double* scal = nullptr;      // dev [N_SCAL] CG scalars
   double* h_scal = nullptr;    // pinned host copy of scal
-  double *r = nullptr, *z = nullptr, *p = nullptr, *q = nullptr;  // dev [n_dofs] CG vectors
+  double *r = nullptr, *z = nullptr, *p = nullptr, *p2 = nullptr, *q = nullptr;  // dev [n_dofs] CG vectors
   double volume = 0.0;
   std::string err;
 };
@@ -150,25 +156,36 @@ __device__ __forceinline__ void bt_apply(const double ga[3], const double ws[6],
   out[2] = ga[2] * ws[2] + ga[1] * ws[3] + ga[0] * ws[4];
 }
 
-// Sums v over the 8 lanes of this Gauss point's element (all lanes of the warp call it).
-__device__ __forceinline__ double elem_sum(double v) {
-  v += __shfl_xor_sync(0xffffffffu, v, 1);
-  v += __shfl_xor_sync(0xffffffffu, v, 2);
-  v += __shfl_xor_sync(0xffffffffu, v, 4);
-  return v;
-}
-
-// Sums the element vector fe [8][3] over the element's 8 Gauss points (lanes);
-// lane g writes the three entries of node g to the element vector out [n_elem][24].
-__device__ __forceinline__ void store_element(int64_t e, int g, bool valid, double fe[8][3], double* out) {
-  double mine[3] = {0.0, 0.0, 0.0};
+// Sums the element vector fe [8][3] over the element's 8 Gauss points (8 consecutive lanes; all lanes of the warp
+// call it); lane g gets the three entries of node g.  Each step halves the nodes a lane keeps: 21 exchanges and
+// sums instead of the 72 of a butterfly per entry, paired in the same order.
+template <typename T>
+__device__ __forceinline__ void element_sum(int g, const T fe[8][3], T mine[3]) {
+  T a[4][3], b[2][3];
 #pragma unroll
-  for (int a = 0; a < 8; ++a)
+  for (int k = 0; k < 4; ++k)
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-      const double s = elem_sum(fe[a][i]);
-      if (a == g) mine[i] = s;
+      const T keep = g & 1 ? fe[2 * k + 1][i] : fe[2 * k][i], give = g & 1 ? fe[2 * k][i] : fe[2 * k + 1][i];
+      a[k][i] = keep + __shfl_xor_sync(0xffffffffu, give, 1);
     }
+#pragma unroll
+  for (int k = 0; k < 2; ++k)
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const T keep = g & 2 ? a[2 * k + 1][i] : a[2 * k][i], give = g & 2 ? a[2 * k][i] : a[2 * k + 1][i];
+      b[k][i] = keep + __shfl_xor_sync(0xffffffffu, give, 2);
+    }
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const T keep = g & 4 ? b[1][i] : b[0][i], give = g & 4 ? b[0][i] : b[1][i];
+    mine[i] = keep + __shfl_xor_sync(0xffffffffu, give, 4);
+  }
+}
+template <typename T>
+__device__ __forceinline__ void store_element(int64_t e, int g, bool valid, const T fe[8][3], T* out) {
+  T mine[3];
+  element_sum<T>(g, fe, mine);
   if (valid) {
 #pragma unroll
     for (int i = 0; i < 3; ++i) out[24 * e + 3 * g + i] = mine[i];
@@ -189,22 +206,65 @@ __global__ void __launch_bounds__(256) k_gather_nodes(int64_t n_nodes, const int
   f[3 * nd] = s0; f[3 * nd + 1] = s1; f[3 * nd + 2] = s2;
 }
 
-__device__ __forceinline__ void gather_element(const int32_t* conn, int64_t e, const double* u, double ue[8][3]) {
-#pragma unroll
-  for (int a = 0; a < 8; ++a) {
-    const int64_t node = conn[8 * e + a];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) ue[a][i] = u[3 * node + i];
+// Sum of part[0 .. nb - 1], nb <= 1024, by every thread of a 256-thread block, in the order of a 1024-thread
+// block's sum of one value each (warps, then their sums); sh: 32 doubles of shared memory.
+__device__ __forceinline__ double sum_parts(const double* __restrict__ part, int nb, double* sh) {
+  const int lane = threadIdx.x & 31;
+  __syncthreads();
+  for (int w = threadIdx.x >> 5; w < 32; w += TPB / 32) {
+    double v = 32 * w + lane < nb ? part[32 * w + lane] : 0.0;
+    if (32 * w < nb)
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) sh[w] = v;
   }
+  __syncthreads();
+  double v = sh[lane];
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// The CG's search direction of iteration k: p = z + beta p_old with beta = r.z / (r.z of the last iteration);
+// p = z in the first.  part_rz: the partial sums of r.z.
+struct Direction {
+  const double *z, *p_old, *part_rz, *rz_last;
+  int nb, first;
+};
+__device__ __forceinline__ double beta_of(const Direction& D, double* sh, double& rz) {
+  rz = sum_parts(D.part_rz, D.nb, sh);
+  if (D.first) return 0.0;
+  const double last = *D.rz_last;
+  return last > 0.0 ? rz / last : 0.0;
+}
+__device__ __forceinline__ double direction(const Direction& D, double beta, int64_t i) {
+  return D.first ? D.z[i] : __fma_rn(beta, D.p_old[i], D.z[i]);
+}
+
+// The 24 nodal values of an element, as type T: lane g of the element's 8 lanes fetches node g's three and they
+// are exchanged, where every Gauss point fetched (and in FP32 converted, on the FP64 pipe) all 24.  value(i): the
+// value of dof i.
+template <typename T, typename F>
+__device__ __forceinline__ void gather_element(const int32_t* __restrict__ conn, int64_t gp, bool valid, T ue[8][3],
+                                               const F& value) {
+  T mine[3] = {(T)0, (T)0, (T)0};
+  if (valid) {
+    const int64_t node = conn[gp];   // 8 e + g
+#pragma unroll
+    for (int i = 0; i < 3; ++i) mine[i] = (T)value(3 * node + i);
+  }
+  const int base = threadIdx.x & 24;
+#pragma unroll
+  for (int a = 0; a < 8; ++a)
+#pragma unroll
+    for (int i = 0; i < 3; ++i) ue[a][i] = __shfl_sync(0xffffffffu, mine[i], base + a);
 }
 
 __global__ void __launch_bounds__(TPB) k_strain(GPView V, const int32_t* __restrict__ conn,
                                                 const double* __restrict__ u, double* __restrict__ E) {
   const int64_t gp = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (gp >= V.n_gp) return;
   double g[8][3], w, ue[8][3], eps[6];
+  gather_element<double>(conn, gp, gp < V.n_gp, ue, [&](int64_t i) { return u[i]; });
+  if (gp >= V.n_gp) return;
   load_grad(V, gp, g, w);
-  gather_element(conn, gp >> 3, u, ue);
   strain_of(g, ue, eps);
 #pragma unroll
   for (int I = 0; I < 6; ++I) E[6 * gp + I] = eps[I];
@@ -226,19 +286,23 @@ __global__ void __launch_bounds__(TPB) k_force(GPView V, const double* __restric
 #pragma unroll
     for (int a = 0; a < 8; ++a) fe[a][0] = fe[a][1] = fe[a][2] = 0.0;
   }
-  store_element(gp >> 3, (int)(gp & 7), valid, fe, fe_out);
+  store_element<double>(gp >> 3, (int)(gp & 7), valid, fe, fe_out);
 }
 
+// Products with K: of the vector v, or (CG) of the search direction.
+template <bool CG>
 __global__ void __launch_bounds__(TPB) k_apply(GPView V, const int32_t* __restrict__ conn,
-                                               const double* __restrict__ C, const double* __restrict__ v,
+                                               const double* __restrict__ C, const double* __restrict__ v, Direction D,
                                                double* __restrict__ fe_out) {
+  __shared__ double sh[32];
   const int64_t gp = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const bool valid = gp < V.n_gp;
-  double fe[8][3];
+  double fe[8][3], ve[8][3], rz, beta = 0.0;
+  if (CG) beta = beta_of(D, sh, rz);
+  gather_element<double>(conn, gp, valid, ve, [&](int64_t i) { return CG ? direction(D, beta, i) : v[i]; });
   if (valid) {
-    double g[8][3], w, ve[8][3], eps[6], tau[6];
+    double g[8][3], w, eps[6], tau[6];
     load_grad(V, gp, g, w);
-    gather_element(conn, gp >> 3, v, ve);
     strain_of(g, ve, eps);
     const double* c = C + 36 * gp;
 #pragma unroll
@@ -256,7 +320,7 @@ __global__ void __launch_bounds__(TPB) k_apply(GPView V, const int32_t* __restri
 #pragma unroll
     for (int a = 0; a < 8; ++a) fe[a][0] = fe[a][1] = fe[a][2] = 0.0;
   }
-  store_element(gp >> 3, (int)(gp & 7), valid, fe, fe_out);
+  store_element<double>(gp >> 3, (int)(gp & 7), valid, fe, fe_out);
 }
 
 // b_{a,i}^T C b_{a,i} w for every dof of the element, with b_{a,i} the Mandel strain of a unit
@@ -294,7 +358,7 @@ __global__ void __launch_bounds__(TPB) k_diag(GPView V, const double* __restrict
 #pragma unroll
     for (int a = 0; a < 8; ++a) fe[a][0] = fe[a][1] = fe[a][2] = 0.0;
   }
-  store_element(gp >> 3, (int)(gp & 7), valid, fe, fe_out);
+  store_element<double>(gp >> 3, (int)(gp & 7), valid, fe, fe_out);
 }
 
 // ---------------------------------------------------------------------------
@@ -314,20 +378,17 @@ __global__ void __launch_bounds__(256) k_pack_c(int64_t n_gp, const double* __re
   for (int k = 0; k < 36; ++k) C32[(size_t)k * n_gp + gp] = (float)C[36 * gp + k];
 }
 
-__device__ __forceinline__ float elem_sum_f(float v) {
-  v += __shfl_xor_sync(0xffffffffu, v, 1);
-  v += __shfl_xor_sync(0xffffffffu, v, 2);
-  v += __shfl_xor_sync(0xffffffffu, v, 4);
-  return v;
-}
-
 __global__ void __launch_bounds__(TPB) k_apply32(int64_t n_gp, const float* __restrict__ G32,
                                                  const int32_t* __restrict__ conn, const float* __restrict__ C32,
-                                                 const double* __restrict__ v, float* __restrict__ fe_out) {
+                                                 Direction D, float* __restrict__ fe_out) {
+  __shared__ double sh[32];
   const int64_t gp = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const bool valid = gp < n_gp;
   const float rs2 = 0.70710678f;
-  float fe[8][3];
+  float fe[8][3], ue[8][3];
+  double rz;
+  const double beta = beta_of(D, sh, rz);
+  gather_element<float>(conn, gp, valid, ue, [&](int64_t i) { return direction(D, beta, i); });
   if (valid) {
     float g[8][3];
 #pragma unroll
@@ -336,13 +397,11 @@ __global__ void __launch_bounds__(TPB) k_apply32(int64_t n_gp, const float* __re
       for (int i = 0; i < 3; ++i) g[a][i] = G32[(size_t)(3 * a + i) * n_gp + gp];
     const float w = G32[(size_t)24 * n_gp + gp];
     float d[3][3] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};
-    const int64_t e = gp >> 3;
 #pragma unroll
     for (int a = 0; a < 8; ++a) {
-      const int64_t node = conn[8 * e + a];
 #pragma unroll
       for (int i = 0; i < 3; ++i) {
-        const float ui = (float)v[3 * node + i];
+        const float ui = ue[a][i];
 #pragma unroll
         for (int j = 0; j < 3; ++j) d[i][j] += ui * g[a][j];
       }
@@ -367,32 +426,7 @@ __global__ void __launch_bounds__(TPB) k_apply32(int64_t n_gp, const float* __re
 #pragma unroll
     for (int a = 0; a < 8; ++a) fe[a][0] = fe[a][1] = fe[a][2] = 0.f;
   }
-  const int gl = (int)(gp & 7);
-  float mine[3] = {0.f, 0.f, 0.f};
-#pragma unroll
-  for (int a = 0; a < 8; ++a)
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      const float sm = elem_sum_f(fe[a][i]);
-      if (a == gl) mine[i] = sm;
-    }
-  if (valid) {
-#pragma unroll
-    for (int i = 0; i < 3; ++i) fe_out[24 * (gp >> 3) + 3 * gl + i] = mine[i];
-  }
-}
-
-__global__ void __launch_bounds__(256) k_gather_nodes32(int64_t n_nodes, const int32_t* __restrict__ nptr,
-                                                        const int32_t* __restrict__ nadj, const float* __restrict__ fe,
-                                                        double* __restrict__ f) {
-  const int64_t nd = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (nd >= n_nodes) return;
-  double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-  for (int k = nptr[nd]; k < nptr[nd + 1]; ++k) {
-    const float* x = fe + 3 * (int64_t)nadj[k];
-    s0 += (double)x[0]; s1 += (double)x[1]; s2 += (double)x[2];
-  }
-  f[3 * nd] = s0; f[3 * nd + 1] = s1; f[3 * nd + 2] = s2;
+  store_element<float>(gp >> 3, (int)(gp & 7), valid, fe, fe_out);
 }
 
 // ---------------------------------------------------------------------------
@@ -422,17 +456,12 @@ __global__ void __launch_bounds__(TPB) k_dot_part(int64_t n, const double* __res
   if (threadIdx.x == 0) part[blockIdx.x] = s;
 }
 
-// out[k] = sum of part[k * nb .. k * nb + nb - 1] for k < nk, in a fixed order (one block of 1024);
-// with rotate, scal[S_RZ] takes scal[S_RZN] first (the CG's r.z of the previous iteration)
-__global__ void k_reduce(const double* __restrict__ part, int nb, int nk, double* scal, int slot0, int rotate) {
+// *out = sum of part[0 .. nb - 1], in a fixed order (one block of 1024)
+__global__ void k_reduce(const double* __restrict__ part, int nb, double* out) {
   __shared__ double sh[32];
-  if (rotate && threadIdx.x == 0) scal[S_RZ] = scal[S_RZN];
-  for (int k = 0; k < nk; ++k) {
-    double v = (threadIdx.x < nb) ? part[k * nb + threadIdx.x] : 0.0;
-    v = block_sum(v, sh);
-    if (threadIdx.x == 0) scal[slot0 + k] = v;
-    __syncthreads();
-  }
+  double v = (threadIdx.x < nb) ? part[threadIdx.x] : 0.0;
+  v = block_sum(v, sh);
+  if (threadIdx.x == 0) *out = v;
 }
 
 __global__ void __launch_bounds__(TPB) k_axpy(int64_t n, double alpha, const double* __restrict__ x,
@@ -441,18 +470,42 @@ __global__ void __launch_bounds__(TPB) k_axpy(int64_t n, double alpha, const dou
     y[i] += alpha * (w ? w[i] : 1.0) * x[i];
 }
 
-// CG start: r = free b, x = 0, z = r / diag, p = z; partials of r.z and r.r
+// CG: q = K p from the element vectors (a thread per dof, its elements in list order), p stored, the partial sums
+// of p . q over the free dofs, and r.z of this iteration for the others' beta and alpha.
+template <typename T>
+__global__ void __launch_bounds__(TPB) k_pcg_dot(int64_t n, const int32_t* __restrict__ nptr,
+                                                 const int32_t* __restrict__ nadj, const T* __restrict__ fe, Direction D,
+                                                 const double* __restrict__ fr, double* __restrict__ p,
+                                                 double* __restrict__ q, double* rz_now, double* __restrict__ part) {
+  __shared__ double sh[32];
+  double rz;
+  const double beta = beta_of(D, sh, rz);
+  if (blockIdx.x == 0 && threadIdx.x == 0) *rz_now = rz;
+  double s = 0.0;
+  for (int64_t i = blockIdx.x * (int64_t)TPB + threadIdx.x; i < n; i += (int64_t)gridDim.x * TPB) {
+    const int64_t nd = i / 3, c = i - 3 * nd;
+    double v = 0.0;
+    for (int k = nptr[nd]; k < nptr[nd + 1]; ++k) v += (double)fe[3 * (int64_t)nadj[k] + c];
+    const double pi = direction(D, beta, i);
+    p[i] = pi;
+    q[i] = v;
+    s = __fma_rn(__dmul_rn(fr[i], pi), v, s);
+  }
+  s = block_sum(s, sh);
+  if (threadIdx.x == 0) part[blockIdx.x] = s;
+}
+
+// CG start: r = free b, x = 0, z = r / diag; partials of r.z and r.r
 __global__ void __launch_bounds__(TPB) k_pcg_init(int64_t n, const double* __restrict__ fr,
                                                   const double* __restrict__ diag, const double* __restrict__ b,
                                                   double* __restrict__ x, double* __restrict__ r,
-                                                  double* __restrict__ z, double* __restrict__ p,
-                                                  double* __restrict__ part) {
+                                                  double* __restrict__ z, double* __restrict__ part) {
   __shared__ double sh[TPB / 32];
   double rz = 0.0, rr = 0.0;
   for (int64_t i = blockIdx.x * (int64_t)TPB + threadIdx.x; i < n; i += (int64_t)gridDim.x * TPB) {
     const double ri = fr[i] * b[i];
     const double zi = (fr[i] != 0.0 && diag[i] > 0.0) ? ri / diag[i] : 0.0;
-    x[i] = 0.0; r[i] = ri; z[i] = zi; p[i] = zi;
+    x[i] = 0.0; r[i] = ri; z[i] = zi;
     rz += ri * zi; rr += ri * ri;
   }
   rz = block_sum(rz, sh);
@@ -463,13 +516,14 @@ __global__ void __launch_bounds__(TPB) k_pcg_init(int64_t n, const double* __res
 
 // x += alpha p, r -= alpha free q, z = r / diag with alpha = r.z / p.q; partials of r.z, r.r
 __global__ void __launch_bounds__(TPB) k_pcg_update(int64_t n, const double* __restrict__ fr,
-                                                    const double* __restrict__ diag, const double* __restrict__ scal,
+                                                    const double* __restrict__ diag, const double* __restrict__ rz_now,
+                                                    const double* __restrict__ part_pq,
                                                     const double* __restrict__ p, const double* __restrict__ q,
                                                     double* __restrict__ x, double* __restrict__ r,
                                                     double* __restrict__ z, double* __restrict__ part) {
-  __shared__ double sh[TPB / 32];
-  const double pq = scal[S_PQ];
-  const double alpha = pq > 0.0 ? scal[S_RZ] / pq : 0.0;
+  __shared__ double sh[32];
+  const double pq = sum_parts(part_pq, gridDim.x, sh);
+  const double alpha = pq > 0.0 ? *rz_now / pq : 0.0;
   double rz = 0.0, rr = 0.0;
   for (int64_t i = blockIdx.x * (int64_t)TPB + threadIdx.x; i < n; i += (int64_t)gridDim.x * TPB) {
     x[i] += alpha * p[i];
@@ -482,15 +536,6 @@ __global__ void __launch_bounds__(TPB) k_pcg_update(int64_t n, const double* __r
   __syncthreads();
   rr = block_sum(rr, sh);
   if (threadIdx.x == 0) { part[blockIdx.x] = rz; part[gridDim.x + blockIdx.x] = rr; }
-}
-
-// p = z + beta p, beta = r.z (new) / r.z (old)
-__global__ void __launch_bounds__(TPB) k_pcg_dir(int64_t n, const double* __restrict__ scal,
-                                                 const double* __restrict__ z, double* __restrict__ p) {
-  const double rz = scal[S_RZ];
-  const double beta = rz > 0.0 ? scal[S_RZN] / rz : 0.0;
-  for (int64_t i = blockIdx.x * (int64_t)TPB + threadIdx.x; i < n; i += (int64_t)gridDim.x * TPB)
-    p[i] = z[i] + beta * p[i];
 }
 
 unsigned op_grid(const fe_mesh* m) { return (unsigned)((m->n_gp + TPB - 1) / TPB); }
@@ -530,8 +575,11 @@ int pcg_run(fe_mesh* m, bool f32, const char* who, const double* C, const double
     k_pack_c<<<(unsigned)((m->n_gp + 255) / 256), 256, 0, s>>>(m->n_gp, C, m->C32);
   }
   const int CHECK = 8;   // iterations between convergence checks on the host
-  k_pcg_init<<<RED_BLOCKS, TPB, 0, s>>>(n, free, diag, b, x, m->r, m->z, m->p, m->part);
-  k_reduce<<<1, 1024, 0, s>>>(m->part, RED_BLOCKS, 2, m->scal, S_RZN, 0);   // r.z -> RZN, r.r -> RR
+  // blocks past the vector's end would add zeros to every sum
+  const unsigned nb = (unsigned)std::min<int64_t>(RED_BLOCKS, (n + TPB - 1) / TPB);
+  double *part_rz = m->part, *part_rr = m->part + nb, *part_pq = m->part + 2 * RED_BLOCKS;
+  k_pcg_init<<<nb, TPB, 0, s>>>(n, free, diag, b, x, m->r, m->z, part_rz);
+  k_reduce<<<1, 1024, 0, s>>>(part_rr, nb, m->scal + S_RR);
   e = cudaMemcpyAsync(m->h_scal, m->scal, sizeof(double) * N_SCAL, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_fail(m, e, who);
@@ -542,20 +590,20 @@ int pcg_run(fe_mesh* m, bool f32, const char* who, const double* C, const double
     res = 1.0;
     while (it < max_iter) {
       const int todo = std::min(CHECK, max_iter - it);
-      for (int k = 0; k < todo; ++k) {
+      for (int k = it; k < it + todo; ++k) {
+        double *p_old = k & 1 ? m->p : m->p2, *p = k & 1 ? m->p2 : m->p;
+        double *rz_now = m->scal + S_RZ + (k & 1), *rz_last = m->scal + S_RZ + (k & 1 ^ 1);
+        const Direction D{m->z, p_old, part_rz, rz_last, (int)nb, k == 0};
         if (f32) {
-          k_apply32<<<op_grid(m), TPB, 0, s>>>(m->n_gp, m->G32, m->conn, m->C32, m->p, m->fe32);
-          k_gather_nodes32<<<node_grid(m), 256, 0, s>>>(m->n_nodes, m->nptr, m->nadj, m->fe32, m->q);
+          k_apply32<<<op_grid(m), TPB, 0, s>>>(m->n_gp, m->G32, m->conn, m->C32, D, m->fe32);
+          k_pcg_dot<float><<<nb, TPB, 0, s>>>(n, m->nptr, m->nadj, m->fe32, D, free, p, m->q, rz_now, part_pq);
         } else {
-          k_apply<<<op_grid(m), TPB, 0, s>>>(view(m), m->conn, C, m->p, m->fe);
-          k_gather_nodes<<<node_grid(m), 256, 0, s>>>(m->n_nodes, m->nptr, m->nadj, m->fe, m->q);
+          k_apply<true><<<op_grid(m), TPB, 0, s>>>(view(m), m->conn, C, nullptr, D, m->fe);
+          k_pcg_dot<double><<<nb, TPB, 0, s>>>(n, m->nptr, m->nadj, m->fe, D, free, p, m->q, rz_now, part_pq);
         }
-        k_dot_part<<<RED_BLOCKS, TPB, 0, s>>>(n, m->p, m->q, free, m->part);
-        k_reduce<<<1, 1024, 0, s>>>(m->part, RED_BLOCKS, 1, m->scal, S_PQ, 1);
-        k_pcg_update<<<RED_BLOCKS, TPB, 0, s>>>(n, free, diag, m->scal, m->p, m->q, x, m->r, m->z, m->part);
-        k_reduce<<<1, 1024, 0, s>>>(m->part, RED_BLOCKS, 2, m->scal, S_RZN, 0);
-        k_pcg_dir<<<RED_BLOCKS, TPB, 0, s>>>(n, m->scal, m->z, m->p);
+        k_pcg_update<<<nb, TPB, 0, s>>>(n, free, diag, rz_now, part_pq, p, m->q, x, m->r, m->z, part_rz);
       }
+      k_reduce<<<1, 1024, 0, s>>>(part_rr, nb, m->scal + S_RR);
       it += todo;
       e = cudaGetLastError();
       if (e == cudaSuccess) e = cudaMemcpyAsync(m->h_scal, m->scal, sizeof(double) * N_SCAL, cudaMemcpyDeviceToHost, s);
@@ -628,10 +676,10 @@ int fe_mesh_create(int64_t n_nodes, int64_t n_elem, const double* xyz, const int
   if (e == cudaSuccess) e = cudaMalloc(&m->nptr, sizeof(int32_t) * nptr.size());
   if (e == cudaSuccess) e = cudaMalloc(&m->nadj, sizeof(int32_t) * nadj.size());
   if (e == cudaSuccess) e = cudaMalloc(&m->fe, sizeof(double) * 24 * n_elem);
-  if (e == cudaSuccess) e = cudaMalloc(&m->part, sizeof(double) * 2 * RED_BLOCKS);
+  if (e == cudaSuccess) e = cudaMalloc(&m->part, sizeof(double) * 3 * RED_BLOCKS);
   if (e == cudaSuccess) e = cudaMalloc(&m->scal, sizeof(double) * N_SCAL);
   if (e == cudaSuccess) e = cudaHostAlloc(&m->h_scal, sizeof(double) * N_SCAL, cudaHostAllocDefault);
-  for (double** v : {&m->r, &m->z, &m->p, &m->q})
+  for (double** v : {&m->r, &m->z, &m->p, &m->p2, &m->q})
     if (e == cudaSuccess) e = cudaMalloc(v, sizeof(double) * nd);
   if (e == cudaSuccess) e = cudaMemcpy(m->conn, conn, sizeof(int32_t) * 8 * n_elem, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(m->G, G.data(), sizeof(double) * G.size(), cudaMemcpyHostToDevice);
@@ -652,7 +700,7 @@ void fe_mesh_destroy(fe_mesh* m) {
   cudaFree(m->conn); cudaFree(m->G); cudaFree(m->part); cudaFree(m->scal);
   cudaFree(m->nptr); cudaFree(m->nadj); cudaFree(m->fe);
   cudaFree(m->G32); cudaFree(m->C32); cudaFree(m->fe32);
-  cudaFree(m->r); cudaFree(m->z); cudaFree(m->p); cudaFree(m->q);
+  cudaFree(m->r); cudaFree(m->z); cudaFree(m->p); cudaFree(m->p2); cudaFree(m->q);
   if (m->h_scal) cudaFreeHost(m->h_scal);
   delete m;
 }
@@ -686,7 +734,7 @@ int fe_apply_tangent(fe_mesh* m, const double* C, const double* v, double* Kv, v
   if (!C || !v || !Kv) return fail(m, -1, "fe_apply_tangent: NULL array");
   if (v == Kv) return fail(m, -1, "fe_apply_tangent: v and Kv must differ");
   cudaStream_t s = (cudaStream_t)stream;
-  k_apply<<<op_grid(m), TPB, 0, s>>>(view(m), m->conn, C, v, m->fe);
+  k_apply<false><<<op_grid(m), TPB, 0, s>>>(view(m), m->conn, C, v, Direction{}, m->fe);
   k_gather_nodes<<<node_grid(m), 256, 0, s>>>(m->n_nodes, m->nptr, m->nadj, m->fe, Kv);
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? 0 : cuda_fail(m, e, "fe_apply_tangent");
@@ -708,7 +756,7 @@ int fe_dot(fe_mesh* m, const double* a, const double* b, const double* free, dou
   cudaStream_t s = (cudaStream_t)stream;
   const int64_t n = 3 * m->n_nodes;
   k_dot_part<<<RED_BLOCKS, TPB, 0, s>>>(n, a, b, free, m->part);
-  k_reduce<<<1, 1024, 0, s>>>(m->part, RED_BLOCKS, 1, m->scal, S_OUT, 0);
+  k_reduce<<<1, 1024, 0, s>>>(m->part, RED_BLOCKS, m->scal + S_OUT);
   cudaError_t e = cudaMemcpyAsync(m->h_scal + S_OUT, m->scal + S_OUT, sizeof(double), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_fail(m, e, "fe_dot");
