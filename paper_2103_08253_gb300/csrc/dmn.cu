@@ -96,6 +96,7 @@ struct dmn_handle {
   int device = 0, n_sm = 0;
   int64_t nslots = 0;
   bool cmp = false;             // trees walked by tables (some tree has weightless leaves)
+  bool own_shape = true, own_stage_shape = true;   // launch shapes chosen here, not by the caller
   WorkSet ws[2];                // [0]: dmn_update; [1]: second stage of dmn_update_host
   HostPipe hp;
   double* gwork = nullptr;      // dmn_grad per-point work, one chunk
@@ -1333,18 +1334,33 @@ void launch_newton_p(const NewtonParams<T>& P, bool ls, int minb, unsigned grid,
 }
 // the first stage's kernel: ctas resident CTAs of 128 threads per SM (registers capped to fit)
 template <bool CMP>
-void launch_stage(const StageParams& P, int ctas, unsigned grid, cudaStream_t s) {
-  if (ctas <= 2) k_stage32<2, CMP><<<grid, 128, 0, s>>>(P);
-  else if (ctas == 3) k_stage32<3, CMP><<<grid, 128, 0, s>>>(P);
-  else if (ctas == 4) k_stage32<4, CMP><<<grid, 128, 0, s>>>(P);
-  else if (ctas <= 6) k_stage32<6, CMP><<<grid, 128, 0, s>>>(P);
-  else k_stage32<8, CMP><<<grid, 128, 0, s>>>(P);
+void launch_stage(const StageParams& P, int ctas, unsigned grid, int block, cudaStream_t s) {
+  if (ctas <= 2) k_stage32<2, CMP><<<grid, block, 0, s>>>(P);
+  else if (ctas == 3) k_stage32<3, CMP><<<grid, block, 0, s>>>(P);
+  else if (ctas == 4) k_stage32<4, CMP><<<grid, block, 0, s>>>(P);
+  else if (ctas <= 6) k_stage32<6, CMP><<<grid, block, 0, s>>>(P);
+  else k_stage32<8, CMP><<<grid, block, 0, s>>>(P);
 }
 
 template <typename T, bool CMP>
 void launch_newton(const NewtonParams<T>& P, bool ls, int minb, unsigned grid, int block, cudaStream_t s) {
   if (P.predictor) launch_newton_p<T, CMP, true>(P, ls, minb, grid, block, s);
   else launch_newton_p<T, CMP, false>(P, ls, minb, grid, block, s);
+}
+
+// CTAs of 32 threads per SM for a call of n points in the thread-per-point organisation, of at most `warps` per
+// SM, or 0 for the full shape.  With the full shape a call of one to two points per lane ends with its last
+// points spread thinly over all warps, each as slow as a full one: fewer lanes, evenly used, are faster.  FP32
+// condensation after the first stage, depth 8, 16 warps per SM (77824 lanes): 50001 points 11.5 ms with all, 8.6
+// ms with 11 warps (a point per lane); 100003 points 19.4 with all, 18.5, 17.8, 15.9, 17.4 ms with 10 .. 13 (two
+// points per lane and a margin of 15 % for uneven iteration counts: 12); 262144 points 39.0 with all, 40 to 41
+// with fewer.  The first stage waits on memory more than it issues: 5.7 -> 5.4 ms at a point per lane, but 12.0
+// instead of 11.0 ms at two (`waves`: the largest number of points per lane that gains).
+unsigned even_warps_per_sm(int64_t n, int n_sm, int warps, int waves) {
+  const int64_t per_warp_row = (int64_t)32 * n_sm, lanes = per_warp_row * warps;
+  if (n > waves * lanes) return 0;
+  const int64_t want = n <= lanes ? n : (n + 1) / 2 * 23 / 20;
+  return (unsigned)std::min<int64_t>(warps, div_up(want, per_warp_row));
 }
 
 // One update on work set w and stream s (the body of dmn_update; arguments checked by the caller).
@@ -1400,13 +1416,14 @@ int update_on(dmn_handle* h, WorkSet& w, int64_t n, int64_t n_call, const int32_
   const dim3 gp(g1, (unsigned)point_split(n, h->n_sm, NM));
   k_prepare<<<gp, 128, 0, s>>>(F, n, tree_id, perm, lam, Q, E_n, dE, w.nbuf, NM);
   if (ev) cudaEventRecord(ev[1], s);
-  const unsigned grid = (unsigned)(h->n_sm * h->opt.ctas_per_sm);
   const bool mixed = h->opt.precision != DMN_PREC_F64;
   const bool sweep = h->opt.precision == DMN_PREC_MIXED;   // FP64 final sweep for stress and tangent
   const int threads_per_sm = h->opt.block * h->opt.ctas_per_sm;
   const int minb = threads_per_sm > 384 ? 4 : threads_per_sm > 256 ? 3 : 2;
   const bool ls = h->opt.line_search != 0;
-  const int cta = h->opt.block;
+  const unsigned even = mixed && h->own_shape && !ls ? even_warps_per_sm(n, h->n_sm, threads_per_sm / 32, 2) : 0;
+  const unsigned grid = (unsigned)h->n_sm * (even ? even : (unsigned)h->opt.ctas_per_sm);
+  const int cta = even ? 32 : h->opt.block;
   const bool warp = warp_on(h, n_call) && w.scr_w;
   const bool stage = first_stage_on(h->opt) && !warp;   // a small batch goes straight to the warp kernel
   const unsigned wgrid = (unsigned)(h->n_sm * WARP_CTAS_PER_SM);
@@ -1418,9 +1435,10 @@ int update_on(dmn_handle* h, WorkSet& w, int64_t n, int64_t n_call, const int32_
     const int max32 = std::max(0, std::min(STAGE_MAX_ITER, h->opt.max_iter - 1));
     StageParams SP{F, n, w.nslots_s, NM, tree_id, perm, state_in, state_out, iters, w.nbuf, w.scr_s,
                    w.counter + 19, STAGE_TOL, max32, passes};
-    const unsigned sgrid = (unsigned)(h->n_sm * h->opt.stage_ctas_per_sm);
-    if (h->cmp) launch_stage<true>(SP, h->opt.stage_ctas_per_sm, sgrid, s);
-    else launch_stage<false>(SP, h->opt.stage_ctas_per_sm, sgrid, s);
+    const unsigned even = h->own_stage_shape ? even_warps_per_sm(n, h->n_sm, 4 * h->opt.stage_ctas_per_sm, 1) : 0;
+    const unsigned sgrid = (unsigned)h->n_sm * (even ? even : (unsigned)h->opt.stage_ctas_per_sm);
+    if (h->cmp) launch_stage<true>(SP, h->opt.stage_ctas_per_sm, sgrid, even ? 32 : 128, s);
+    else launch_stage<false>(SP, h->opt.stage_ctas_per_sm, sgrid, even ? 32 : 128, s);
   }
   if (ev) cudaEventRecord(ev[2], s);
   const dim3 gf(g1, final_split(n, h->n_sm));
@@ -1651,6 +1669,8 @@ int dmn_create(const dmn_tree_desc* trees, int32_t n_trees, const dmn_options* o
   dmn_handle* h = new dmn_handle();
   h->trees = tv;
   h->cmp = cmp;
+  h->own_shape = !opt || (opt->block <= 0 && opt->ctas_per_sm <= 0);
+  h->own_stage_shape = !opt || opt->stage_ctas_per_sm == 0;
   h->N_max = std::max(N_max, 1);
   for (const Tree& t : tv) h->K_max = std::max(h->K_max, t.K);
   h->S_max = S_max;
