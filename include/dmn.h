@@ -169,7 +169,10 @@ typedef struct {
   int32_t warp_lanes;     /* lanes per point in that organisation: 32 (one point per warp), 16 or 8 (two
                            * or four points per warp, side by side); 0 (default) chooses by the call's
                            * size: 32 up to 16 points per SM, then 8 in the FP64 form, 16 in the mixed
-                           * forms */
+                           * forms.  The FP64 form's trees of depth 3 or more (without the extrapolated
+                           * start or the first stage) run a third organisation at every size, in which a
+                           * CTA's threads share its points' trees; both options then only choose the
+                           * kernels of the few points handed back to the all-FP64 iteration. */
 } dmn_options;
 
 /* Create a handle for n_trees DMNs (1 <= n_trees <= DMN_MAX_TREES; trees may

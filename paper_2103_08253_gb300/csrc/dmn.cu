@@ -1286,13 +1286,13 @@ cudaError_t alloc_ws(const dmn_handle* h, WorkSet& w) {
   const size_t sd = h->opt.line_search ? 9 : 6, stt = h->opt.line_search ? 45 : 24;
   cudaError_t e = cudaMalloc(&w.scr_d, sizeof(double) * (size_t)(sd * h->N_max) * h->nslots);
   if (e == cudaSuccess) e = cudaMalloc(&w.scr_t, sizeof(double) * (size_t)(stt * h->N_max) * h->nslots);
-  if (e == cudaSuccess) e = cudaMalloc(&w.counter, sizeof(unsigned long long) * 32);
+  if (e == cudaSuccess) e = cudaMalloc(&w.counter, sizeof(unsigned long long) * (32 + BLOCK_TOKENS));
   if (e == cudaSuccess && first_stage_on(h->opt)) {
     w.nslots_s = (int64_t)h->n_sm * h->opt.stage_ctas_per_sm * 128;
     e = cudaMalloc(&w.scr_s, sizeof(float) * (size_t)(27 * h->N_max) * w.nslots_s);
   }
   if (e == cudaSuccess && block_on(h))
-    e = cudaMalloc(&w.scr_b, block_scratch_bytes(block_leaf_slots(h), h->opt.line_search != 0) * (size_t)(h->n_sm * BLOCK_CTAS_PER_SM));
+    e = cudaMalloc(&w.scr_b, block_scratch_bytes(BLOCK_THREADS, block_leaf_slots(h), h->opt.line_search != 0) * (size_t)(h->n_sm * BLOCK_CTAS_PER_SM));
   if (e == cudaSuccess && warp_possible(h)) {
     // one slot per group of the smallest size the handle may use
     w.nwarps_w = (int64_t)h->n_sm * WARP_CTAS_PER_SM * 128 / (h->opt.warp_lanes ? h->opt.warp_lanes : WARP_MIN_LANES);
@@ -1404,7 +1404,7 @@ int update_on(dmn_handle* h, WorkSet& w, int64_t n, int64_t n_call, const int32_
   }
   // counters: [0] work, [1..9] points per tree, [10..18] cursors, [19] first stage,
   // [21..29] the CTA organisation
-  e = cudaMemsetAsync(w.counter, 0, sizeof(unsigned long long) * 32, s);
+  e = cudaMemsetAsync(w.counter, 0, sizeof(unsigned long long) * (32 + BLOCK_TOKENS), s);
   if (e != cudaSuccess) return cuda_fail(h, e, "dmn_update: counter reset");
   const int64_t* perm = nullptr;
   if (sort) {
@@ -1466,10 +1466,9 @@ int update_on(dmn_handle* h, WorkSet& w, int64_t n, int64_t n_call, const int32_
     return launch_sweep_block(P, h->cmp, states, (unsigned)std::min<int64_t>(ctas, (int64_t)h->n_sm * SWEEP_CTAS_PER_SM), s);
   };
   if (block) {
-    BlockParams P{F, n, NM, block_leaf_slots(h), tree_id, perm, state_in, state_out, stress, tangent, iters, status,
+    BlockParams P{F, n, NM, h->n_sm, block_leaf_slots(h), tree_id, perm, state_in, state_out, stress, tangent, iters, status,
                   w.nbuf, w.scr_b, w.counter, w.list, h->opt.tol, h->opt.max_iter, passes ? passes + 1 : nullptr};
-    const int64_t ctas = div_up(n, BLOCK_THREADS >> (h->K_max - 3));
-    e = launch_block(P, ls, h->cmp, (unsigned)std::min<int64_t>(ctas, (int64_t)h->n_sm * BLOCK_CTAS_PER_SM), s);
+    e = launch_block(P, h->K_max, ls, h->cmp, s);
     if (e != cudaSuccess) return cuda_fail(h, e, "dmn_update: launch");
   } else if (!mixed) {
     newton_f64(DP);

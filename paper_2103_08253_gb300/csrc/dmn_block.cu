@@ -7,15 +7,21 @@
 //   S  condenses the leaf tangents in FP32 and solves for da1 (relative error some 1e-6),
 //   B  forms R + J da1 with pairs of FP32 numbers (about 46 bits) and solves again in FP32 for da2,
 // and applies da = da1 + da2, whose relative error is the product of the two solves' (1e-11, at most
-// some 1e-10 on the workloads' plastic paths), far below what the quadratic convergence leaves: the
-// iterates are those of the all-FP64 condensation, with its iteration counts.  A costs about 22 k FP64
-// instructions, a pass of the all-FP64 kernel 122 k; S and B cost none.  The tangent comes from one FP64
+// some 1e-10 on the workloads' plastic paths).  Where a large step ends in a fixed set of plastic leaves, no
+// quadratic term hides what the solves left of its linear residual: a residual above the criterion but no larger
+// than that is taken off by a further round that belongs to the same step and is not counted.  So the iterates
+// are those of the all-FP64 condensation, with its iteration counts.  A costs about 21 k FP64 instructions, a
+// pass of the all-FP64 kernel 122 k; S and B cost none.  The tangent comes from one FP64
 // sweep at the converged jumps, as in the mixed form.
 //
 // A point for which the FP32 solve does not contract (|R + J da1| > REFINE_MAX |R|: tangents near
 // singular, moduli outside the FP32 range), which is not finite or which has not converged within BLOCK_ITERS
 // corrections is put on a list (status RETRY) and updated from its start by the
 // all-FP64 kernels, so that every call keeps their results and statuses.
+//
+// Components.  Strains are engineering, stresses, tangents and flow directions tensor components (Voigt): N(n) has
+// the bare components of n, which saves the 6 multiplications per laminate of the Mandel form's 1 / sqrt 2.  The
+// leaf tangents are formed in pairs.  Depth 8 compressed, 20001 points: 10.7 -> 9.7 ms; 8 points: 0.45 -> 0.42.
 //
 // Organisation.  A CTA of 256 threads holds 256 / S points, S = 2^(K-3) threads per point: thread (s, p)
 // owns the s-th subtree of depth 3 (7 laminates, 8 leaves) of the point in slot p and, for s >= 1, the
@@ -35,8 +41,9 @@ namespace dmn {
 
 namespace {
 
-constexpr int BT = BLOCK_THREADS;
 constexpr float REFINE_MAX = 1e-3f;
+// A residual this many times what the solves left of the last step's linear system, or less, belongs to that step
+constexpr double LEFT_MAX = 4.0;
 constexpr int BLOCK_ITERS = 16;
 
 // scratch fields of a thread, in units of 8 laminates (7 of the subtree, then the top laminate)
@@ -74,6 +81,15 @@ __device__ __forceinline__ pair split(double x) {
   return {float_of(sign | h), float_of(sign | bits_of(l))};
 }
 
+}  // namespace
+
+// flags of a slot
+enum { B_ACT = 1, B_FIRST = 4, B_CONT = 8, B_CONV = 16, B_CUR = 32 };
+
+// The Newton kernel for CTAs of BT threads.  A point's results do not depend on BT, bit for bit.
+template <int BT>
+struct Block {
+
 struct Ctx {
   double* D;      // this thread's FP64 scratch: field f of laminate j at D[(8 f + j) BT]
   float* F;       // this thread's FP32 scratch
@@ -83,17 +99,17 @@ struct Ctx {
   __device__ float& f(int f, int j) const { return F[(8 * f + j) * BT]; }
 };
 
-__device__ __forceinline__ void load3(const Ctx& c, int f, int j, double v[3]) {
+static __device__ __forceinline__ void load3(const Ctx& c, int f, int j, double v[3]) {
 #pragma unroll
   for (int k = 0; k < 3; ++k) v[k] = c.d(f + k, j);
 }
-__device__ __forceinline__ void normal32(const Ctx& c, int j, float n[3], float nr[3]) {
+static __device__ __forceinline__ void normal32(const Ctx& c, int j, float n[3]) {
 #pragma unroll
-  for (int k = 0; k < 3; ++k) { n[k] = narrow_rn(c.d(D_N + k, j)); nr[k] = n[k] * (float)RS2; }
+  for (int k = 0; k < 3; ++k) n[k] = narrow_rn(c.d(D_N + k, j));
 }
 
 // The FP32 step of laminate j, g + H de.
-__device__ __forceinline__ void step32(const Ctx& c, int j, const float de[6], float da[3]) {
+static __device__ __forceinline__ void step32(const Ctx& c, int j, const float de[6], float da[3]) {
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     float v = c.f(F_G + k, j);
@@ -106,7 +122,7 @@ __device__ __forceinline__ void step32(const Ctx& c, int j, const float de[6], f
 // A, downwards: the jumps of laminate j corrected (apply) and the children's strains.  de: the FP32
 // correction of the second solve handed down (dL, dR: to the children; NULL for leaves).
 template <bool CMP, bool LS>
-__device__ __forceinline__ void down_a(const TreeDev& t, const Ctx& c, int h, int j, int a_in, int a_out, bool apply,
+static __device__ __forceinline__ void down_a(const TreeDev& t, const Ctx& c, int h, int j, int a_in, int a_out, bool apply,
                                        double step, const double e[6], const float de[6], double eL[6], double eR[6],
                                        float* dL, float* dR) {
   const Lam<CMP> q(t, h);
@@ -124,9 +140,8 @@ __device__ __forceinline__ void down_a(const TreeDev& t, const Ctx& c, int h, in
     if (dL) {
       const float c1 = __ldg(t.c1f + q.id), c2 = __ldg(t.c2f + q.id);
       const float n[3] = {narrow_rn(nd[0]), narrow_rn(nd[1]), narrow_rn(nd[2])};
-      const float nr[3] = {n[0] * (float)RS2, n[1] * (float)RS2, n[2] * (float)RS2};
       float Nd[6];
-      N_apply<float>(n, nr, da, Nd);
+      N_apply<float>(n, n, da, Nd);
 #pragma unroll
       for (int I = 0; I < 6; ++I) { dL[I] = de[I] - c2 * Nd[I]; dR[I] = de[I] + c1 * Nd[I]; }
     }
@@ -146,23 +161,21 @@ __device__ __forceinline__ void down_a(const TreeDev& t, const Ctx& c, int h, in
       for (int k = 0; k < 3; ++k) c.d(a_out + k, j) = a[k];
     }
   }
-  const double ndr[3] = {nd[0] * RS2, nd[1] * RS2, nd[2] * RS2};
   double Na[6];
-  N_apply<double>(nd, ndr, a, Na);
+  N_apply<double>(nd, nd, a, Na);
 #pragma unroll
   for (int I = 0; I < 6; ++I) { eL[I] = e[I] - q.c2 * Na[I]; eR[I] = e[I] + q.c1 * Na[I]; }
 }
 
-// N(n) x for x in FP32 and N(n)^T v, in pairs
-__device__ __forceinline__ void pair_normal(const Ctx& c, int j, pair n[3], pair nr[3]) {
+static __device__ __forceinline__ void pair_normal(const Ctx& c, int j, pair n[3]) {
 #pragma unroll
-  for (int k = 0; k < 3; ++k) { n[k] = split(c.d(D_N + k, j)); nr[k] = mul(n[k], split(RS2)); }
+  for (int k = 0; k < 3; ++k) n[k] = split(c.d(D_N + k, j));
 }
 
 // B, downwards: the step da1 of laminate j stored, and its strains in the children.
 template <bool CMP>
-__device__ __forceinline__ void down_b(const TreeDev& t, const Ctx& c, int h, int j, const pair e[6], pair eL[6],
-                                       pair eR[6]) {
+static __device__ __forceinline__ void down_b(const TreeDev& t, const Ctx& c, int h, int j, const pair e[6],
+                                       pair eL[6], pair eR[6]) {
   const Lam<CMP> q(t, h);
   if (CMP && q.mode) {
 #pragma unroll
@@ -175,10 +188,10 @@ __device__ __forceinline__ void down_b(const TreeDev& t, const Ctx& c, int h, in
   step32(c, j, de, x);
 #pragma unroll
   for (int k = 0; k < 3; ++k) c.f(F_D + k, j) = x[k];
-  pair n[3], nr[3];
-  pair_normal(c, j, n, nr);
-  const pair Nx[6] = {mul(n[0], x[0]), mul(n[1], x[1]), mul(n[2], x[2]), add(mul(nr[2], x[1]), mul(nr[1], x[2])),
-                      add(mul(nr[2], x[0]), mul(nr[0], x[2])), add(mul(nr[1], x[0]), mul(nr[0], x[1]))};
+  pair n[3];
+  pair_normal(c, j, n);
+  const pair Nx[6] = {mul(n[0], x[0]), mul(n[1], x[1]), mul(n[2], x[2]), add(mul(n[2], x[1]), mul(n[1], x[2])),
+                      add(mul(n[2], x[0]), mul(n[0], x[2])), add(mul(n[1], x[0]), mul(n[0], x[1]))};
   const pair c2 = split(-q.c2);
 #pragma unroll
   for (int I = 0; I < 6; ++I) { eL[I] = add(e[I], mul(c2, Nx[I])); eR[I] = add(eL[I], Nx[I]); }   // c1 = 1 - c2
@@ -186,7 +199,7 @@ __device__ __forceinline__ void down_b(const TreeDev& t, const Ctx& c, int h, in
 
 // A, upwards: residual of laminate j (t = N^T (s_R - s_L), stored) and the average stress.
 template <bool CMP>
-__device__ __forceinline__ void up_a(const TreeDev& t, const Ctx& c, int h, int j, const double sL[6],
+static __device__ __forceinline__ void up_a(const TreeDev& t, const Ctx& c, int h, int j, const double sL[6],
                                      const double sR[6], double sb[6], double& r2) {
   const Lam<CMP> q(t, h);
   if (CMP && q.mode) {
@@ -196,7 +209,12 @@ __device__ __forceinline__ void up_a(const TreeDev& t, const Ctx& c, int h, int 
   }
   double nd[3], u[3];
   load3(c, D_N, j, nd);
-  residual_share<double>(nd, q.c1, q.c2, __ldg(t.sc + q.id), sL, sR, sb, u, r2);
+  double d[6];
+#pragma unroll
+  for (int I = 0; I < 6; ++I) { d[I] = sR[I] - sL[I]; sb[I] = sL[I] + q.c2 * d[I]; }
+  Nt_apply<double>(nd, nd, d, u);
+  const double sc = __ldg(t.sc + q.id);
+  r2 += sc * sc * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     const pair v = split(u[k]);
@@ -210,7 +228,7 @@ __device__ __forceinline__ void up_a(const TreeDev& t, const Ctx& c, int h, int 
 //   u += N^T (ds_R - ds_L),  g = -Kn^-1 u,  ds = c1 ds_L + c2 ds_R + c1 c2 H^T u.
 // BOT: the children are leaves (ds = 0 there).
 template <bool CMP, bool BOT>
-__device__ __forceinline__ void up_b(const TreeDev& t, const Ctx& c, int h, int j, const pair tL[6], const pair tR[6],
+static __device__ __forceinline__ void up_b(const TreeDev& t, const Ctx& c, int h, int j, const pair tL[6], const pair tR[6],
                                      const float dsL[6], const float dsR[6], pair tb[6], float ds[6], float& r2) {
   const Lam<CMP> q(t, h);
   if (CMP && q.mode) {
@@ -221,14 +239,14 @@ __device__ __forceinline__ void up_b(const TreeDev& t, const Ctx& c, int h, int 
     }
     return;
   }
-  pair n[3], nr[3], d[6];
-  pair_normal(c, j, n, nr);
+  pair n[3], d[6];
+  pair_normal(c, j, n);
   const pair p2 = split(q.c2);
 #pragma unroll
   for (int I = 0; I < 6; ++I) { d[I] = add(tR[I], neg(tL[I])); tb[I] = add(tL[I], mul(p2, d[I])); }
-  const pair v[3] = {add(mul(n[0], d[0]), add(mul(nr[2], d[4]), mul(nr[1], d[5]))),
-                     add(mul(n[1], d[1]), add(mul(nr[2], d[3]), mul(nr[0], d[5]))),
-                     add(mul(n[2], d[2]), add(mul(nr[1], d[3]), mul(nr[0], d[4])))};
+  const pair v[3] = {add(mul(n[0], d[0]), add(mul(n[2], d[4]), mul(n[1], d[5]))),
+                     add(mul(n[1], d[1]), add(mul(n[2], d[3]), mul(n[0], d[5]))),
+                     add(mul(n[2], d[2]), add(mul(n[1], d[3]), mul(n[0], d[4])))};
   float u[3];
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
@@ -240,11 +258,11 @@ __device__ __forceinline__ void up_b(const TreeDev& t, const Ctx& c, int h, int 
   for (int k = 0; k < 3; ++k) r2 += (sc * u[k]) * (sc * u[k]);
   float dd[6];
   if (!BOT) {
-    const float m[3] = {n[0].h, n[1].h, n[2].h}, mr[3] = {nr[0].h, nr[1].h, nr[2].h};
+    const float m[3] = {n[0].h, n[1].h, n[2].h};
     float w[3];
 #pragma unroll
     for (int I = 0; I < 6; ++I) dd[I] = dsR[I] - dsL[I];
-    Nt_apply<float>(m, mr, dd, w);
+    Nt_apply<float>(m, m, dd, w);
 #pragma unroll
     for (int k = 0; k < 3; ++k) u[k] += w[k];
   }
@@ -270,7 +288,7 @@ struct Sub32 {
   float ds[6], C[21];
 };
 
-__device__ __forceinline__ void solve32(const Ctx& c, int j, float c12, const float Ki[3][3], const float B[6][3],
+static __device__ __forceinline__ void solve32(const Ctx& c, int j, float c12, const float Ki[3][3], const float B[6][3],
                                         const float u[3], float ds[6], float C[21]) {
   float H[3][6], g[3];
 #pragma unroll
@@ -297,7 +315,7 @@ __device__ __forceinline__ void solve32(const Ctx& c, int j, float c12, const fl
 }
 
 template <bool CMP>
-__device__ __forceinline__ void condense32(const TreeDev& t, const Ctx& c, int h, int j, const Sub32& L, const Sub32& R,
+static __device__ __forceinline__ void condense32(const TreeDev& t, const Ctx& c, int h, int j, const Sub32& L, const Sub32& R,
                                            Sub32& o) {
   const Lam<CMP> q(t, h);
   if (CMP && q.mode) {
@@ -305,26 +323,26 @@ __device__ __forceinline__ void condense32(const TreeDev& t, const Ctx& c, int h
     return;
   }
   const float c2 = __ldg(t.c2f + q.id), c12 = __ldg(t.c12f + q.id);
-  float n[3], nr[3];
-  normal32(c, j, n, nr);
+  float n[3];
+  normal32(c, j, n);
   float dC[21], Ch[21], X[6][3], B[6][3], u[3], w[3], dd[6];
 #pragma unroll
   for (int k = 0; k < 21; ++k) { dC[k] = R.C[k] - L.C[k]; Ch[k] = R.C[k] - c2 * dC[k]; }
-  SN_apply<float>(Ch, n, nr, X);
+  SN_apply<float>(Ch, n, n, X);
   float Ki[3][3];
   {
-    const float k00 = n[0] * X[0][0] + nr[2] * X[4][0] + nr[1] * X[5][0];
-    const float k10 = n[1] * X[1][0] + nr[2] * X[3][0] + nr[0] * X[5][0];
-    const float k20 = n[2] * X[2][0] + nr[1] * X[3][0] + nr[0] * X[4][0];
-    const float k11 = n[1] * X[1][1] + nr[2] * X[3][1] + nr[0] * X[5][1];
-    const float k21 = n[2] * X[2][1] + nr[1] * X[3][1] + nr[0] * X[4][1];
-    const float k22 = n[2] * X[2][2] + nr[1] * X[3][2] + nr[0] * X[4][2];
+    const float k00 = n[0] * X[0][0] + n[2] * X[4][0] + n[1] * X[5][0];
+    const float k10 = n[1] * X[1][0] + n[2] * X[3][0] + n[0] * X[5][0];
+    const float k20 = n[2] * X[2][0] + n[1] * X[3][0] + n[0] * X[4][0];
+    const float k11 = n[1] * X[1][1] + n[2] * X[3][1] + n[0] * X[5][1];
+    const float k21 = n[2] * X[2][1] + n[1] * X[3][1] + n[0] * X[4][1];
+    const float k22 = n[2] * X[2][2] + n[1] * X[3][2] + n[0] * X[4][2];
     inv3_sym<float>(k00, k10, k20, k11, k21, k22, Ki);
   }
-  SN_apply<float>(dC, n, nr, B);
+  SN_apply<float>(dC, n, n, B);
 #pragma unroll
   for (int I = 0; I < 6; ++I) dd[I] = R.ds[I] - L.ds[I];
-  Nt_apply<float>(n, nr, dd, w);
+  Nt_apply<float>(n, n, dd, w);
 #pragma unroll
   for (int k = 0; k < 3; ++k) u[k] = c.f(F_T + k, j) + w[k];
 #pragma unroll
@@ -335,7 +353,7 @@ __device__ __forceinline__ void condense32(const TreeDev& t, const Ctx& c, int h
 }
 
 // leaf tangent in FP32: the phase's constants or the stored mu, c, m
-__device__ __forceinline__ void leaf_tan32(const PhaseDev& ph, const float* s, LeafTan<float>& D) {
+static __device__ __forceinline__ void leaf_tan32(const PhaseDev& ph, const float* s, LeafTan<float>& D) {
   if (ph.kind == 0) {
     D.lam = ph.lamf; D.mu = ph.Gf; D.c = 0.f;
 #pragma unroll
@@ -350,7 +368,7 @@ __device__ __forceinline__ void leaf_tan32(const PhaseDev& ph, const float* s, L
 
 // the structured condensation of a bottom laminate (condense_bottom); a side passed on keeps its leaf's tangent
 template <bool CMP>
-__device__ __forceinline__ void condense32_bottom(const TreeDev& t, const Ctx& c, int h, int j,
+static __device__ __forceinline__ void condense32_bottom(const TreeDev& t, const Ctx& c, int h, int j,
                                                   const LeafTan<float>& L, const LeafTan<float>& R, bool elL, bool elR,
                                                   Sub32& o) {
   const Lam<CMP> q(t, h);
@@ -368,7 +386,7 @@ __device__ __forceinline__ void condense32_bottom(const TreeDev& t, const Ctx& c
 #pragma unroll
     for (int J = I; J < 6; ++J) {
       float v = I < 3 && J < 3 ? lam : 0.f;
-      if (I == J) v += mu2;
+      if (I == J) v += I < 3 ? mu2 : 0.5f * mu2;
       if (!elL) v -= hL * L.m[J];
       if (!elR) v -= hR * R.m[J];
       o.C[sidx(I, J)] = v;
@@ -376,8 +394,8 @@ __device__ __forceinline__ void condense32_bottom(const TreeDev& t, const Ctx& c
   }
   if (CMP && q.mode) return;
   const float c12 = __ldg(t.c12f + q.id);
-  float n[3], nr[3];
-  normal32(c, j, n, nr);
+  float n[3];
+  normal32(c, j, n);
   const float a = c2 * L.mu + c1 * R.mu, b = c2 * (L.lam + L.mu) + c1 * (R.lam + R.mu);
   const float dlam = R.lam - L.lam, dmu2 = 2.f * (R.mu - L.mu), dld = dlam + dmu2;
   float k[3][3], B[6][3];
@@ -389,10 +407,10 @@ __device__ __forceinline__ void condense32_bottom(const TreeDev& t, const Ctx& c
   for (int I = 0; I < 6; ++I)
 #pragma unroll
     for (int l = 0; l < 3; ++l)
-      B[I][l] = I < 3 ? (I == l ? dld : dlam) * n[l] : (N_nonzero(I, l) ? dmu2 * N_entry<float>(n, nr, I, l) : 0.f);
+      B[I][l] = I < 3 ? (I == l ? dld : dlam) * n[l] : (N_nonzero(I, l) ? 0.5f * dmu2 * N_entry<float>(n, n, I, l) : 0.f);
   if (!elL) {
     float v[3];
-    Nt_apply<float>(n, nr, L.m, v);
+    Nt_apply<float>(n, n, L.m, v);
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
@@ -404,7 +422,7 @@ __device__ __forceinline__ void condense32_bottom(const TreeDev& t, const Ctx& c
   }
   if (!elR) {
     float v[3];
-    Nt_apply<float>(n, nr, R.m, v);
+    Nt_apply<float>(n, n, R.m, v);
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
@@ -420,13 +438,71 @@ __device__ __forceinline__ void condense32_bottom(const TreeDev& t, const Ctx& c
   solve32(c, j, c12, Ki, B, u, o.ds, o.C);
 }
 
+// A, the leaf: stress from the strain e and the state z (shear entries times 1 / sqrt 2), the law of leaf_iso in
+// Voigt components; the tangent mu, c, m for S and B goes to T as pairs, formed in pairs from FP64 xi, 1 / |xi| and
+// k2.  An elastic leaf's tangent is its phase's.
+static __device__ __forceinline__ void leaf_a(const PhaseDev& ph, const double e[6], const double* zp, double sig[6], float* T) {
+  const double tr = e[0] + e[1] + e[2];
+  if (ph.kind == 0) {
+    const double lt = ph.lam * tr, g2 = 2.0 * ph.G;
+#pragma unroll
+    for (int I = 0; I < 6; ++I) sig[I] = I < 3 ? g2 * e[I] + lt : ph.G * e[I];
+    return;
+  }
+  double z[6];
+#pragma unroll
+  for (int k = 0; k < 6; ++k) z[k] = zp[k * BT];
+  const double twoG = 2.0 * ph.G, m3 = tr * (1.0 / 3.0);
+  const double xi[6] = {e[0] - m3 - z[1],      e[1] - m3 - z[2],      e[2] - m3 + (z[1] + z[2]),
+                        0.5 * e[3] - z[3], 0.5 * e[4] - z[4], 0.5 * e[5] - z[5]};
+  const double n2 = xi[0] * xi[0] + xi[1] * xi[1] + xi[2] * xi[2] +
+                    2.0 * (xi[3] * xi[3] + xi[4] * xi[4] + xi[5] * xi[5]);
+  const double inx = rsqrt(fmax(n2, tiny_s<double>())), ns = twoG * (n2 * inx);   // 1 / |xi|, |s_tr|
+  const bool explin = ph.kind == 2;
+  const double e_n = explin ? exp(-ph.rate * z[0]) : 1.0;
+  const double sy = ph.s0 + ph.H * z[0] + (explin ? ph.ds * (1.0 - e_n) : 0.0);
+  const double f = ns - SQ23 * sy;
+  const bool plastic = f > 0.0;
+  double dg = plastic ? f * ph.inv_den : 0.0, thb0 = ph.thb0;
+  if (explin && plastic) {   // the scalar Newton iteration of leaf_iso
+    double slope = ph.H + ph.dk * e_n, ex = e_n, step = 0.0;
+    dg = f / (twoG + (2.0 / 3.0) * slope);
+    for (int it = 0; it < 40; ++it) {
+      const double a = z[0] + SQ23 * dg;
+      ex = exp(-ph.rate * a);
+      slope = ph.H + ph.dk * ex;
+      const double r = ns - twoG * dg - SQ23 * (ph.s0 + ph.H * a + ph.ds * (1.0 - ex));
+      step = r / (twoG + (2.0 / 3.0) * slope);
+      dg += step;
+      if (fabs(step) <= 1e-10 * dg) break;
+    }
+    slope -= ph.rate * ph.dk * ex * SQ23 * step;
+    thb0 = 1.0 / (1.0 + slope / (3.0 * ph.G));
+  }
+  const double k2 = dg * inx, Kt = ph.K * tr, g2 = twoG - twoG * k2;
+#pragma unroll
+  for (int I = 0; I < 6; ++I) sig[I] = I < 3 ? g2 * xi[I] + Kt : g2 * xi[I];
+  const pair nk2 = neg(split(k2)), G = split(ph.G);
+  pair ix = split(inx);
+  if (!(ix.h < 1e37f)) ix = pair{0.f, 0.f};   // no strain: no direction (and c = 0)
+  pair v = mul(G, add(pair{1.f, 0.f}, nk2));               // mu = G (1 - k2)
+  T[0] = v.h; T[8 * BT] = v.l;
+  v = mul(pair{2.f * G.h, 2.f * G.l}, add(split(thb0), nk2));   // c = 2 G (thb0 - k2)
+  T[BT] = plastic ? v.h : 0.f; T[9 * BT] = plastic ? v.l : 0.f;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    v = mul(split(xi[k]), ix);
+    T[(2 + k) * BT] = v.h; T[(10 + k) * BT] = v.l;
+  }
+}
+
 // D e of a leaf in pairs (B): the phase's constants or the stored mu, c, m
-__device__ __forceinline__ void leaf_apply(const PhaseDev& ph, const float* s, const pair e[6], pair tau[6]) {
+static __device__ __forceinline__ void leaf_apply(const PhaseDev& ph, const float* s, const pair e[6], pair tau[6]) {
   const pair tr = add(add(e[0], e[1]), e[2]);
   if (ph.kind == 0) {
-    const pair lt = mul(split(ph.lam), tr), g2 = split(2.0 * ph.G);
+    const pair lt = mul(split(ph.lam), tr), g = split(ph.G), g2 = {2.f * g.h, 2.f * g.l};
 #pragma unroll
-    for (int I = 0; I < 6; ++I) { tau[I] = mul(g2, e[I]); if (I < 3) tau[I] = add(tau[I], lt); }
+    for (int I = 0; I < 6; ++I) tau[I] = I < 3 ? add(mul(g2, e[I]), lt) : mul(g, e[I]);
     return;
   }
   pair m[6], me;
@@ -439,42 +515,37 @@ __device__ __forceinline__ void leaf_apply(const PhaseDev& ph, const float* s, c
   const pair lt = mul(add(split(ph.K), mul(split(-2.0 / 3.0), mu)), tr);
 #pragma unroll
   for (int I = 0; I < 6; ++I) {
-    tau[I] = add(mul(g2, e[I]), mul(cm, m[I]));
+    tau[I] = add(mul(I < 3 ? g2 : mu, e[I]), mul(cm, m[I]));
     if (I < 3) tau[I] = add(tau[I], lt);
   }
 }
 
-}  // namespace
-
-// flags of a slot
-enum { B_ACT = 1, B_FIRST = 4, B_CONT = 8, B_CONV = 16, B_CUR = 32 };
-
 // Own-column accesses: a thread's vector of 6 in rows 0 .. 5 of a shared array, at column x.
 template <typename T>
-__device__ __forceinline__ void put6(T (*m)[BT], int x, const T v[6]) {
+static __device__ __forceinline__ void put6(T (*m)[BT], int x, const T v[6]) {
 #pragma unroll
   for (int I = 0; I < 6; ++I) m[I][x] = v[I];
 }
 template <typename T>
-__device__ __forceinline__ void get6(T (*m)[BT], int x, T v[6]) {
+static __device__ __forceinline__ void get6(T (*m)[BT], int x, T v[6]) {
 #pragma unroll
   for (int I = 0; I < 6; ++I) v[I] = m[I][x];
 }
-__device__ __forceinline__ void put6(float (*m)[BT], int x, const pair v[6]) {
+static __device__ __forceinline__ void put6(float (*m)[BT], int x, const pair v[6]) {
 #pragma unroll
   for (int I = 0; I < 6; ++I) { m[I][x] = v[I].h; m[6 + I][x] = v[I].l; }
 }
-__device__ __forceinline__ void get6(float (*m)[BT], int x, pair v[6]) {
+static __device__ __forceinline__ void get6(float (*m)[BT], int x, pair v[6]) {
 #pragma unroll
   for (int I = 0; I < 6; ++I) v[I] = pair{m[I][x], m[6 + I][x]};
 }
-__device__ __forceinline__ void put27(float (*m)[BT], int x, const Sub32& v) {
+static __device__ __forceinline__ void put27(float (*m)[BT], int x, const Sub32& v) {
 #pragma unroll
   for (int I = 0; I < 6; ++I) m[I][x] = v.ds[I];
 #pragma unroll
   for (int k = 0; k < 21; ++k) m[6 + k][x] = v.C[k];
 }
-__device__ __forceinline__ void get27(float (*m)[BT], int x, Sub32& v) {
+static __device__ __forceinline__ void get27(float (*m)[BT], int x, Sub32& v) {
 #pragma unroll
   for (int I = 0; I < 6; ++I) v.ds[I] = m[I][x];
 #pragma unroll
@@ -497,25 +568,33 @@ struct BlockShared {
 };
 
 // Laminate h (0-based) of the full tree of depth Kt + 3 lies with subtree thread s as its laminate j.
-__device__ __forceinline__ void owner(int h, int Kt, int& s, int& j) {
+static __device__ __forceinline__ void owner(int h, int Kt, int& s, int& j) {
   const int h1 = h + 1, d = 31 - __clz(h1) - Kt, S = 1 << Kt;
   if (d < 0) { s = h1; j = 7; }
   else { s = (h1 >> d) - S; j = (1 << d) - 1 + (h1 & ((1 << d) - 1)); }
 }
 
-// The two CTAs of an SM alternate between the FP64 phase A and the FP32 phases S and B.  Started together
-// they run in step, both in A or both out of it, and the FP64 units idle half of the time; started half a
-// round apart they stay apart (100003 points: 35.7 ms always, against 35.8 to 43 ms).  The launch's second
-// half of the CTAs lands beside the first; the wait is bounded.
-__device__ __forceinline__ void stagger() {
-  constexpr long long HALF_ROUND = 150000;   // cycles
-  if (gridDim.x < 2 || 2 * blockIdx.x < gridDim.x) return;
-  const long long t0 = clock64();
-  for (int k = 0; k < 2000 && clock64() - t0 < HALF_ROUND; ++k) __nanosleep(100);
+// The two CTAs of an SM should alternate between the FP64 phase A and the FP32 phases S and B: in step, both in A
+// or both out of it, the FP64 units idle half of the time.  A token per SM is held during A.  The wait for it is
+// bounded, and its holder waits for nothing; a CTA that gives up goes on without it (two SMs whose ids share a
+// token only wait more).  Depth 8, 200003 points: 72.8 ms always; without it 70 ms to 87 ms, also where the two
+// CTAs start half a round apart.  With several trees the rounds of an SM's CTAs differ in length and the wait
+// costs more than it orders (depths 3 to 8 with the line search: 5.9 against 5.4 ms).
+static __device__ __forceinline__ unsigned long long* token(const BlockParams& P) {
+  unsigned smid;
+  asm volatile("mov.u32 %0, %%smid;" : "=r"(smid));
+  return P.counter + 32 + (smid & (BLOCK_TOKENS - 1));
+}
+static __device__ __forceinline__ bool acquire(unsigned long long* tok) {
+  for (int k = 0; k < 500; ++k) {
+    if (atomicCAS(tok, 0ull, 1ull) == 0ull) return true;
+    __nanosleep(400);
+  }
+  return false;
 }
 
 template <bool LS, bool CMP>
-__global__ void __launch_bounds__(BT, BLOCK_CTAS_PER_SM) k_newton_block(BlockParams P) {
+static __device__ void newton(const BlockParams& P) {
   extern __shared__ __align__(16) char dyn[];
   BlockShared& M = *reinterpret_cast<BlockShared*>(dyn);
   double (*const sh_e)[BT] = M.e;
@@ -527,12 +606,14 @@ __global__ void __launch_bounds__(BT, BLOCK_CTAS_PER_SM) k_newton_block(BlockPar
   long long* const sh_pt = M.pt;
   int* const sh_fl = M.fl;
   float* const sh_st = M.st;
-  const int tid = threadIdx.x, lane = tid & 31;
+  const int tid = threadIdx.x;
   const size_t n = (size_t)P.n;
+  unsigned long long* const tok = token(P);
+  bool own = false;
   Ctx c;
   double *D0, *z0;
   {
-    char* base = P.scratch + (size_t)blockIdx.x * block_scratch_bytes(P.leaf_slots, LS);
+    char* base = P.scratch + (size_t)blockIdx.x * block_scratch_bytes(BT, P.leaf_slots, LS);
     double* D = (double*)base;
     D0 = D;
     z0 = D + (size_t)8 * (LS ? 9 : 6) * BT;
@@ -557,11 +638,11 @@ __global__ void __launch_bounds__(BT, BLOCK_CTAS_PER_SM) k_newton_block(BlockPar
     auto heap = [&](int j) { return (j == 0 ? R1 : j < 3 ? 2 * R1 + j - 1 : j < 7 ? 4 * R1 + j - 3 : s) - 1; };
     // a subtree with nothing alive in it is skipped (its results are never used, only kept finite)
     const bool dead = CMP && __ldg(t.hdir + heap(0)) == 3;
-    if (tr == 0) stagger();
     // state of slot p, kept by thread p < nP
     long long pt = -1;
     int it = 0, halv = 0, np = 0;
-    double rn_acc = 0.0;
+    double rn_acc = 0.0, left = 0.0;
+    bool again = false;   // a step in two parts (LEFT_MAX)
     bool more = tid < nP;
     if (tid < nP) sh_fl[tid] = 0;
     if (tid == 0) M.n_in = 0;
@@ -575,7 +656,7 @@ __global__ void __launch_bounds__(BT, BLOCK_CTAS_PER_SM) k_newton_block(BlockPar
           int64_t x;
           point_of(P.perm, P.tid, P.F.n, (int64_t)i, x, tt);
           if (tt == tr) {
-            pt = x; it = 0; halv = 0; np = 0; rn_acc = 0.0;
+            pt = x; it = 0; halv = 0; np = 0; rn_acc = 0.0; left = 0.0; again = false;
             sh_pt[tid] = pt; sh_st[tid] = 1.f;
             sh_fl[tid] = B_ACT | B_FIRST;
             M.in[atomicAdd(&M.n_in, 1)] = (short)tid;
@@ -611,10 +692,14 @@ __global__ void __launch_bounds__(BT, BLOCK_CTAS_PER_SM) k_newton_block(BlockPar
           const int l = leaf & 7;
           double* w = z0 + (6 * (both ? l : l >> 1)) * BT + (leaf >> 3) * nP + x;
 #pragma unroll
-          for (int k = 0; k < 6; ++k) w[k * BT] = slot >= 0 ? __ldg(P.state_in + (6 * slot + k) * n + q) : 0.0;
+          for (int k = 0; k < 6; ++k)
+            w[k * BT] = slot >= 0 ? (k < 3 ? 1.0 : RS2) * __ldg(P.state_in + (6 * slot + k) * n + q) : 0.0;
         }
       }
-      if (tid == 0) M.n_out = 0;
+      if (tid == 0) {
+        M.n_out = 0;
+        own = P.F.n == 1 && acquire(tok);
+      }
       const bool act = fl & B_ACT, apply = act && !(fl & B_FIRST);
       const int a_in = LS && (fl & B_CUR) ? D_A2 : D_A, a_out = LS ? (a_in == D_A ? D_A2 : D_A) : D_A;
       const double step = LS ? (double)sh_st[p] : 1.0;
@@ -622,7 +707,10 @@ __global__ void __launch_bounds__(BT, BLOCK_CTAS_PER_SM) k_newton_block(BlockPar
       float(*sd)[BT] = sh_c;
       if (act && s == 0) {
 #pragma unroll
-        for (int I = 0; I < 6; ++I) { sh_e[I][p] = P.nbuf[(3 * P.N_max + I) * n + mypt]; sd[I][p] = 0.f; }
+        for (int I = 0; I < 6; ++I) {
+          sh_e[I][p] = (I < 3 ? 1.0 : 1.41421356237309504880) * P.nbuf[(3 * P.N_max + I) * n + mypt];
+          sd[I][p] = 0.f;
+        }
       }
       __syncthreads();
       for (int l = 0; l < Kt; ++l) {
@@ -659,27 +747,11 @@ __global__ void __launch_bounds__(BT, BLOCK_CTAS_PER_SM) k_newton_block(BlockPar
             for (int I = 0; I < 6; ++I) { e[I] = eL[I]; de[I] = dL[I]; }
           }
           down_a<CMP, LS>(t, c, heap(3 + q), 3 + q, a_in, a_out, apply, step, e, de, eL, eR, nullptr, nullptr);
-          double z[6], s0[6], s1[6];
+          double s0[6], s1[6];
 #pragma unroll
           for (int side = 0; side < 2; ++side) {
             const int ls = both ? 2 * q + side : q;
-            const bool el = t.ph[side].kind == 0;
-#pragma unroll
-            for (int k = 0; k < 6; ++k) z[k] = el ? 0.0 : c.z[(6 * ls + k) * BT];
-            LeafTan<double> D;
-            leaf_iso<double, double>(t.ph[side], side ? eR : eL, z, side ? s1 : s0, &D, nullptr, nullptr);
-            if (!el) {
-              float* T = c.tan + 16 * ls * BT;
-              pair v = split(D.mu);
-              T[0] = v.h; T[8 * BT] = v.l;
-              v = split(D.c);
-              T[BT] = v.h; T[9 * BT] = v.l;
-#pragma unroll
-              for (int k = 0; k < 6; ++k) {
-                v = split(D.m[k]);
-                T[(2 + k) * BT] = v.h; T[(10 + k) * BT] = v.l;
-              }
-            }
+            leaf_a(t.ph[side], side ? eR : eL, c.z + 6 * ls * BT, side ? s1 : s0, c.tan + 16 * ls * BT);
           }
           up_a<CMP>(t, c, heap(3 + q), 3 + q, s0, s1, sb, r2);
           if (!(q & 1)) {
@@ -716,22 +788,23 @@ __global__ void __launch_bounds__(BT, BLOCK_CTAS_PER_SM) k_newton_block(BlockPar
         }
         __syncthreads();
       }
-      // sum of the point's shares in a fixed order: the warp's lanes of one slot, then the warps
-      for (int o = 16; o >= nP; o >>= 1) r2 += __shfl_xor_sync(0xffffffffu, r2, o);
-      const int groups = nP < 32 ? BT / 32 : S;
-      if (nP >= 32) sh_r[tid] = r2;
-      else if (lane < nP) sh_r[(tid >> 5) * nP + lane] = r2;
+      // sum of the point's shares in an order that does not depend on BT: 2^nb neighbouring subtrees by shuffles
+      // (as many as a warp of the large CTA holds), then the groups in turn
+      const int nb = Kt > 3 ? Kt - 3 : 0, groups = S >> nb;
+      for (int b = nb - 1; b >= 0; --b) r2 += __shfl_xor_sync(0xffffffffu, r2, nP << b);
+      if (!(s & ((1 << nb) - 1))) sh_r[(s >> nb) * nP + p] = r2;
       __syncthreads();
+      if (own) { own = false; atomicExch(tok, 0ull); }
       double rn = 0.0;
       if (tid < nP && (sh_fl[tid] & B_ACT)) {
         double r = 0.0, sn2 = 0.0;
         for (int k = 0; k < groups; ++k) r += sh_r[k * nP + tid];
         rn = sqrt(r);
 #pragma unroll
-        for (int I = 0; I < 6; ++I) sn2 += sh_e[I][tid] * sh_e[I][tid];
+        for (int I = 0; I < 6; ++I) sn2 += (I < 3 ? 1.0 : 2.0) * sh_e[I][tid] * sh_e[I][tid];
         const double sn = sqrt(sn2);
         int f = sh_fl[tid] & (B_ACT | B_FIRST | B_CUR);
-        ++np;
+        if (!again) ++np;
         bool retry = false;
         int st = -1;   // the point's status once it is done
         const bool ok = !LS || (f & B_FIRST) || rn < rn_acc;
@@ -741,9 +814,10 @@ __global__ void __launch_bounds__(BT, BLOCK_CTAS_PER_SM) k_newton_block(BlockPar
           f &= ~B_FIRST;
           if (!isfinite(rn) || !isfinite(sn)) retry = true;
           else if (rn <= P.tol * (double)t.N * sn) st = DMN_STATUS_OK;
+          else if (!again && rn <= LEFT_MAX * left) { again = true; f |= B_CONT; }
           else if (it >= P.max_iter) st = DMN_STATUS_MAXITER;
           else if (it >= BLOCK_ITERS) retry = true;
-          else { ++it; f |= B_CONT; }
+          else { ++it; again = false; f |= B_CONT; }
         } else if (++halv > 8) {
           st = DMN_STATUS_LINESEARCH;   // no halving lowered the residual: the accepted iterate stands
           ++it;
@@ -816,7 +890,7 @@ __global__ void __launch_bounds__(BT, BLOCK_CTAS_PER_SM) k_newton_block(BlockPar
         }
         __syncthreads();
       }
-      // ---- B: da1 down, J da1 up (pairs), second FP32 solve up
+      // ---- B: the step down, J times it up (pairs), the second FP32 solve up
       if (cont && s == 0) {
 #pragma unroll
         for (int I = 0; I < 12; ++I) sh_p[I][p] = 0.f;
@@ -900,18 +974,22 @@ __global__ void __launch_bounds__(BT, BLOCK_CTAS_PER_SM) k_newton_block(BlockPar
         }
         __syncthreads();
       }
-      for (int o = 16; o >= nP; o >>= 1) q2 += __shfl_xor_sync(0xffffffffu, q2, o);
-      if (nP >= 32) sh_r[tid] = (double)q2;
-      else if (lane < nP) sh_r[(tid >> 5) * nP + lane] = (double)q2;
+      for (int b = nb - 1; b >= 0; --b) q2 += __shfl_xor_sync(0xffffffffu, q2, nP << b);
+      if (!(s & ((1 << nb) - 1))) sh_r[(s >> nb) * nP + p] = (double)q2;
       __syncthreads();
       if (tid < nP) {
-        int f = sh_fl[tid];
+        int f = sh_fl[tid] & ~B_CONV;
         if (f & B_CONT) {
           double r = 0.0;
           for (int k = 0; k < groups; ++k) r += sh_r[k * nP + tid];
-          if (!(r <= (double)REFINE_MAX * REFINE_MAX * rn_acc * rn_acc)) { block_retry(P, pt); f = 0; }
+          r = sqrt(r);                 // of the linear residual; the second solve leaves about r / rn_acc of it
+          left = r * (r / rn_acc);
+          if (!(r <= (double)REFINE_MAX * rn_acc)) {
+            block_retry(P, pt);
+            f = 0;
+          }
         }
-        sh_fl[tid] = f & ~(B_CONT | B_CONV);
+        sh_fl[tid] = f;
       }
     }
     __syncthreads();
@@ -923,6 +1001,13 @@ __global__ void __launch_bounds__(BT, BLOCK_CTAS_PER_SM) k_newton_block(BlockPar
          i += (unsigned long long)gridDim.x * BT)
       block_bad_tree(P, P.perm[i]);
   }
+}
+
+};
+
+template <int BT, bool LS, bool CMP>
+__global__ void __launch_bounds__(BT, BLOCK_THREADS * BLOCK_CTAS_PER_SM / BT) k_newton_block(BlockParams P) {
+  Block<BT>::template newton<LS, CMP>(P);
 }
 
 // ---------------------------------------------------------------------------
@@ -1164,20 +1249,33 @@ cudaError_t launch_sweep_block(const SweepParams& P, bool cmp, bool states, unsi
   return states ? sweep<false, true>(P, grid, s) : sweep<false, false>(P, grid, s);
 }
 
-template <bool LS, bool CMP>
+template <int BT, bool LS, bool CMP>
 static cudaError_t launch(const BlockParams& P, unsigned grid, cudaStream_t s) {
-  const cudaError_t e = cudaFuncSetAttribute(k_newton_block<LS, CMP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)sizeof(BlockShared));
+  const int bytes = (int)sizeof(typename Block<BT>::BlockShared);
+  const cudaError_t e = cudaFuncSetAttribute(k_newton_block<BT, LS, CMP>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e != cudaSuccess) return e;
-  k_newton_block<LS, CMP><<<grid, BT, sizeof(BlockShared), s>>>(P);
+  k_newton_block<BT, LS, CMP><<<grid, BT, bytes, s>>>(P);
   return cudaSuccess;
 }
+template <int BT>
+static cudaError_t launch(const BlockParams& P, bool ls, bool cmp, unsigned grid, cudaStream_t s) {
+  if (ls && cmp) return launch<BT, true, true>(P, grid, s);
+  if (ls) return launch<BT, true, false>(P, grid, s);
+  if (cmp) return launch<BT, false, true>(P, grid, s);
+  return launch<BT, false, false>(P, grid, s);
+}
 
-cudaError_t launch_block(const BlockParams& P, bool ls, bool cmp, unsigned grid, cudaStream_t s) {
-  if (ls && cmp) return launch<true, true>(P, grid, s);
-  if (ls) return launch<true, false>(P, grid, s);
-  if (cmp) return launch<false, true>(P, grid, s);
-  return launch<false, false>(P, grid, s);
+// K: the depth of the handle's deepest tree.  A call that gives every SM at most one CTA of 256 threads runs in
+// CTAs of 128, a warp per FP64 unit instead of two (8 points of depth 8: 0.58 -> 0.42 ms).  With more points the
+// larger CTA is ahead (100003 points: 36 against 43 ms), whose top levels lie on more warps.
+cudaError_t launch_block(const BlockParams& P, int K, bool ls, bool cmp, cudaStream_t s) {
+  const int64_t big = (P.n + (BLOCK_THREADS >> (K - 3)) - 1) / (BLOCK_THREADS >> (K - 3));
+  if (big <= P.n_sm) {
+    constexpr int SMALL = BLOCK_THREADS / 2;
+    return launch<SMALL>(P, ls, cmp, (unsigned)((P.n + (SMALL >> (K - 3)) - 1) / (SMALL >> (K - 3))), s);
+  }
+  const int64_t most = (int64_t)P.n_sm * BLOCK_CTAS_PER_SM;
+  return launch<BLOCK_THREADS>(P, ls, cmp, (unsigned)(big < most ? big : most), s);
 }
 
 }  // namespace dmn

@@ -87,10 +87,11 @@ void launch_warp(const NewtonParams<T>& P, bool ls, int lanes, unsigned grid, do
 // [10..18] their ends in perm (several trees), [21..28] work counters per tree, [29] points on the list.
 constexpr int BLOCK_THREADS = 256;
 constexpr int BLOCK_CTAS_PER_SM = 2;
+constexpr int BLOCK_TOKENS = 256;   // counters [32 ..]: an SM's FP64 phase is taken
 struct BlockParams {
   Forest F;
   int64_t n;
-  int N_max, leaf_slots;   // leaf_slots: leaves with a state in a subtree of 8 (4, or 8 with two inelastic phases)
+  int N_max, n_sm, leaf_slots;   // leaf_slots: leaves with a state in a subtree of 8 (4, or 8 with two inelastic phases)
   const int32_t* tid;
   const int64_t* perm;
   const double* state_in;
@@ -106,8 +107,8 @@ struct BlockParams {
 };
 // per thread, for 8 laminates: jumps (two buffers with the line search) and normals (FP64), H, Kn^-1, g, step
 // and residual (FP32: 36 fields); per leaf its state (FP64: 6) and tangent (FP32: 16)
-__host__ __device__ inline size_t block_scratch_bytes(int leaf_slots, bool line_search) {
-  return (size_t)BLOCK_THREADS * (sizeof(double) * (8 * (line_search ? 9 : 6) + 6 * leaf_slots) +
+__host__ __device__ inline size_t block_scratch_bytes(int threads, int leaf_slots, bool line_search) {
+  return (size_t)threads * (sizeof(double) * (8 * (line_search ? 9 : 6) + 6 * leaf_slots) +
                                   sizeof(float) * (8 * 36 + 16 * leaf_slots));
 }
 __device__ __forceinline__ void block_bad_tree(const BlockParams& P, int64_t pt) {
@@ -138,7 +139,8 @@ struct SweepParams {
   const unsigned long long* counter;
 };
 cudaError_t launch_sweep_block(const SweepParams& P, bool cmp, bool states, unsigned grid, cudaStream_t s);
-cudaError_t launch_block(const BlockParams& P, bool ls, bool cmp, unsigned grid, cudaStream_t s);
+// K: the depth of the handle's deepest tree; scratch for BLOCK_CTAS_PER_SM CTAs of BLOCK_THREADS per SM
+cudaError_t launch_block(const BlockParams& P, int K, bool ls, bool cmp, cudaStream_t s);
 
 // The adjoints in the CTA organisation (csrc/dmn_grad.cu): one chunk of nc points from n0 on.  work, field-major
 // over the chunk: normals [3 N], sin(alpha), cos(beta), sin(beta) [3 N], dL/d alpha [N], dL/d beta [N], dL/dw [L],

@@ -126,3 +126,40 @@ def test_points_the_fp32_solve_cannot_take_go_to_the_fp64_kernels(n):
     o = m.update(d(lam), d(Q), torch.zeros_like(d(E)), d(E), torch.zeros((m.state_size, n), dtype=torch.float64, device=DEV))
     stat, it = o["status"].cpu().numpy(), o["iters"].cpu().numpy()
     assert (stat[ok] == dmn.STATUS_MAXITER).all() and (it[ok] == 1).all()
+
+
+@pytest.mark.parametrize("K,n", [(3, 9), (5, 37), (7, 21), (8, 41)])
+def test_a_small_calls_smaller_ctas_give_the_same_bits(K, n):
+    """At most as many 256-thread CTAs as SMs: CTAs of 128 threads.  The same points at the head of a larger call
+    run in CTAs of 256."""
+    n_sm = torch.cuda.get_device_properties(DEV).multi_processor_count
+    big = n_sm * (256 >> (K - 3)) + 1
+    tree = W.tree_d10_fit(K, seed=760 + K, phases=(W.FIBER, W.MATRIX_EXPLIN))
+    lam, Q, Ef = inputs(big, 761)
+    m = dmn.DMN(tree)
+    outs = []
+    for k in (big, n):
+        z = torch.zeros((m.state_size, k), dtype=torch.float64, device=DEV)
+        outs.append(m.update(d(lam[:k]), d(Q[:k]), torch.zeros_like(d(Ef[:k])), d(Ef[:k] * 0.2), z))
+    for k in ("stress", "tangent", "iters", "status"):
+        assert torch.equal(outs[0][k][:n], outs[1][k]), k
+    assert torch.equal(outs[0]["state_out"][:, :n], outs[1]["state_out"])
+
+
+def test_iteration_counts_on_large_steps():
+    """Increments whose last Newton step is large (it ends in a fixed set of plastic leaves, so that no quadratic
+    term follows): what the FP32 solves leave of the linear residual must not show in the criterion."""
+    import oracle
+    n = 400
+    lam, Q, Ef = inputs(n, 770, eps=0.02)
+    for K in (5, 6, 8):
+        tree = W.tree_d10_fit(K, seed=300 + K)
+        m = dmn.DMN(tree)
+        for scale in (0.0005, 0.25):
+            st = np.zeros((m.state_size, n))
+            _, sig, C, it, stat, gap = oracle.update(tree, lam, Q, np.zeros_like(Ef), scale * Ef, st)
+            o = m.update(d(lam), d(Q), torch.zeros_like(d(Ef)), d(scale * Ef), d(st))
+            ok = (stat == 0) & (o["status"].cpu().numpy() == 0)
+            assert (stat != o["status"].cpu().numpy()).sum() == 0
+            np.testing.assert_array_equal(o["iters"].cpu().numpy()[ok], it[ok])
+            assert rel(o["stress"].cpu().numpy()[ok], sig[ok]).max() <= 1e-10
