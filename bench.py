@@ -177,6 +177,16 @@ def newton_flops(K, iters_sum, npts, mixed, w=None):
     return (F64, FT) if mixed else (F64 + FT, 0.0)
 
 
+def block_flops(K, iters_sum, npts, w=None):
+    """(FP64, FP32) flops of k_newton_block over npts points with iters_sum corrections: FP64 strains, leaf
+    laws and residuals in every pass; per correction the FP32 condensation, the residual of its linear system
+    (strains, leaf tangents and tractions, counted once although they run in pairs of FP32 numbers) and two
+    FP32 solves."""
+    f64, ft = pass_flops(K, w, t_is_f64=False)
+    c64, ct = corr_flops(K, w)
+    return (iters_sum + npts) * f64 + iters_sum * c64, iters_sum * (ft + f64 + 2 * ct)
+
+
 def final_flops(K, npts, sweep, w=None):
     """FP64 flops of the final kernel (state pass and rotation; mixed form: plus one FP64 pass)."""
     c = tree_counts(np.ones(1 << K) if w is None else w)
@@ -189,7 +199,8 @@ def final_flops(K, npts, sweep, w=None):
 
 # ---------------------------------------------------------------------------------------------
 SRC_FILES = ("paper_2103_08253_gb300/csrc/dmn.cu", "paper_2103_08253_gb300/csrc/dmn_device.cuh",
-             "paper_2103_08253_gb300/csrc/dmn_warp.cu", "paper_2103_08253_gb300/csrc/dmn_launch.cuh")
+             "paper_2103_08253_gb300/csrc/dmn_warp.cu", "paper_2103_08253_gb300/csrc/dmn_launch.cuh",
+             "paper_2103_08253_gb300/csrc/dmn_block.cu", "paper_2103_08253_gb300/csrc/dmn_block.cuh")
 
 
 def code_only(text):
@@ -482,15 +493,19 @@ def run_form(form, ctx, args, dist):
     clk = clocks.stop() if clocks else None
     kms, passes, cnt = m.profile_read_stages()
     m.profile(False)
-    lanes = m.lanes_per_point(n)   # a small call runs the warp organisation, without the first stage
-    warp = lanes > 1
+    # the FP64 form from depth 3 on runs k_newton_block at every size; of the others a small call runs the warp
+    # organisation, without the first stage
+    block = m.precision == "f64" and not m.predictor and not m.first_stage and K_DEPTH >= 3
+    lanes = m.lanes_per_point(n)
+    warp = lanes > 1 and not block
     if not form_stage(form) or warp:
         kms.pop("stage")
     its = iters_steps.to(torch.int64).sum().item()
     hist = torch.bincount(iters_steps.reshape(-1).to(torch.int64), minlength=1).cpu().numpy()
     res = dict(t_ms=t_ms, kms=kms, updates=cnt, clocks=clk, iters_sum=int(its), iters_hist=hist.tolist(),
-               passes=passes, warp=warp,
-               launch=("%d lanes per point (k_newton_warp, 2 CTAs of 4 warps per SM)" % lanes if warp else
+               passes=passes, warp=warp, block=block,
+               launch=("CTAs of 256 threads, %d per point (k_newton_block)" % (1 << (K_DEPTH - 3)) if block else
+                       "%d lanes per point (k_newton_warp, 2 CTAs of 4 warps per SM)" % lanes if warp else
                        dict(block=shape["block"], ctas_per_sm=shape["ctas_per_sm"], tuned_on_points=shape["points"],
                             table=shape["table"], stage_ctas_per_sm=shape["stage_ctas_per_sm"],
                             stage_table=shape["stage_table"]) if shape else "defaults"),
@@ -591,6 +606,21 @@ def roofline_f64(r, n, steps, w=None, peaks=None):
     npts = n * steps
     passes = r.get("passes") or {}
     corr = passes["newton"] - npts if passes.get("newton") else r["iters_sum"]
+    if r.get("block"):
+        F64, F32 = block_flops(K_DEPTH, corr, npts, w=w)
+        t = r["kms"]["newton"] * 1e-3
+        tb = F64 / (P64 * 1e9) + F32 / (pk["f32"] * 1e9)
+        Ff = final_flops(K_DEPTH, npts, sweep=True, w=w)
+        tf = r["kms"]["final"] * 1e-3
+        cmp = "_compressed" if w is not None and (np.asarray(w) == 0).any() else ""
+        return {"bound": "alu", "kernel": "k_newton_block", "achieved": tb / t * P64, "peak": P64,
+                "unit": "GFLOP/s (FP64-equivalent: F64/P64 + F32/P32)", "frac": tb / t,
+                "traffic": ncu_traffic("k_newton_block" + cmp, n), "flops_f64_per_launch": F64 / steps,
+                "flops_f32_per_launch": F32 / steps, "launch_ms": r["kms"]["newton"] / steps,
+                "peak_note": pk["note"], "passes_per_update": (corr + npts) / npts,
+                "final_kernel": {"kernel": "k_sweep_block", "achieved": Ff / tf / 1e9, "peak": P64,
+                                 "unit": "GFLOP/s (FP64)", "frac": Ff / tf / 1e9 / P64,
+                                 "launch_ms": r["kms"]["final"] / steps}}
     F, _ = newton_flops(K_DEPTH, corr, npts, mixed=False, w=w)
     t = r["kms"]["newton"] * 1e-3
     ach = F / t / 1e9
@@ -632,7 +662,7 @@ def roofline_mixed(r, n, steps, w=None, sweep=True, peaks=None):
     tb = F64 / (P64 * 1e9) + F32 / (P32 * 1e9)
     Ff = final_flops(K_DEPTH, n * steps, sweep=sweep, w=w)
     tf = r["kms"]["final"] * 1e-3
-    fin = {"kernel": "k_final<sweep>" if sweep else "k_final", "achieved": Ff / tf / 1e9, "peak": P64,
+    fin = {"kernel": "k_sweep_block, k_final" if sweep else "k_final", "achieved": Ff / tf / 1e9, "peak": P64,
            "unit": "GFLOP/s (FP64)", "frac": Ff / tf / 1e9 / P64, "launch_ms": r["kms"]["final"] / steps}
     cmp = "_compressed" if w is not None and (np.asarray(w) == 0).any() else ""
     stg = "stage" in r["kms"]
@@ -1008,7 +1038,7 @@ def run_gpu(args):
                              % (state_fields(tree) * n * 8e-6),
                        "parallelism": "independent point shards per GPU, no collective"},
             "roofline": forms_out[main_form]["roofline"], "cpu_baseline": cpu, "e2e": e2e,
-            "gpu_launches": (4 + ("stage" in mr["kms"]) + (bool(mr.get("warp")) and main_form.split("/")[0] == "mixed"))
+            "gpu_launches": (4 + ("stage" in mr["kms"]) + (main_form.split("/")[0] == "mixed") + 2 * bool(mr.get("block")))
                             * steps, "clocks": mr["clocks"],
             "peaks": {"fp64_gflops": peaks["f64"], "fp32_gflops": peaks["f32"], "note": peaks["note"]}}
     # the other forms side by side with the headline: value, roofline and error against the oracle

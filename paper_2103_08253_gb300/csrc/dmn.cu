@@ -1,19 +1,21 @@
 // Kernels and C ABI of the batched DMN material-point update (include/dmn.h).
 //
-// Per update three kernels run on the caller's stream:
-//   k_prepare  one thread per point: lamination normals of every laminate from
+// Per update these kernels run on the caller's stream:
+//   k_prepare  one thread per point (small calls: several): lamination normals of every laminate from
 //              the orientation (barycentric coordinates, shape functions,
 //              interpolated angles, spherical normal; Sec. 2.3) and the macro
 //              strain in the principal frame;
-//   k_newton   persistent, one thread per point slot: the Newton loop of
-//              Sec. 3.2.  A lane that converges writes its results and takes
-//              the next point from a global counter at once, so lanes stay busy
-//              although points need different numbers of Newton steps;
-//   k_final    one thread per point: the return mapping at the converged jumps
-//              writes z^{n+1}, and stress and tangent are rotated back to the
-//              global frame; in the mixed form this kernel first runs the FP64
-//              sweep that yields them (the form with an FP32 tangent skips it
-//              and rotates what the last Newton pass condensed).
+//   the Newton iteration of Sec. 3.2.  FP64 form, depth 3 and more: k_newton_block
+//              (csrc/dmn_block.cu), then k_newton or k_newton_warp on the points it hands back.
+//              Otherwise k_newton, persistent, one thread per point slot -- a lane that converges
+//              takes the next point from a global counter at once, so lanes stay busy
+//              although points need different numbers of Newton steps -- or, for small calls,
+//              k_newton_warp (csrc/dmn_warp.cu);
+//   k_sweep_block  (FP64 and mixed form, depth 3 and more) stress and tangent by one FP64
+//              condensation at the converged jumps, rotated back to the global frame;
+//   k_final    one thread per point (small calls: several), for what the sweep does not write: the
+//              return mapping at the converged jumps gives z^{n+1}, and stress and tangent are rotated back
+//              to the global frame; below depth 3 the mixed form's FP64 sweep runs here.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -1403,7 +1405,7 @@ int update_on(dmn_handle* h, WorkSet& w, int64_t n, int64_t n_call, const int32_
     cudaEventRecord(ev[0], s);
   }
   // counters: [0] work, [1..9] points per tree, [10..18] cursors, [19] first stage,
-  // [21..29] the CTA organisation
+  // [21..29] the CTA organisation, [32..] its tokens
   e = cudaMemsetAsync(w.counter, 0, sizeof(unsigned long long) * (32 + BLOCK_TOKENS), s);
   if (e != cudaSuccess) return cuda_fail(h, e, "dmn_update: counter reset");
   const int64_t* perm = nullptr;
