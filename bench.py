@@ -105,6 +105,7 @@ F_STATE_NODE = 39       # state pass: per laminate (strains from the jumps)
 F_STATE_J2 = 68         # state pass: per J2 leaf (return mapping and new state)
 
 
+SWEEP_BLOCK_MAX = 4096 * 152   # points up to which the mixed form's sweep is a kernel of its own
 F_LEAF_SUB = 84         # a leaf whose sibling is a laminate: its 21 tangent entries as a subtree (T)
 
 
@@ -662,7 +663,7 @@ def roofline_mixed(r, n, steps, w=None, sweep=True, peaks=None):
     tb = F64 / (P64 * 1e9) + F32 / (P32 * 1e9)
     Ff = final_flops(K_DEPTH, n * steps, sweep=sweep, w=w)
     tf = r["kms"]["final"] * 1e-3
-    fin = {"kernel": "k_sweep_block, k_final" if sweep else "k_final", "achieved": Ff / tf / 1e9, "peak": P64,
+    fin = {"kernel": ("k_sweep_block, k_final" if n <= SWEEP_BLOCK_MAX else "k_final<sweep>") if sweep else "k_final", "achieved": Ff / tf / 1e9, "peak": P64,
            "unit": "GFLOP/s (FP64)", "frac": Ff / tf / 1e9 / P64, "launch_ms": r["kms"]["final"] / steps}
     cmp = "_compressed" if w is not None and (np.asarray(w) == 0).any() else ""
     stg = "stage" in r["kms"]
@@ -1038,7 +1039,8 @@ def run_gpu(args):
                              % (state_fields(tree) * n * 8e-6),
                        "parallelism": "independent point shards per GPU, no collective"},
             "roofline": forms_out[main_form]["roofline"], "cpu_baseline": cpu, "e2e": e2e,
-            "gpu_launches": (4 + ("stage" in mr["kms"]) + (main_form.split("/")[0] == "mixed") + 2 * bool(mr.get("block")))
+            "gpu_launches": (4 + ("stage" in mr["kms"]) + (main_form.split("/")[0] == "mixed" and n <= SWEEP_BLOCK_MAX)
+                             + 2 * bool(mr.get("block")))
                             * steps, "clocks": mr["clocks"],
             "peaks": {"fp64_gflops": peaks["f64"], "fp32_gflops": peaks["f32"], "note": peaks["note"]}}
     # the other forms side by side with the headline: value, roofline and error against the oracle

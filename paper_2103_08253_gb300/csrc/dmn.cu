@@ -1350,6 +1350,12 @@ void launch_newton(const NewtonParams<T>& P, bool ls, int minb, unsigned grid, i
   else launch_newton_p<T, CMP, false>(P, ls, minb, grid, block, s);
 }
 
+// Points per SM up to which the mixed form's sweep runs k_sweep_block and a pass of k_final for the leaf states.
+// Above, k_final<sweep> does both in one pass, and its last wave is short beside the others: 100003 points of depth 8
+// 20.3 against 22.4 ms, 200003 40.3 against 41.0, 2^20 208 against 200 ms.  The whole call's size decides, so that
+// the chunks of dmn_update_host get what dmn_update gets.
+constexpr int SWEEP_BLOCK_MAX = 4096;
+
 // CTAs of 32 threads per SM for a call of n points in the thread-per-point organisation, of at most `warps` per
 // SM, or 0 for the full shape.  With the full shape a call of one to two points per lane ends with its last
 // points spread thinly over all warps, each as slow as a full one: fewer lanes, evenly used, are faster.  FP32
@@ -1494,7 +1500,7 @@ int update_on(dmn_handle* h, WorkSet& w, int64_t n, int64_t n_call, const int32_
     P.n_list = FP.n_list = w.counter + 29;
     newton_f64(P);
     final_pass(FP, false);
-  } else if (sweep && block_trees(h)) {
+  } else if (sweep && block_trees(h) && n_call <= (int64_t)SWEEP_BLOCK_MAX * h->n_sm) {
     e = sweep_pass(false);
     if (e != cudaSuccess) return cuda_fail(h, e, "dmn_update: launch");
     FP.states_only = 1;
