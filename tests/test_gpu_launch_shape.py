@@ -25,3 +25,24 @@ def test_results_do_not_depend_on_the_shape(prec, compressed, rows, extra):
         outs.append(m.update(lam, Q, torch.zeros_like(Ef), Ef * 0.2, st))
     for k, v in outs[0].items():
         assert torch.equal(v, outs[1][k]), k
+
+
+@pytest.mark.parametrize("compressed", [False, True])
+def test_the_mixed_sweep_above_and_below_its_size_limit(compressed):
+    """4096 points per SM run the CTA organisation's sweep, one more the fused final kernel: the same jumps and
+    leaf states bit for bit, stress and tangent to the rounding of two FP64 condensations of depth 3."""
+    n = 4096 * torch.cuda.get_device_properties(DEV).multi_processor_count + 1
+    tree = (W.tree_with_zero_weights if compressed else W.tree_d10_fit)(3, seed=810)
+    lam, Q, Ef = (d(x) for x in inputs(1024, 811))
+    lam, Q, dE = (x.repeat(n // 1024 + 1, 1)[:n].contiguous() for x in (lam, Q, Ef * 0.2))
+    m = dmn.DMN(tree, precision="mixed")
+    outs = []
+    for k in (n - 1, n):
+        st = torch.zeros((m.state_size, k), dtype=torch.float64, device=DEV)
+        o = m.update(lam[:k], Q[:k], torch.zeros_like(dE[:k]), dE[:k], st)
+        outs.append({key: (v[:, :1024] if key == "state_out" else v[:1024]).clone() for key, v in o.items()})
+    for key in ("state_out", "iters", "status"):
+        assert torch.equal(outs[0][key], outs[1][key]), key
+    for key in ("stress", "tangent"):
+        a, b = (o[key].reshape(1024, -1) for o in outs)
+        assert ((a - b).norm(dim=1) <= 1e-12 * b.norm(dim=1)).all(), key
