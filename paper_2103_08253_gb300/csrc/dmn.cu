@@ -772,9 +772,10 @@ struct FinalParams {
   int states_only = 0;     // stress and tangent are done (k_sweep_block)
 };
 
-// Without the sweep a point may be split over gridDim.y = 2^s threads (final_split), each of which takes
-// the leaves below one position of level s + 1; the first also rotates stress and tangent.
-template <bool SWEEP, bool CMP>
+// SPLIT (without the sweep): a point is split over gridDim.y = 2^s threads (final_split), each of which takes
+// the leaves below one position of level s + 1; the first also rotates stress and tangent.  An instantiation
+// of its own: in one kernel with the whole walk it cost that walk 3 to 6 %.
+template <bool SWEEP, bool CMP, bool SPLIT>
 __global__ void __launch_bounds__(128) k_final(FinalParams P) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= (int64_t)n_work(P.n, P.n_list)) return;
@@ -784,8 +785,8 @@ __global__ void __launch_bounds__(128) k_final(FinalParams P) {
   if (tr >= P.F.n) return;  // unknown tree: reported by the Newton kernel
   if (P.status[pt] == STATUS_RETRY) return;
   const TreeDev& t = P.F.t[tr];
-  const int part = SWEEP ? 0 : blockIdx.y, split = SWEEP ? 0 : min(31 - __clz((int)gridDim.y), t.K - 1);
-  if (part >> split) return;   // a shallower tree has fewer parts
+  const int part = SPLIT ? blockIdx.y : 0, split = SPLIT ? min(31 - __clz((int)gridDim.y), t.K - 1) : 0;
+  if (SPLIT && part >> split) return;   // a shallower tree has fewer parts
   const int st = P.status[pt];
   double Eloc[6];
 #pragma unroll
@@ -818,7 +819,7 @@ __global__ void __launch_bounds__(128) k_final(FinalParams P) {
     for (int k = 0; k < 21; ++k) C[k] = P.tangent[36 * pt + k];
     write_stress_tangent<double>(P.Q + 9 * pt, sb, C, P.stress + 6 * pt, P.tangent + 36 * pt);
   }
-  if (!SWEEP && split) write_leaf_states_part(t, Eloc, A, P.state_out + pt, (size_t)P.n, st == DMN_STATUS_NONFINITE, split, part);
+  if (SPLIT) write_leaf_states_part(t, Eloc, A, P.state_out + pt, (size_t)P.n, st == DMN_STATUS_NONFINITE, split, part);
   else if (CMP) write_leaf_states_c(t, Eloc, A, P.state_out + pt, (size_t)P.n, st == DMN_STATUS_NONFINITE);
   else write_leaf_states(t, Eloc, A, P.state_out + pt, (size_t)P.n, st == DMN_STATUS_NONFINITE);
 }
@@ -1449,7 +1450,7 @@ int update_on(dmn_handle* h, WorkSet& w, int64_t n, int64_t n_call, const int32_
     else launch_stage<false>(SP, h->opt.stage_ctas_per_sm, sgrid, even ? 32 : 128, s);
   }
   if (ev) cudaEventRecord(ev[2], s);
-  const dim3 gf(g1, final_split(n, h->n_sm));
+  const dim3 gf(g1, final_split(n_call, h->n_sm));
   FinalParams FP{F, n, NM, tree_id, perm, Q, state_in, state_out, stress, tangent, status, w.nbuf};
   NewtonParams<double> DP{F, n, h->nslots, NM, tree_id, perm, state_in, state_out, stress, tangent, iters, status,
                           w.nbuf, w.scr_d, (double*)w.scr_t, w.counter, h->opt.tol, h->opt.max_iter, 1,
@@ -1462,10 +1463,12 @@ int update_on(dmn_handle* h, WorkSet& w, int64_t n, int64_t n_call, const int32_
     else launch_newton<double, false>(P, ls, minb, grid, cta, s);
   };
   auto final_pass = [&](const FinalParams& P, bool with_sweep) {
-    if (with_sweep && h->cmp) k_final<true, true><<<g1, 128, 0, s>>>(P);
-    else if (with_sweep) k_final<true, false><<<g1, 128, 0, s>>>(P);
-    else if (h->cmp) k_final<false, true><<<gf, 128, 0, s>>>(P);
-    else k_final<false, false><<<gf, 128, 0, s>>>(P);
+    if (with_sweep && h->cmp) k_final<true, true, false><<<g1, 128, 0, s>>>(P);
+    else if (with_sweep) k_final<true, false, false><<<g1, 128, 0, s>>>(P);
+    else if (gf.y > 1 && h->cmp) k_final<false, true, true><<<gf, 128, 0, s>>>(P);
+    else if (gf.y > 1) k_final<false, false, true><<<gf, 128, 0, s>>>(P);
+    else if (h->cmp) k_final<false, true, false><<<gf, 128, 0, s>>>(P);
+    else k_final<false, false, false><<<gf, 128, 0, s>>>(P);
   };
   // the FP64 sweep for stress, tangent and, in the FP64 form, the leaf states
   auto sweep_pass = [&](bool states) -> cudaError_t {

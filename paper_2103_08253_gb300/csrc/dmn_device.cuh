@@ -1043,6 +1043,18 @@ __device__ void tree_pass_c(const TreeDev& t, const S Eloc[6], const PointArrays
   }
 }
 
+// Strains of the children of a laminate with normal nd and jump a, for the walks that write leaf states.  The
+// roundings are written out, so that the walks below, compiled apart, give a leaf the same strain bit for bit: a
+// point's state must not depend on how many threads its call gives it.
+__device__ __forceinline__ void child_strains(const double nd[3], const double a[3], double c1, double c2,
+                                              const double e[6], double eL[6], double eR[6]) {
+  const double ndr[3] = {nd[0] * RS2, nd[1] * RS2, nd[2] * RS2};
+  const double Na[6] = {nd[0] * a[0], nd[1] * a[1], nd[2] * a[2], fma(ndr[2], a[1], ndr[1] * a[2]),
+                        fma(ndr[2], a[0], ndr[0] * a[2]), fma(ndr[1], a[0], ndr[0] * a[1])};
+#pragma unroll
+  for (int I = 0; I < 6; ++I) { const double x = e[I]; eL[I] = fma(-c2, Na[I], x); eR[I] = fma(c1, Na[I], x); }
+}
+
 // write_leaf_states for a compressed tree (tables of TreeDev).
 __device__ inline void write_leaf_states_c(const TreeDev& t, const double Eloc[6], const PointArrays& P, double* zout,
                                            size_t zos, bool nan_out) {
@@ -1060,11 +1072,7 @@ __device__ inline void write_leaf_states_c(const TreeDev& t, const double Eloc[6
       const double c1 = __ldg(t.c1 + node), c2 = __ldg(t.c2 + node);
       const double* ap = P.a + (size_t)(3 * node) * P.as;
       const double a[3] = {ap[0], ap[P.as], ap[2 * P.as]};
-      const double ndr[3] = {nd[0] * RS2, nd[1] * RS2, nd[2] * RS2};
-      double Na[6];
-      N_apply<double>(nd, ndr, a, Na);
-#pragma unroll
-      for (int I = 0; I < 6; ++I) { epsR[d + 1][I] = e[I] + c1 * Na[I]; e[I] -= c2 * Na[I]; }
+      child_strains(nd, a, c1, c2, e, e, epsR[d + 1]);
     }
     const int slot = lf_slot(f.w);
     if (slot < 0) continue;
@@ -1096,11 +1104,7 @@ __device__ inline void write_leaf_states(const TreeDev& t, const double Eloc[6],
       const double c1 = __ldg(t.c1 + node), c2 = __ldg(t.c2 + node);
       const double* ap = P.a + (size_t)(3 * jump_index(P, K, lvl, node)) * P.as;
       const double a[3] = {ap[0], ap[P.as], ap[2 * P.as]};
-      const double ndr[3] = {nd[0] * RS2, nd[1] * RS2, nd[2] * RS2};
-      double Na[6];
-      N_apply<double>(nd, ndr, a, Na);
-#pragma unroll
-      for (int I = 0; I < 6; ++I) { eL[I] = e[I] - c2 * Na[I]; eR[I] = e[I] + c1 * Na[I]; }
+      child_strains(nd, a, c1, c2, e, eL, eR);
       if (lvl < K) {
 #pragma unroll
         for (int I = 0; I < 6; ++I) { epsR[lvl + 1][I] = eR[I]; e[I] = eL[I]; }
@@ -1141,11 +1145,7 @@ __device__ inline void write_leaf_states_part(const TreeDev& t, const double Elo
     const double c1 = __ldg(t.c1 + node), c2 = __ldg(t.c2 + node);
     const double* ap = P.a + (size_t)(3 * (t.hcid ? node : jump_index(P, K, lvl, node))) * P.as;
     const double a[3] = {ap[0], ap[P.as], ap[2 * P.as]};
-    const double ndr[3] = {nd[0] * RS2, nd[1] * RS2, nd[2] * RS2};
-    double Na[6];
-    N_apply<double>(nd, ndr, a, Na);
-#pragma unroll
-    for (int I = 0; I < 6; ++I) { eL[I] = e[I] - c2 * Na[I]; eR[I] = e[I] + c1 * Na[I]; }
+    child_strains(nd, a, c1, c2, e, eL, eR);
   };
 #pragma unroll
   for (int I = 0; I < 6; ++I) e[I] = Eloc[I];
