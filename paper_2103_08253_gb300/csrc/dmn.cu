@@ -475,7 +475,7 @@ __global__ void __launch_bounds__(128, MINB) k_newton(NewtonParams<T> P) {
   Sub<T> root_acc;   // line search: results at the accepted iterate
   double Eloc[6];
   unsigned long long npass = 0;
-  const int64_t nw = (int64_t)n_work(P.n, P.n_list);
+  const int64_t nw = (int64_t)n_work(P);
   // the extrapolated start failed: continue from the stored jumps a^n, as a new point would
   auto restart = [&](const TreeDev& t) {
     const int nzf = 6 * t.nz;
@@ -768,7 +768,6 @@ struct FinalParams {
   double *state_out, *stress, *tangent;
   const int32_t* status;
   const double* nbuf;
-  const unsigned long long* n_list = nullptr;  // the points are perm[0 .. *n_list) instead of all n
   int states_only = 0;     // stress and tangent are done (k_sweep_block)
 };
 
@@ -776,9 +775,7 @@ struct FinalParams {
 // the leaves below one position of level s + 1; the first also rotates stress and tangent.  An instantiation
 // of its own: in one kernel with the whole walk it cost that walk 3 to 6 %.
 template <bool SWEEP, bool CMP, bool SPLIT>
-__global__ void __launch_bounds__(128) k_final(FinalParams P) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= (int64_t)n_work(P.n, P.n_list)) return;
+__device__ __forceinline__ void final_point(const FinalParams& P, int64_t i) {
   int64_t pt;
   int tr;
   point_of(P.perm, P.tid, P.F.n, i, pt, tr);
@@ -822,6 +819,18 @@ __global__ void __launch_bounds__(128) k_final(FinalParams P) {
   if (SPLIT) write_leaf_states_part(t, Eloc, A, P.state_out + pt, (size_t)P.n, st == DMN_STATUS_NONFINITE, split, part);
   else if (CMP) write_leaf_states_c(t, Eloc, A, P.state_out + pt, (size_t)P.n, st == DMN_STATUS_NONFINITE);
   else write_leaf_states(t, Eloc, A, P.state_out + pt, (size_t)P.n, st == DMN_STATUS_NONFINITE);
+}
+template <bool SWEEP, bool CMP, bool SPLIT>
+__global__ void __launch_bounds__(128) k_final(FinalParams P) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i < P.n) final_point<SWEEP, CMP, SPLIT>(P, i);
+}
+// the points perm[0 .. *n_list), each split over gridDim.y threads
+template <bool CMP>
+__global__ void __launch_bounds__(128) k_final_list(FinalParams P, const unsigned long long* n_list) {
+  const int64_t n = (int64_t)*n_list;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    final_point<false, CMP, true>(P, i);
 }
 
 // threads per point of k_final without the sweep: a power of two, at most 32 (each thread walks from the
@@ -1258,12 +1267,13 @@ bool warp_on(const dmn_handle* h, int64_t n) {
   return warp_possible(h) && (h->opt.warp_per_point == 1 ||
                               (h->opt.first_stage != 1 && n <= (int64_t)warp_auto_points_per_sm(h) * h->n_sm));
 }
+constexpr int WARP_FULL_POINTS_PER_SM = 16;
 // lanes per point of the warp organisation: the option's, else by the call's size: 32 while there
 // are few points per SM (latency), then fewer (fewer idle lanes on the upper levels): 8 for the
 // FP64 condensation, 16 for the FP32 one (whose FP64 work is a smaller part)
 int warp_lanes_for(const dmn_handle* h, int64_t n) {
   if (h->opt.warp_lanes) return h->opt.warp_lanes;
-  if (n <= 16 * (int64_t)h->n_sm) return 32;
+  if (n <= (int64_t)WARP_FULL_POINTS_PER_SM * h->n_sm) return 32;
   return h->opt.precision == DMN_PREC_F64 ? 8 : 16;
 }
 
@@ -1287,18 +1297,20 @@ int block_leaf_slots(const dmn_handle* h) {
 cudaError_t alloc_ws(const dmn_handle* h, WorkSet& w) {
   // per slot: normals + one or two jump buffers (FP64); one or two g, H buffers + FP32 normals
   const size_t sd = h->opt.line_search ? 9 : 6, stt = h->opt.line_search ? 45 : 24;
-  cudaError_t e = cudaMalloc(&w.scr_d, sizeof(double) * (size_t)(sd * h->N_max) * h->nslots);
-  if (e == cudaSuccess) e = cudaMalloc(&w.scr_t, sizeof(double) * (size_t)(stt * h->N_max) * h->nslots);
+  const bool block = block_on(h);   // runs no thread-per-point kernel: 3.6 GB less at depth 8
+  cudaError_t e = cudaSuccess;
+  if (!block) e = cudaMalloc(&w.scr_d, sizeof(double) * (size_t)(sd * h->N_max) * h->nslots);
+  if (e == cudaSuccess && !block) e = cudaMalloc(&w.scr_t, sizeof(double) * (size_t)(stt * h->N_max) * h->nslots);
   if (e == cudaSuccess) e = cudaMalloc(&w.counter, sizeof(unsigned long long) * (32 + BLOCK_TOKENS));
   if (e == cudaSuccess && first_stage_on(h->opt)) {
     w.nslots_s = (int64_t)h->n_sm * h->opt.stage_ctas_per_sm * 128;
     e = cudaMalloc(&w.scr_s, sizeof(float) * (size_t)(27 * h->N_max) * w.nslots_s);
   }
-  if (e == cudaSuccess && block_on(h))
+  if (e == cudaSuccess && block)
     e = cudaMalloc(&w.scr_b, block_scratch_bytes(BLOCK_THREADS, block_leaf_slots(h), h->opt.line_search != 0) * (size_t)(h->n_sm * BLOCK_CTAS_PER_SM));
-  if (e == cudaSuccess && warp_possible(h)) {
+  if (e == cudaSuccess && (block || warp_possible(h))) {   // block: for the points handed back
     // one slot per group of the smallest size the handle may use
-    w.nwarps_w = (int64_t)h->n_sm * WARP_CTAS_PER_SM * 128 / (h->opt.warp_lanes ? h->opt.warp_lanes : WARP_MIN_LANES);
+    w.nwarps_w = (int64_t)h->n_sm * WARP_CTAS_PER_SM * 128 / (!block && h->opt.warp_lanes ? h->opt.warp_lanes : WARP_MIN_LANES);
     const size_t per = h->opt.precision != DMN_PREC_F64 ? warp_slot_doubles<float>(h->N_max)
                                                         : warp_slot_doubles<double>(h->N_max);
     e = cudaMalloc(&w.scr_w, sizeof(double) * per * (size_t)w.nwarps_w);
@@ -1437,7 +1449,7 @@ int update_on(dmn_handle* h, WorkSet& w, int64_t n, int64_t n_call, const int32_
   const bool stage = first_stage_on(h->opt) && !warp;   // a small batch goes straight to the warp kernel
   const unsigned wgrid = (unsigned)(h->n_sm * WARP_CTAS_PER_SM);
   const bool block = w.scr_b != nullptr;
-  const int lanes = warp && !block ? warp_lanes_for(h, n_call) : 32;
+  const int lanes = warp ? warp_lanes_for(h, n_call) : 32;
   unsigned long long* passes = h->profiling ? h->d_passes : nullptr;
   if (stage) {   // counter [19]: the first stage's work counter
     // its corrections count against max_iter: the FP64-residual iteration keeps at least one
@@ -1496,13 +1508,16 @@ int update_on(dmn_handle* h, WorkSet& w, int64_t n, int64_t n_call, const int32_
   if (block) {
     e = sweep_pass(true);
     if (e != cudaSuccess) return cuda_fail(h, e, "dmn_update: launch");
-    // the points it left: the all-FP64 iteration from their start, in the organisation of the call's size (few
-    // points: a warp each)
+    // the points it left: the all-FP64 iteration from their start, then their leaf states and outputs
     NewtonParams<double> P = DP;
     P.perm = FP.perm = w.list;
-    P.n_list = FP.n_list = w.counter + 29;
-    newton_f64(P);
-    final_pass(FP, false);
+    P.n_list = w.counter + 29;
+    const int64_t few = (int64_t)WARP_FULL_POINTS_PER_SM * h->n_sm;
+    if (h->cmp) launch_list<true>(P, ls, few, wgrid, w.scr_w, s);
+    else launch_list<false>(P, ls, few, wgrid, w.scr_w, s);
+    const dim3 gl((unsigned)std::min<int64_t>(g1, 2 * h->n_sm), 32);
+    if (h->cmp) k_final_list<true><<<gl, 128, 0, s>>>(FP, P.n_list);
+    else k_final_list<false><<<gl, 128, 0, s>>>(FP, P.n_list);
   } else if (sweep && block_trees(h) && n_call <= (int64_t)SWEEP_BLOCK_MAX * h->n_sm) {
     e = sweep_pass(false);
     if (e != cudaSuccess) return cuda_fail(h, e, "dmn_update: launch");
@@ -1564,7 +1579,7 @@ cudaError_t pipe_ready(dmn_handle* h, int64_t cap) {
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&P.start, cudaEventDisableTiming);
     if (e != cudaSuccess) { free_pipe(P); return e; }
   }
-  if (!h->ws[1].scr_d) {
+  if (!h->ws[1].counter) {
     e = alloc_ws(h, h->ws[1]);
     if (e != cudaSuccess) { free_ws(h->ws[1]); return e; }
   }

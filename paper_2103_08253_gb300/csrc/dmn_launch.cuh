@@ -56,9 +56,10 @@ struct NewtonParams {
 // Status of a point that k_newton_block leaves to the all-FP64 kernels; never returned to a caller.
 constexpr int32_t STATUS_RETRY = -1;
 
-// number of points a launch works through
-__device__ __forceinline__ unsigned long long n_work(int64_t n, const unsigned long long* n_list) {
-  return n_list ? *n_list : (unsigned long long)n;
+// number of points a launch works through (lists hold points of the FP64 form only)
+template <typename T>
+__device__ __forceinline__ unsigned long long n_work(const NewtonParams<T>& P) {
+  return sizeof(T) == 8 && P.n_list ? *P.n_list : (unsigned long long)P.n;
 }
 
 // Small calls: one point per group of G lanes of a warp (G = 32, 16 or 8; the paper's start; heap
@@ -83,6 +84,9 @@ constexpr int WARP_MIN_LANES = 8;     // the smallest group: the scratch holds 3
 // grid * 128 / lanes slots of warp_slot_doubles<T>(P.N_max) doubles
 template <typename T, bool CMP>
 void launch_warp(const NewtonParams<T>& P, bool ls, int lanes, unsigned grid, double* scr, cudaStream_t s);
+// the points on P.n_list in this organisation, 32 lanes each if there are at most `few`, else 8
+template <bool CMP>
+void launch_list(const NewtonParams<double>& P, bool ls, int64_t few, unsigned grid, double* scr, cudaStream_t s);
 // The CTA organisation of the FP64 form (csrc/dmn_block.cu).  counter: [1..9] points per tree and
 // [10..18] their ends in perm (several trees), [21..28] work counters per tree, [29] points on the list.
 constexpr int BLOCK_THREADS = 256;

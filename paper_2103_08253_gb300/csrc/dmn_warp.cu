@@ -10,7 +10,7 @@
 namespace dmn {
 
 template <typename T, bool LS, int G, bool CMP>
-__global__ void __launch_bounds__(128) k_newton_warp(NewtonParams<T> P, double* scratch) {
+__device__ __forceinline__ void newton_warp(const NewtonParams<T>& P, double* scratch) {
   static_assert(G == 8 || G == 16 || G == 32, "8, 16 or 32 lanes per point");
   const int64_t grp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / G;
   const int lane = threadIdx.x % G;
@@ -47,7 +47,7 @@ __global__ void __launch_bounds__(128) k_newton_warp(NewtonParams<T> P, double* 
       unsigned long long i = 0;
       if (lane == 0) i = atomicAdd(P.counter, 1ull);
       i = __shfl_sync(gmask, i, 0, G);
-      if (i >= n_work(P.n, P.n_list)) return false;
+      if (i >= n_work(P)) return false;
       point_of(P.perm, P.tid, P.F.n, (int64_t)i, pt, tr);
       if (tr < P.F.n) break;
       if (lane == 0) {   // unknown tree: report and take the next point
@@ -145,6 +145,31 @@ __global__ void __launch_bounds__(128) k_newton_warp(NewtonParams<T> P, double* 
   }
   if (lane == 0 && P.passes && npass) atomicAdd(P.passes, npass);
 }
+
+template <typename T, bool LS, int G, bool CMP>
+__global__ void __launch_bounds__(128) k_newton_warp(NewtonParams<T> P, double* scratch) {
+  newton_warp<T, LS, G, CMP>(P, scratch);
+}
+
+// The points that k_newton_block handed back.  Only the device knows how many, normally none: up to `few` run 32
+// lanes each (a chain of passes as short as it gets), more run 8 (fewer idle lanes), whatever the size of the
+// call they come from.  One point of a 200003-point call of depth 8 otherwise waits for a whole
+// thread-per-point iteration (148 ms for the call; 120 here, 118 with none on the list).
+template <bool LS, bool CMP>
+__global__ void __launch_bounds__(128) k_newton_list(NewtonParams<double> P, double* scratch, unsigned long long few) {
+  const unsigned long long n = *P.n_list;
+  if (n == 0) return;
+  if (n <= few) newton_warp<double, LS, 32, CMP>(P, scratch);
+  else newton_warp<double, LS, 8, CMP>(P, scratch);
+}
+
+template <bool CMP>
+void launch_list(const NewtonParams<double>& P, bool ls, int64_t few, unsigned grid, double* scr, cudaStream_t s) {
+  if (ls) k_newton_list<true, CMP><<<grid, 128, 0, s>>>(P, scr, (unsigned long long)few);
+  else k_newton_list<false, CMP><<<grid, 128, 0, s>>>(P, scr, (unsigned long long)few);
+}
+template void launch_list<false>(const NewtonParams<double>&, bool, int64_t, unsigned, double*, cudaStream_t);
+template void launch_list<true>(const NewtonParams<double>&, bool, int64_t, unsigned, double*, cudaStream_t);
 
 template <typename T, bool CMP>
 void launch_warp(const NewtonParams<T>& P, bool ls, int lanes, unsigned grid, double* scr, cudaStream_t s) {
