@@ -75,7 +75,16 @@ enum { DMN_OK = 0, DMN_ERR_ARG = -1, DMN_ERR_CUDA = -2 };
  * alpha_bar is the equivalent plastic strain. */
 enum { DMN_PHASE_ELASTIC = 0, DMN_PHASE_J2_LINEAR = 1, DMN_PHASE_J2_EXPLIN = 2 };
 
-/* DMN_PREC_F64: every step in FP64.
+/* DMN_PREC_F64: strains, leaf laws, jumps, the Newton residual and its criterion, the sweep that yields
+ * stress and tangent, and the states in FP64.  Below depth 3, with the extrapolated start, after the first
+ * stage and in the warp organisation asked for by name (dmn_options.warp_per_point) so is the linear solve of
+ * the Newton step.  Otherwise that solve condenses the leaf tangents in FP32 and refines: the residual
+ * R + J da1 of its result is formed in pairs of FP32 numbers (about 46 bits) and solved for in FP32 again, so
+ * that the step's relative error is about the square of the FP32 solve's (1e-11 on the plastic paths
+ * measured).  A point whose first solve leaves more than 1e-3 of the residual (the step's error is then
+ * bounded by 1e-6 of it), which is not finite or not converged after 16 corrections starts again in the
+ * all-FP64 iteration.  A residual that meets the criterion may hold, below tol, what the refinement left of
+ * the last step.
  * DMN_PREC_MIXED: leaf tangents, laminate condensation and jump corrections
  * in FP32; leaf stresses, strains, jumps, the Newton residual and the final
  * sweep that yields stress and tangent in FP64.
@@ -121,10 +130,13 @@ typedef struct {
 
 typedef struct {
   double tol;          /* ||A^T W sigma|| / ((2^K - 1) ||sigma_bar||) <= tol (Sec. 4.6); <= 0 selects 1e-12 */
-  int32_t max_iter;    /* Newton corrections before status MAXITER; <= 0 selects 50 */
+  int32_t max_iter;    /* Newton corrections before status MAXITER; <= 0 selects 50.  Where the FP64 form's
+                        * refined step leaves a residual above tol no larger than 4 times its own linear
+                        * system's, a further solve finishes that step; neither max_iter nor iters nor the
+                        * pass counters count it apart, and one may follow the last correction */
   int32_t precision;   /* DMN_PREC_F64, DMN_PREC_MIXED or DMN_PREC_MIXED_F32_TANGENT */
-  int32_t block;       /* threads per CTA of the Newton kernel (multiple of 32); 0 selects 128 */
-  int32_t ctas_per_sm; /* resident CTAs per SM of the persistent Newton kernel; 0 selects 384 threads
+  int32_t block;       /* threads per CTA of the thread-per-point Newton kernel (multiple of 32); 0 selects 128 */
+  int32_t ctas_per_sm; /* resident CTAs per SM of that persistent kernel; 0 selects 384 threads
                         * per SM for DMN_PREC_F64 and 512 for the mixed forms;
                         * block * ctas_per_sm <= 512 (registers are capped to fit) */
   int32_t line_search; /* 0: full Newton steps; 1: backtracking (Sec. 3.2 allows a step in (0, 1]):
@@ -156,23 +168,26 @@ typedef struct {
                         * Not run with line_search or predictor. */
   int32_t stage_ctas_per_sm; /* resident CTAs of 128 threads per SM of the first stage's persistent kernel:
                               * 2, 3, 4, 6 or 8 (registers capped to fit); 0 selects the default */
-  int32_t warp_per_point; /* small batches: 0 (default) updates a call of at most 1024 points per SM
-                           * of the device in the FP64 form, 256 in the mixed forms (155648 / 38912 on
-                           * 152 SMs) in the warp organisation: a point per group of 32, 16 or 8 lanes
-                           * of a warp, the group's lanes sharing each level of the tree (the same
-                           * arithmetic per laminate and the same iterates to rounding), where one point
-                           * per thread would leave SMs idle; 1 does so for every call; -1 never.  The choice is made per call (for
-                           * dmn_update_host on the whole batch, not per chunk); first_stage = 1 turns
-                           * the default off.  The extrapolated start always runs one point per thread; the
-                           * first stage is not run in this organisation.  Compressed trees (weightless
-                           * leaves) run it level by level of the full tree's heap positions. */
-  int32_t warp_lanes;     /* lanes per point in that organisation: 32 (one point per warp), 16 or 8 (two
+  int32_t warp_per_point; /* the organisation of the kernels that update a whole tree per thread: 0 (default)
+                           * runs a call of at most 1024 points per SM of the device in the FP64 form, 256 in
+                           * the mixed forms (155648 / 38912 on 152 SMs) in the warp organisation: a point per
+                           * group of 32, 16 or 8 lanes of a warp, the group's lanes sharing each level of
+                           * the tree (the same arithmetic per laminate and the same iterates to rounding),
+                           * where one point per thread would leave SMs idle; 1 does so for every call; -1
+                           * never.  The choice is made per call (for dmn_update_host on the whole batch, not
+                           * per chunk); first_stage = 1 turns the default off.  The extrapolated start always
+                           * runs one point per thread; the first stage is not run in this organisation.
+                           * Compressed trees (weightless leaves) run it level by level of the full tree's
+                           * heap positions.
+                           * The FP64 form of trees of depth 3 or more, without the extrapolated start or the
+                           * first stage, runs a third organisation instead, whatever this option says: a
+                           * CTA's threads share its points' trees (see DMN_PREC_F64).  It ignores warp_lanes,
+                           * block and ctas_per_sm.  warp_per_point = 1 with warp_lanes given names the warp
+                           * organisation, and runs it: the all-FP64 iteration. */
+  int32_t warp_lanes;     /* lanes per point in the warp organisation: 32 (one point per warp), 16 or 8 (two
                            * or four points per warp, side by side); 0 (default) chooses by the call's
                            * size: 32 up to 16 points per SM, then 8 in the FP64 form, 16 in the mixed
-                           * forms.  The FP64 form's trees of depth 3 or more (without the extrapolated
-                           * start or the first stage) run a third organisation at every size, in which a
-                           * CTA's threads share its points' trees; both options then only choose the
-                           * kernels of the few points handed back to the all-FP64 iteration. */
+                           * forms */
 } dmn_options;
 
 /* Create a handle for n_trees DMNs (1 <= n_trees <= DMN_MAX_TREES; trees may

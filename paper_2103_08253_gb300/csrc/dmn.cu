@@ -1285,7 +1285,8 @@ bool block_trees(const dmn_handle* h) {
   return true;
 }
 bool block_on(const dmn_handle* h) {
-  return h->opt.precision == DMN_PREC_F64 && !h->opt.predictor && !first_stage_on(h->opt) && block_trees(h);
+  const bool warp_asked = h->opt.warp_per_point == 1 && h->opt.warp_lanes;   // the warp organisation, by name
+  return h->opt.precision == DMN_PREC_F64 && !h->opt.predictor && !first_stage_on(h->opt) && !warp_asked && block_trees(h);
 }
 int block_leaf_slots(const dmn_handle* h) {
   for (const Tree& t : h->trees)
@@ -1310,7 +1311,7 @@ cudaError_t alloc_ws(const dmn_handle* h, WorkSet& w) {
     e = cudaMalloc(&w.scr_b, block_scratch_bytes(BLOCK_THREADS, block_leaf_slots(h), h->opt.line_search != 0) * (size_t)(h->n_sm * BLOCK_CTAS_PER_SM));
   if (e == cudaSuccess && (block || warp_possible(h))) {   // block: for the points handed back
     // one slot per group of the smallest size the handle may use
-    w.nwarps_w = (int64_t)h->n_sm * WARP_CTAS_PER_SM * 128 / (!block && h->opt.warp_lanes ? h->opt.warp_lanes : WARP_MIN_LANES);
+    w.nwarps_w = (int64_t)h->n_sm * WARP_CTAS_PER_SM * 128 / (h->opt.warp_lanes && !block ? h->opt.warp_lanes : WARP_MIN_LANES);
     const size_t per = h->opt.precision != DMN_PREC_F64 ? warp_slot_doubles<float>(h->N_max)
                                                         : warp_slot_doubles<double>(h->N_max);
     e = cudaMalloc(&w.scr_w, sizeof(double) * per * (size_t)w.nwarps_w);
