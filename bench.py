@@ -105,7 +105,6 @@ F_STATE_NODE = 39       # state pass: per laminate (strains from the jumps)
 F_STATE_J2 = 68         # state pass: per J2 leaf (return mapping and new state)
 
 
-SWEEP_BLOCK_MAX = 4096 * 152   # points up to which the mixed form's sweep is a kernel of its own
 F_LEAF_SUB = 84         # a leaf whose sibling is a laminate: its 21 tangent entries as a subtree (T)
 
 
@@ -356,7 +355,9 @@ def form_opts(form):
     """(precision, extrapolated start) of a form name such as "f64", "mixed-f32-tangent/extrap",
     "mixed/no-stage" (the mixed iteration without its all-FP32 first stage), "f64/stage" (the FP64
     iteration after that stage), "f64/thread" (one point per thread whatever the batch size) or
-    "f64/w8" (the warp organisation with 8, 16 or 32 lanes per point whatever the batch size)."""
+    "f64/w8" (the warp organisation with 8, 16 or 32 lanes per point whatever the batch size).  At the
+    bench's depth the FP64 form runs the CTA organisation; of these names "/stage" and "/extrap" (one point
+    per thread) and "/w8", "/w16", "/w32" leave it, "f64/thread" does not."""
     prec, _, start = form.partition("/")
     if start not in ("", "extrap", "no-stage", "stage", "thread", "w8", "w16", "w32"):
         raise ValueError("unknown start in form %r" % form)
@@ -403,13 +404,32 @@ def form_warp_option(form):
     return 0, 0
 
 
+def n_sm():
+    import torch
+    return torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
+
+
+def cta_size(n, threads):
+    """Threads per CTA of k_newton_block for n points of `threads` threads each (launch_block's rule)."""
+    return 128 if -(-n * threads // 256) <= n_sm() else 256
+
+
+def sweep_apart(n, sms):
+    """Whether the mixed form's FP64 sweep is a kernel of its own (k_sweep_block) in a call of n points."""
+    return n <= 4096 * sms
+
+
 def tune_shape(form, ctx, args):
     """Launch shape of the Newton kernel from the autotuner, tuned on the first 2^18 points at the
     first timed increment (after the warm-up increments).  Forms that differ only in the start
-    share the kernel and its shape."""
+    share the kernel and its shape; in the FP64 form those that run one point per thread are tuned
+    with the first stage, the others take no shape (None)."""
     import torch
     from paper_2103_08253_gb300 import autotune, dmn
-    form, _ = form_opts(form)
+    form, start = form_opts(form)[0], form.partition("/")[2]
+    if form == "f64" and start not in ("stage", "extrap"):
+        return None
+    stage = True if form == "f64" else None
     cache = ctx.setdefault("shapes", {})
     if form in cache:
         return cache[form]
@@ -424,7 +444,7 @@ def tune_shape(form, ctx, args):
     h.close()
     s = args.warmup + 1
     res = autotune.tune(ctx["tree"], form, lam, Q, ctx["En"][s - 1][:m].contiguous(),
-                        ctx["dE"][s - 1][:m].contiguous(), st, reps=1)
+                        ctx["dE"][s - 1][:m].contiguous(), st, reps=1, first_stage=stage)
     # the first stage's own launch shape, at the Newton kernel's tuned one
     ts = autotune.tune_stage(ctx["tree"], form, lam, Q, ctx["En"][s - 1][:m].contiguous(),
                              ctx["dE"][s - 1][:m].contiguous(), st, block=res["block"], ctas_per_sm=res["ctas_per_sm"])
@@ -494,9 +514,9 @@ def run_form(form, ctx, args, dist):
     clk = clocks.stop() if clocks else None
     kms, passes, cnt = m.profile_read_stages()
     m.profile(False)
-    # the FP64 form from depth 3 on runs k_newton_block at every size; of the others a small call runs the warp
-    # organisation, without the first stage
-    block = m.precision == "f64" and not m.predictor and not m.first_stage and K_DEPTH >= 3
+    # the FP64 form runs k_newton_block; of the others a small call runs the warp organisation, without the
+    # first stage
+    block = m.cta_threads(n)
     lanes = m.lanes_per_point(n)
     warp = lanes > 1 and not block
     if not form_stage(form) or warp:
@@ -504,8 +524,8 @@ def run_form(form, ctx, args, dist):
     its = iters_steps.to(torch.int64).sum().item()
     hist = torch.bincount(iters_steps.reshape(-1).to(torch.int64), minlength=1).cpu().numpy()
     res = dict(t_ms=t_ms, kms=kms, updates=cnt, clocks=clk, iters_sum=int(its), iters_hist=hist.tolist(),
-               passes=passes, warp=warp, block=block,
-               launch=("CTAs of 256 threads, %d per point (k_newton_block)" % (1 << (K_DEPTH - 3)) if block else
+               passes=passes, warp=warp, block=block, n_sm=n_sm(),
+               launch=("CTAs of %d threads, %d per point (k_newton_block)" % (cta_size(n, block), block) if block else
                        "%d lanes per point (k_newton_warp, 2 CTAs of 4 warps per SM)" % lanes if warp else
                        dict(block=shape["block"], ctas_per_sm=shape["ctas_per_sm"], tuned_on_points=shape["points"],
                             table=shape["table"], stage_ctas_per_sm=shape["stage_ctas_per_sm"],
@@ -663,7 +683,7 @@ def roofline_mixed(r, n, steps, w=None, sweep=True, peaks=None):
     tb = F64 / (P64 * 1e9) + F32 / (P32 * 1e9)
     Ff = final_flops(K_DEPTH, n * steps, sweep=sweep, w=w)
     tf = r["kms"]["final"] * 1e-3
-    fin = {"kernel": ("k_sweep_block, k_final" if n <= SWEEP_BLOCK_MAX else "k_final<sweep>") if sweep else "k_final", "achieved": Ff / tf / 1e9, "peak": P64,
+    fin = {"kernel": ("k_sweep_block, k_final" if sweep_apart(n, r.get("n_sm", 152)) else "k_final<sweep>") if sweep else "k_final", "achieved": Ff / tf / 1e9, "peak": P64,
            "unit": "GFLOP/s (FP64)", "frac": Ff / tf / 1e9 / P64, "launch_ms": r["kms"]["final"] / steps}
     cmp = "_compressed" if w is not None and (np.asarray(w) == 0).any() else ""
     stg = "stage" in r["kms"]
@@ -779,7 +799,8 @@ def run_mixed_depth(args):
         el = torch.from_numpy(elastic).to(dev)
         line["forms"][form] = {
             "value": n * G / (t_ms * 1e-3), "unit": UNIT, "ms_per_step": t_ms / G,
-            "launch": {"block": best[0], "ctas_per_sm": best[1], "autotuner_table": tuned["table"]},
+            "launch": ({"block": best[0], "ctas_per_sm": best[1], "autotuner_table": tuned["table"]} if tuned["used"]
+                       else "CTA organisation, no launch shape"),
             "iters_elastic_half": torch.bincount(its[:, el].reshape(-1)).cpu().tolist(),
             "iters_cyclic_half": torch.bincount(its[:, ~el].reshape(-1)).cpu().tolist(),
             "status_counts": torch.bincount(stat.reshape(-1).to(torch.int64)).cpu().tolist(),
@@ -1039,7 +1060,7 @@ def run_gpu(args):
                              % (state_fields(tree) * n * 8e-6),
                        "parallelism": "independent point shards per GPU, no collective"},
             "roofline": forms_out[main_form]["roofline"], "cpu_baseline": cpu, "e2e": e2e,
-            "gpu_launches": (4 + ("stage" in mr["kms"]) + (main_form.split("/")[0] == "mixed" and n <= SWEEP_BLOCK_MAX)
+            "gpu_launches": (4 + ("stage" in mr["kms"]) + (main_form.split("/")[0] == "mixed" and sweep_apart(n, n_sm()))
                              + 2 * bool(mr.get("block")))
                             * steps, "clocks": mr["clocks"],
             "peaks": {"fp64_gflops": peaks["f64"], "fp32_gflops": peaks["f32"], "note": peaks["note"]}}

@@ -217,8 +217,14 @@ int64_t dmn_state_size(const dmn_handle* h, int32_t tree_id);
 /* The organisation dmn_update (and dmn_update_host) gives a call of n points on this handle, as
  * lanes per point: 1 one point per thread of the persistent kernel, 32 / 16 / 8 the warp
  * organisation with one / two / four points per warp (dmn_options.warp_per_point, warp_lanes);
- * -1 on a NULL handle or n < 0.  A query only: no device work. */
+ * -1 on a NULL handle or n < 0.  Where dmn_update_cta_threads is not 0 the call runs neither, and the value
+ * is what the all-FP64 iteration would get.  A query only: no device work. */
 int dmn_update_lanes_per_point(const dmn_handle* h, int64_t n);
+
+/* The threads that share a point of the handle's deepest tree (2^(K-3)) if a call of n points runs the CTA
+ * organisation (the FP64 form from depth 3 on, dmn_options.warp_per_point); 0 if it does not; -1 on a NULL
+ * handle or n < 0.  A query only: no device work. */
+int dmn_update_cta_threads(const dmn_handle* h, int64_t n);
 
 /* Orientation set-up (Sec. 2.2, Eq. of the eigen decomposition of A2):
  * A2 dev [n][6] (plain components, symmetric positive semi-definite, unit

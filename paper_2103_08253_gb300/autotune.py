@@ -6,6 +6,8 @@ several trees (mixed depths) are tuned on their own batch and cached under a
 key of their own.  The FP64 form is
 bound by the FP64 pipe once each SM holds a few warps, the FP32 form hides
 latency with more resident warps, and both trade occupancy against registers.
+The FP64 form's handles that run the CTA organisation (`dmn.DMN.cta_threads`)
+take no launch shape: `tune` times one such handle and returns the first candidate.
 `tune` times every candidate shape on a caller-provided batch through the C ABI
 (per-kernel CUDA events of the Newton kernel) and returns the fastest;
 `tune_stage` does the same for the first stage's kernel, which has a launch
@@ -53,7 +55,7 @@ def cached(tree, precision, device=None):
 def tune(tree, precision, lam, Q, E_n, dE, state_in, reps=2, candidates=CANDIDATES, save=True, tree_id=None,
          first_stage=None):
     """Time the Newton kernel of every candidate shape on this batch; returns
-    dict(block, ctas_per_sm, newton_ms, table).  tree may be a list of trees (one handle with
+    dict(block, ctas_per_sm, newton_ms, table, used: whether that kernel takes a shape).  tree may be a list of trees (one handle with
     several trees, as dmn.DMN takes it), with tree_id [n] (int32, device) selecting each
     point's tree.  first_stage as in dmn.DMN; with the first stage the time is that of the stage
     and the Newton kernel together (the stage keeps its own launch shape)."""
@@ -61,9 +63,14 @@ def tune(tree, precision, lam, Q, E_n, dE, state_in, reps=2, candidates=CANDIDAT
     dev = lam.device
     n = lam.shape[0]
     table = []
+    cta = False        # the CTA organisation, which takes no launch shape
     for block, cps in candidates:
+        if cta:
+            table.append((block, cps, table[0][2]))
+            continue
         m = dmn.DMN(tree, precision=precision, block=block, ctas_per_sm=cps, first_stage=first_stage,
                     warp_per_point=-1)
+        cta = m.cta_threads(n) > 0
         out = m.alloc_outputs(n, dev)
         m.update(lam, Q, E_n, dE, state_in, out=out, tree_id=tree_id)
         torch.cuda.synchronize()
@@ -77,7 +84,7 @@ def tune(tree, precision, lam, Q, E_n, dE, state_in, reps=2, candidates=CANDIDAT
         table.append((block, cps, kms["newton"] / cnt))
     torch.cuda.empty_cache()
     block, cps, ms = min(table, key=lambda r: r[2])
-    res = dict(block=block, ctas_per_sm=cps, newton_ms=ms, points=n,
+    res = dict(block=block, ctas_per_sm=cps, newton_ms=ms, points=n, used=not cta,
                table=[dict(block=b, ctas_per_sm=c, newton_ms=t) for b, c, t in table])
     if save:
         data = _load()

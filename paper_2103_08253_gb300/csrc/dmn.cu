@@ -1783,6 +1783,11 @@ int dmn_update_lanes_per_point(const dmn_handle* h, int64_t n) {
   return warp_on(h, n) ? warp_lanes_for(h, n) : 1;
 }
 
+int dmn_update_cta_threads(const dmn_handle* h, int64_t n) {
+  if (!h || n < 0) return -1;
+  return block_on(h) ? 1 << (h->K_max - 3) : 0;
+}
+
 int dmn_profile_enable(dmn_handle* h, int32_t enable) {
   if (!h) return fail(nullptr, DMN_ERR_ARG, "dmn_profile_enable: NULL handle");
   if (enable) {

@@ -16,8 +16,8 @@ from . import build as _build
 _lib = None
 
 # ABI symbols declared in include/dmn.h
-EXPORTS = ("dmn_create", "dmn_destroy", "dmn_state_size", "dmn_update_lanes_per_point", "dmn_interp_orientation",
-           "dmn_update",
+EXPORTS = ("dmn_create", "dmn_destroy", "dmn_state_size", "dmn_update_lanes_per_point", "dmn_update_cta_threads",
+           "dmn_interp_orientation", "dmn_update",
            "dmn_set_params", "dmn_grad", "dmn_profile_enable", "dmn_profile_read", "dmn_profile_read_stages",
            "dmn_update_noalloc",
            "dmn_update_host", "dmn_last_error")
@@ -76,6 +76,8 @@ def load_library(build_if_missing: bool = True):
     lib.dmn_state_size.restype = i64
     lib.dmn_update_lanes_per_point.restype = ctypes.c_int
     lib.dmn_update_lanes_per_point.argtypes = [ctypes.c_void_p, i64]
+    lib.dmn_update_cta_threads.restype = ctypes.c_int
+    lib.dmn_update_cta_threads.argtypes = [ctypes.c_void_p, i64]
     lib.dmn_interp_orientation.argtypes = [vp, i64, vp, vp, vp, vp]
     lib.dmn_interp_orientation.restype = ctypes.c_int
     lib.dmn_update.argtypes = [vp, i64, vp, vp, vp, vp, vp, vp, vp, vp, vp, vp, vp, vp]
@@ -291,10 +293,19 @@ class DMN:
 
     def lanes_per_point(self, n: int) -> int:
         """dmn_update_lanes_per_point: the organisation of a call of n points, as lanes per point (1
-        one point per thread of the persistent kernel; 32, 16 or 8 the warp organisation)."""
+        one point per thread of the persistent kernel; 32, 16 or 8 the warp organisation); a call whose
+        cta_threads is not 0 runs neither."""
         r = self._lib.dmn_update_lanes_per_point(self._h, int(n))
         if r < 0:
             raise ValueError("lanes_per_point: n must be >= 0 on an open handle")
+        return int(r)
+
+    def cta_threads(self, n: int) -> int:
+        """dmn_update_cta_threads: threads per point (of the deepest tree) if a call of n points runs the CTA
+        organisation, else 0."""
+        r = self._lib.dmn_update_cta_threads(self._h, int(n))
+        if r < 0:
+            raise ValueError("cta_threads: n must be >= 0 on an open handle")
         return int(r)
 
     def close(self):

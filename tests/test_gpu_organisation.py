@@ -1,8 +1,9 @@
-"""Which organisation a handle's calls run: the options that name one get it."""
+"""Which organisation a handle's calls run: the options that name one get it, the query reports it, and the launch
+shape's tuner does not time shapes that it does not take."""
 import pytest
 import torch
 
-from paper_2103_08253_gb300 import dmn, workloads as W
+from paper_2103_08253_gb300 import autotune, dmn, workloads as W
 from test_gpu_block import inputs
 from test_gpu_parity import d
 
@@ -26,3 +27,36 @@ def test_lanes_asked_for_run_the_all_fp64_warp_kernel(lanes, kind):
         m.close()
     for k, v in outs[0].items():
         assert torch.equal(v, outs[1][k]), k
+
+
+@pytest.mark.parametrize("K,opts,want", [(8, {}, 32), (4, dict(warp_per_point=-1, line_search=True), 2), (2, {}, 0),
+                                         (8, dict(first_stage=True), 0), (8, dict(predictor=True), 0),
+                                         (8, dict(precision="mixed"), 0), (6, dict(warp_per_point=1), 8),
+                                         (6, dict(warp_per_point=1, warp_lanes=8), 0)])
+def test_the_query_reports_the_cta_organisation(K, opts, want):
+    m = dmn.DMN(W.tree_d10_fit(K, seed=872), **opts)
+    assert m.cta_threads(1000) == want
+    m.close()
+    m = dmn.DMN([W.tree_d10_fit(3, seed=873), W.tree_d10_fit(K, seed=874)], **opts)
+    assert m.cta_threads(1 << 20) == want
+    with pytest.raises(ValueError):
+        m.cta_threads(-1)
+    m.close()
+
+
+def test_the_tuner_times_a_kernel_without_a_launch_shape_once(tmp_path, monkeypatch):
+    monkeypatch.setattr(autotune, "CACHE", str(tmp_path / "autotune.json"))
+    n = 3000
+    tree = W.tree_d10_fit(4, seed=875)
+    lam, Q, Ef = (d(x) for x in inputs(n, 876))
+    st = torch.zeros((W.state_size(4), n), dtype=torch.float64, device=DEV)
+    made = []
+    real = dmn.DMN
+    monkeypatch.setattr(dmn, "DMN", lambda *a, **k: made.append(k) or real(*a, **k))
+    for stage, handles in ((None, 1), (True, 3)):
+        made.clear()
+        res = autotune.tune(tree, "f64", lam, Q, torch.zeros_like(Ef), Ef * 0.1, st, reps=1, first_stage=stage,
+                            candidates=((128, 2), (64, 4), (32, 8)))
+        assert len(made) == handles and len(res["table"]) == 3 and res["used"] == (stage is True)
+        if not res["used"]:
+            assert (res["block"], res["ctas_per_sm"]) == (128, 2)
