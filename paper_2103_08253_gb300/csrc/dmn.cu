@@ -475,7 +475,6 @@ __global__ void __launch_bounds__(128, MINB) k_newton(NewtonParams<T> P) {
   Sub<T> root_acc;   // line search: results at the accepted iterate
   double Eloc[6];
   unsigned long long npass = 0;
-  const int64_t nw = (int64_t)n_work(P);
   // the extrapolated start failed: continue from the stored jumps a^n, as a new point would
   auto restart = [&](const TreeDev& t) {
     const int nzf = 6 * t.nz;
@@ -501,7 +500,7 @@ __global__ void __launch_bounds__(128, MINB) k_newton(NewtonParams<T> P) {
       base = __shfl_sync(0xffffffffu, base, leader);
       if (need) {
         const int64_t i = (int64_t)(base + __popc(mask & ((1u << lane) - 1u)));
-        if (i >= nw) {
+        if (i >= P.n) {
           pt = P.n;
         } else {
           point_of(P.perm, P.tid, P.F.n, i, pt, tr);
@@ -780,7 +779,6 @@ __device__ __forceinline__ void final_point(const FinalParams& P, int64_t i) {
   int tr;
   point_of(P.perm, P.tid, P.F.n, i, pt, tr);
   if (tr >= P.F.n) return;  // unknown tree: reported by the Newton kernel
-  if (P.status[pt] == STATUS_RETRY) return;
   const TreeDev& t = P.F.t[tr];
   const int part = SPLIT ? blockIdx.y : 0, split = SPLIT ? min(31 - __clz((int)gridDim.y), t.K - 1) : 0;
   if (SPLIT && part >> split) return;   // a shallower tree has fewer parts

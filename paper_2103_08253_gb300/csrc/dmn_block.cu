@@ -1020,6 +1020,8 @@ __global__ void __launch_bounds__(BT, BLOCK_THREADS * BLOCK_CTAS_PER_SM / BT) k_
 // bare components of n; Kn as quadratic forms in n instead of N^T (C N); and, without a Newton step to store,
 // Kn = L D L^T and C -= c1 c2 (B L^-T) D^-1 (B L^-T)^T in place of the inverse and H.  88 k FP64 instructions
 // per point at depth 8 instead of 107 k.
+// Points left to the all-FP64 kernels (RETRY) are skipped; a point that the mixed forms' Newton kernel found not finite
+// gets NaN here, its leaf states in k_final (k_newton_block leaves no such point).
 // STATES: also the leaf states.  The mixed form leaves them to k_final, as its FP32-tangent variant does: the two
 // return the same state bit for bit.
 template <bool CMP, bool STATES>
@@ -1091,14 +1093,6 @@ __global__ void __launch_bounds__(ST, SWEEP_CTAS_PER_SM) k_sweep_block(SweepPara
       normal(q, v);
       condense64(v, q.c2, q.c1 * q.c2, L, R, o, Downdate{});
     };
-    if (STATES && st == DMN_STATUS_NONFINITE) {   // NaN outputs and leaf states; the Newton kernel wrote the jumps
-      for (int l = 0; l < 8; ++l) {
-        const int leaf = 8 * s + l;
-        const int slot = t.ph[l & 1].kind == 0 ? -1 : CMP ? __ldg(t.lslot + leaf) : both ? leaf : leaf >> 1;
-        if (slot < 0) continue;
-        for (int k = 0; k < 6; ++k) zout[(6 * slot + k) * n] = qnan;
-      }
-    }
     if (act && s == 0) {
 #pragma unroll
       for (int I = 0; I < 6; ++I) M.e[I][p] = P.nbuf[(3 * P.N_max + I) * n + pt];
