@@ -415,8 +415,11 @@ def cta_size(n, threads):
 
 
 def sweep_apart(n, sms):
-    """Whether the mixed form's FP64 sweep is a kernel of its own (k_sweep_block) in a call of n points."""
-    return n <= 4096 * sms
+    """Whether the mixed form's FP64 sweep is a kernel of its own (k_sweep_block) in a call of n points of depth 8
+    (sweep_block_on's rule)."""
+    step = 128 * sms
+    steps = -(-n // step)
+    return n <= 4096 * sms and (steps < 4 or 100 * n < 97 * steps * step)
 
 
 def tune_shape(form, ctx, args):

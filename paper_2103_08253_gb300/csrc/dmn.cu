@@ -1362,11 +1362,22 @@ void launch_newton(const NewtonParams<T>& P, bool ls, int minb, unsigned grid, i
   else launch_newton_p<T, CMP, false>(P, ls, minb, grid, block, s);
 }
 
-// Points per SM up to which the mixed form's sweep runs k_sweep_block and a pass of k_final for the leaf states.
-// Above, k_final<sweep> does both in one pass, and its last wave is short beside the others: 100003 points of depth 8
-// 20.3 against 22.4 ms, 200003 40.3 against 41.0, 2^20 208 against 200 ms.  The whole call's size decides, so that
-// the chunks of dmn_update_host get what dmn_update gets.
+// Whether the mixed form's FP64 sweep of a call of n points runs k_sweep_block and a pass of k_final for the leaf
+// states, or k_final<sweep>, which does both, a thread per point.  The latter's time is that of the SM with the
+// most CTAs, 128 points each: at depth 8 3.73 ms for every started 128 points per SM, against 3.85 ms per 128
+// points per SM and no steps.  So k_sweep_block is ahead unless the last step is nearly full (143974 points 28.7
+// against 29.8 ms, 155648 points, 8 full steps, 30.8 against 29.9); the line lies at 0.97.  At depths 4 to 7 its
+// share per point is smaller (depth 6: 3.58 against 3.76 ms per 512 points per SM) and it is ahead at every size
+// tried; at depth 3, a point per thread in both, the fused pass is (8 points 0.130 against 0.123 ms, 200 points 0.139
+// against 0.147, 54476 points 0.38 against 0.50).  Above 4096 points per SM the fused pass.  The whole call's size
+// decides, so that the chunks of dmn_update_host get what dmn_update gets.
 constexpr int SWEEP_BLOCK_MAX = 4096;
+bool sweep_block_on(const dmn_handle* h, int64_t n) {
+  if (!block_trees(h) || h->K_max == 3 || n > (int64_t)SWEEP_BLOCK_MAX * h->n_sm) return false;
+  if (h->K_max < 8) return true;
+  const int64_t step = 128 * (int64_t)h->n_sm, steps = div_up(n, step);
+  return steps < 4 || 100 * n < 97 * steps * step;
+}
 
 // CTAs of 32 threads per SM for a call of n points in the thread-per-point organisation, of at most `warps` per
 // SM, or 0 for the full shape.  With the full shape a call of one to two points per lane ends with its last
@@ -1517,7 +1528,7 @@ int update_on(dmn_handle* h, WorkSet& w, int64_t n, int64_t n_call, const int32_
     const dim3 gl((unsigned)std::min<int64_t>(g1, 2 * h->n_sm), 32);
     if (h->cmp) k_final_list<true><<<gl, 128, 0, s>>>(FP, P.n_list);
     else k_final_list<false><<<gl, 128, 0, s>>>(FP, P.n_list);
-  } else if (sweep && block_trees(h) && n_call <= (int64_t)SWEEP_BLOCK_MAX * h->n_sm) {
+  } else if (sweep && sweep_block_on(h, n_call)) {
     e = sweep_pass(false);
     if (e != cudaSuccess) return cuda_fail(h, e, "dmn_update: launch");
     FP.states_only = 1;

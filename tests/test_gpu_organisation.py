@@ -60,3 +60,28 @@ def test_the_tuner_times_a_kernel_without_a_launch_shape_once(tmp_path, monkeypa
         assert len(made) == handles and len(res["table"]) == 3 and res["used"] == (stage is True)
         if not res["used"]:
             assert (res["block"], res["ctas_per_sm"]) == (128, 2)
+
+
+@pytest.mark.parametrize("apart,fused", [(480, 512), (520, 630)])
+def test_the_mixed_sweeps_two_organisations_agree(apart, fused):
+    """Points per SM on both sides of the rule that chooses the mixed form's sweep at depth 8 (the last 128 points per
+    SM nearly full): the same states and counts bit for bit, stress and tangent to the rounding of two FP64
+    condensations."""
+    n_sm = torch.cuda.get_device_properties(DEV).multi_processor_count
+    sizes, k = (apart * n_sm, fused * n_sm), 512
+    tree = W.tree_d10_fit(8, seed=880)
+    lam, Q, Ef = (d(x) for x in inputs(512, 881))
+    lam, Q, dE = (x.repeat(max(sizes) // 512 + 1, 1) for x in (lam, Q, Ef * 0.1))
+    m = dmn.DMN(tree, precision="mixed", warp_per_point=-1)
+    outs = []
+    for n in sizes:
+        st = torch.zeros((m.state_size, n), dtype=torch.float64, device=DEV)
+        o = m.update(lam[:n].contiguous(), Q[:n].contiguous(), torch.zeros_like(dE[:n]), dE[:n].contiguous(), st)
+        outs.append({key: (v[:, :k] if key == "state_out" else v[:k]).clone() for key, v in o.items()})
+        del o, st
+    for key in ("state_out", "iters", "status"):
+        assert torch.equal(outs[0][key], outs[1][key]), key
+    for key in ("stress", "tangent"):
+        a, b = (o[key].reshape(k, -1) for o in outs)
+        assert ((a - b).norm(dim=1) <= 1e-12 * b.norm(dim=1)).all(), key
+    m.close()
