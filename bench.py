@@ -426,12 +426,12 @@ def tune_shape(form, ctx, args):
     """Launch shape of the Newton kernel from the autotuner, tuned on the first 2^18 points at the
     first timed increment (after the warm-up increments).  Forms that differ only in the start
     share the kernel and its shape; in the FP64 form those that run one point per thread are tuned
-    with the first stage, the others take no shape (None)."""
+    with the first stage, the others take none (0 selects the defaults)."""
     import torch
     from paper_2103_08253_gb300 import autotune, dmn
     form, start = form_opts(form)[0], form.partition("/")[2]
     if form == "f64" and start not in ("stage", "extrap"):
-        return None
+        return dict(block=0, ctas_per_sm=0, stage_ctas_per_sm=0, points=0, table=[], stage_table=[])
     stage = True if form == "f64" else None
     cache = ctx.setdefault("shapes", {})
     if form in cache:
