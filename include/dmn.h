@@ -182,7 +182,9 @@ typedef struct {
                            * The FP64 form of trees of depth 3 or more, without the extrapolated start or the
                            * first stage, runs a third organisation instead, whatever this option says: a
                            * CTA's threads share its points' trees (see DMN_PREC_F64).  It ignores warp_lanes,
-                           * block and ctas_per_sm.  warp_per_point = 1 with warp_lanes given names the warp
+                           * block and ctas_per_sm.  (Up to 8 points of trees no deeper than 3, or 4 with an
+                           * exponential-linear phase, run the warp organisation unless -1 is given:
+                           * dmn_update_cta_threads.)  warp_per_point = 1 with warp_lanes given names the warp
                            * organisation, and runs it: the all-FP64 iteration. */
   int32_t warp_lanes;     /* lanes per point in the warp organisation: 32 (one point per warp), 16 or 8 (two
                            * or four points per warp, side by side); 0 (default) chooses by the call's

@@ -1282,9 +1282,22 @@ bool block_trees(const dmn_handle* h) {
     if (t.K < 3 || t.N < 1) return false;
   return true;
 }
-bool block_on(const dmn_handle* h) {
+// whether the handle holds the CTA organisation's scratch, and whether a call of n points runs it.  The smallest calls
+// of the shallowest trees do not: up to 8 points (one element) at depth 3, where a thread walks a whole tree, and
+// at depth 4 with an exponential-linear phase, whose scalar iterations one thread runs in turn, 32 lanes per point
+// are ahead.  8 points: depth 3 0.35 against 0.40 ms, exponential-linear 0.47 against 0.66; depth 4
+// exponential-linear 0.57 against 0.65, linear 0.48 against 0.45.  32 points of depth 3: 0.53 against 0.45.
+constexpr int64_t WARP_SMALLEST = 8;
+bool block_handle(const dmn_handle* h) {
   const bool warp_asked = h->opt.warp_per_point == 1 && h->opt.warp_lanes;   // the warp organisation, by name
   return h->opt.precision == DMN_PREC_F64 && !h->opt.predictor && !first_stage_on(h->opt) && !warp_asked && block_trees(h);
+}
+bool block_on(const dmn_handle* h, int64_t n) {
+  if (!block_handle(h)) return false;
+  if (n > WARP_SMALLEST || h->K_max > 4 || h->opt.warp_per_point < 0) return true;
+  for (const Tree& t : h->trees)
+    if (t.ph[0].kind == DMN_PHASE_J2_EXPLIN || t.ph[1].kind == DMN_PHASE_J2_EXPLIN) return false;
+  return h->K_max == 4;
 }
 int block_leaf_slots(const dmn_handle* h) {
   for (const Tree& t : h->trees)
@@ -1296,7 +1309,7 @@ int block_leaf_slots(const dmn_handle* h) {
 cudaError_t alloc_ws(const dmn_handle* h, WorkSet& w) {
   // per slot: normals + one or two jump buffers (FP64); one or two g, H buffers + FP32 normals
   const size_t sd = h->opt.line_search ? 9 : 6, stt = h->opt.line_search ? 45 : 24;
-  const bool block = block_on(h);   // runs no thread-per-point kernel: 3.6 GB less at depth 8
+  const bool block = block_handle(h);   // runs no thread-per-point kernel: 3.6 GB less at depth 8
   cudaError_t e = cudaSuccess;
   if (!block) e = cudaMalloc(&w.scr_d, sizeof(double) * (size_t)(sd * h->N_max) * h->nslots);
   if (e == cudaSuccess && !block) e = cudaMalloc(&w.scr_t, sizeof(double) * (size_t)(stt * h->N_max) * h->nslots);
@@ -1458,7 +1471,7 @@ int update_on(dmn_handle* h, WorkSet& w, int64_t n, int64_t n_call, const int32_
   const bool warp = warp_on(h, n_call) && w.scr_w;
   const bool stage = first_stage_on(h->opt) && !warp;   // a small batch goes straight to the warp kernel
   const unsigned wgrid = (unsigned)(h->n_sm * WARP_CTAS_PER_SM);
-  const bool block = w.scr_b != nullptr;
+  const bool block = block_on(h, n_call);
   const int lanes = warp ? warp_lanes_for(h, n_call) : 32;
   unsigned long long* passes = h->profiling ? h->d_passes : nullptr;
   if (stage) {   // counter [19]: the first stage's work counter
@@ -1794,7 +1807,7 @@ int dmn_update_lanes_per_point(const dmn_handle* h, int64_t n) {
 
 int dmn_update_cta_threads(const dmn_handle* h, int64_t n) {
   if (!h || n < 0) return -1;
-  return block_on(h) ? 1 << (h->K_max - 3) : 0;
+  return block_on(h, n) ? 1 << (h->K_max - 3) : 0;
 }
 
 int dmn_profile_enable(dmn_handle* h, int32_t enable) {

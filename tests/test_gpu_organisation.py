@@ -85,3 +85,26 @@ def test_the_mixed_sweeps_two_organisations_agree(apart, fused):
         a, b = (o[key].reshape(k, -1) for o in outs)
         assert ((a - b).norm(dim=1) <= 1e-12 * b.norm(dim=1)).all(), key
     m.close()
+
+
+@pytest.mark.parametrize("K,explin,opts,small,larger", [(3, False, {}, 0, 1), (3, True, {}, 0, 1), (4, True, {}, 0, 2),
+                                                        (4, False, {}, 2, 2), (5, True, {}, 4, 4),
+                                                        (3, True, dict(warp_per_point=-1), 1, 1),
+                                                        (3, False, dict(line_search=True), 0, 1)])
+def test_one_elements_points_at_shallow_depth(K, explin, opts, small, larger):
+    """Up to 8 points the warp organisation at depth 3, and 4 with an exponential-linear phase: the results of the
+    same points in a call of 9, to rounding."""
+    tree = W.tree_d10_fit(K, seed=890 + K, phases=(W.FIBER, W.MATRIX_EXPLIN if explin else W.MATRIX))
+    lam, Q, Ef = (d(x) for x in inputs(9, 891))
+    m = dmn.DMN(tree, **opts)
+    assert m.cta_threads(8) == small and m.cta_threads(9) == larger
+    outs = []
+    for n in (9, 8, 1):
+        st = torch.zeros((m.state_size, n), dtype=torch.float64, device=DEV)
+        outs.append(m.update(lam[:n], Q[:n], torch.zeros_like(Ef[:n]), Ef[:n] * 0.1, st))
+    for o, n in zip(outs[1:], (8, 1)):
+        assert torch.equal(o["status"], outs[0]["status"][:n]) and torch.equal(o["iters"], outs[0]["iters"][:n])
+        for key in ("stress", "tangent", "state_out"):
+            a, b = o[key], outs[0][key][:, :n] if key == "state_out" else outs[0][key][:n]
+            assert (a - b).norm() <= 1e-10 * b.norm(), key
+    m.close()
