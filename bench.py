@@ -103,6 +103,11 @@ F_LEAF_EL, F_LEAF_J2, F_TEST = 13, 56 + 12, 15
 F_ROTATE = 1150         # per point: stress and tangent back to the global frame (k_final)
 F_STATE_NODE = 39       # state pass: per laminate (strains from the jumps)
 F_STATE_J2 = 68         # state pass: per J2 leaf (return mapping and new state)
+# k_sweep_block (csrc/dmn_block.cuh), all FP64: condensation of an inner laminate (average stress 18, C_R - C_L and the
+# two averages 105, acoustic tensor 84, B 90, L D L^T 22, B L^-T 36, rank-3 downdate 144) and of a bottom laminate
+# with an elastic and an inelastic leaf (18 + 41 for the isotropic parts + 130 for the inelastic leaf + 202); with
+# the states a J2 leaf's new state 12
+F_SWEEP, F_SWEEP_BOTTOM, F_SWEEP_STATE = 499, 391, 12
 
 
 F_LEAF_SUB = 84         # a leaf whose sibling is a laminate: its 21 tangent entries as a subtree (T)
@@ -185,6 +190,14 @@ def block_flops(K, iters_sum, npts, w=None):
     f64, ft = pass_flops(K, w, t_is_f64=False)
     c64, ct = corr_flops(K, w)
     return (iters_sum + npts) * f64 + iters_sum * c64, iters_sum * (ft + f64 + 2 * ct)
+
+
+def sweep_flops(K, npts, states, w=None):
+    """FP64 flops of k_sweep_block over npts points: strains down, leaf laws (and, with `states`, their new states),
+    condensation in its shortest form, rotation of the outputs."""
+    c = tree_counts(np.ones(1 << K) if w is None else w)
+    return npts * (c["N"] * F_NODE_F64 + c["inner"] * F_SWEEP + c["pairs"] * F_SWEEP_BOTTOM + c["single"] * F_LEAF_SUB
+                   + c["el"] * F_LEAF_EL + c["j2"] * (F_LEAF_J2 + (F_SWEEP_STATE if states else 0)) + F_ROTATE)
 
 
 def final_flops(K, npts, sweep, w=None):
@@ -634,7 +647,7 @@ def roofline_f64(r, n, steps, w=None, peaks=None):
         F64, F32 = block_flops(K_DEPTH, corr, npts, w=w)
         t = r["kms"]["newton"] * 1e-3
         tb = F64 / (P64 * 1e9) + F32 / (pk["f32"] * 1e9)
-        Ff = final_flops(K_DEPTH, npts, sweep=True, w=w)
+        Ff = sweep_flops(K_DEPTH, npts, states=True, w=w)
         tf = r["kms"]["final"] * 1e-3
         cmp = "_compressed" if w is not None and (np.asarray(w) == 0).any() else ""
         return {"bound": "alu", "kernel": "k_newton_block", "achieved": tb / t * P64, "peak": P64,
@@ -684,10 +697,16 @@ def roofline_mixed(r, n, steps, w=None, sweep=True, peaks=None):
     F64, F32 = newton_flops(K_DEPTH, newton_corr, npts, mixed=True, w=w)
     t = r["kms"]["newton"] * 1e-3
     tb = F64 / (P64 * 1e9) + F32 / (P32 * 1e9)
-    Ff = final_flops(K_DEPTH, n * steps, sweep=sweep, w=w)
+    apart = sweep and sweep_apart(n, r.get("n_sm", 152))
+    if apart:       # the sweep, then the state pass
+        Ff = sweep_flops(K_DEPTH, n * steps, states=False, w=w) + final_flops(K_DEPTH, n * steps, False, w=w) \
+            - n * steps * F_ROTATE
+    else:
+        Ff = final_flops(K_DEPTH, n * steps, sweep=sweep, w=w)
     tf = r["kms"]["final"] * 1e-3
-    fin = {"kernel": ("k_sweep_block, k_final" if sweep_apart(n, r.get("n_sm", 152)) else "k_final<sweep>") if sweep else "k_final", "achieved": Ff / tf / 1e9, "peak": P64,
-           "unit": "GFLOP/s (FP64)", "frac": Ff / tf / 1e9 / P64, "launch_ms": r["kms"]["final"] / steps}
+    fin = {"kernel": "k_sweep_block, k_final" if apart else "k_final<sweep>" if sweep else "k_final",
+           "achieved": Ff / tf / 1e9, "peak": P64, "unit": "GFLOP/s (FP64)", "frac": Ff / tf / 1e9 / P64,
+           "launch_ms": r["kms"]["final"] / steps}
     cmp = "_compressed" if w is not None and (np.asarray(w) == 0).any() else ""
     stg = "stage" in r["kms"]
     org = "_warp" if r.get("warp") else ""
