@@ -1294,7 +1294,7 @@ bool block_handle(const dmn_handle* h) {
 }
 bool block_on(const dmn_handle* h, int64_t n) {
   if (!block_handle(h)) return false;
-  if (n > WARP_SMALLEST || h->K_max > 4 || h->opt.warp_per_point < 0) return true;
+  if (n > WARP_SMALLEST || h->K_max > 4 || !warp_on(h, n)) return true;   // no thread-per-point scratch here
   for (const Tree& t : h->trees)
     if (t.ph[0].kind == DMN_PHASE_J2_EXPLIN || t.ph[1].kind == DMN_PHASE_J2_EXPLIN) return false;
   return h->K_max == 4;
@@ -1417,6 +1417,9 @@ int update_on(dmn_handle* h, WorkSet& w, int64_t n, int64_t n_call, const int32_
   cudaError_t e;
   const int NM = h->N_max;
   const bool sort = tree_id && h->trees.size() > 1;
+  const bool block = block_on(h, n_call), warp = !block && warp_on(h, n_call);
+  if (block ? !w.scr_b || !w.scr_w : warp ? !w.scr_w : !w.scr_d)
+    return fail(h, DMN_ERR_CUDA, "dmn_update: the handle holds no work space for this organisation");
   if (n > w.nbuf_cap) {
     e = cudaStreamSynchronize(s);
     if (e == cudaSuccess) {
@@ -1468,10 +1471,8 @@ int update_on(dmn_handle* h, WorkSet& w, int64_t n, int64_t n_call, const int32_
   const unsigned even = mixed && h->own_shape && !ls ? even_warps_per_sm(n, h->n_sm, threads_per_sm / 32, 2) : 0;
   const unsigned grid = (unsigned)h->n_sm * (even ? even : (unsigned)h->opt.ctas_per_sm);
   const int cta = even ? 32 : h->opt.block;
-  const bool warp = warp_on(h, n_call) && w.scr_w;
   const bool stage = first_stage_on(h->opt) && !warp;   // a small batch goes straight to the warp kernel
   const unsigned wgrid = (unsigned)(h->n_sm * WARP_CTAS_PER_SM);
-  const bool block = block_on(h, n_call);
   const int lanes = warp ? warp_lanes_for(h, n_call) : 32;
   unsigned long long* passes = h->profiling ? h->d_passes : nullptr;
   if (stage) {   // counter [19]: the first stage's work counter

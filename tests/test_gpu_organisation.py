@@ -90,7 +90,9 @@ def test_the_mixed_sweeps_two_organisations_agree(apart, fused):
 @pytest.mark.parametrize("K,explin,opts,small,larger", [(3, False, {}, 0, 1), (3, True, {}, 0, 1), (4, True, {}, 0, 2),
                                                         (4, False, {}, 2, 2), (5, True, {}, 4, 4),
                                                         (3, True, dict(warp_per_point=-1), 1, 1),
-                                                        (3, False, dict(line_search=True), 0, 1)])
+                                                        (3, False, dict(line_search=True), 0, 1),
+                                                        # first_stage = 1 turns the warp organisation's default off
+                                                        (3, True, dict(line_search=True, first_stage=True), 1, 1)])
 def test_one_elements_points_at_shallow_depth(K, explin, opts, small, larger):
     """Up to 8 points the warp organisation at depth 3, and 4 with an exponential-linear phase: the results of the
     same points in a call of 9, to rounding."""
