@@ -83,8 +83,8 @@ enum { DMN_PHASE_ELASTIC = 0, DMN_PHASE_J2_LINEAR = 1, DMN_PHASE_J2_EXPLIN = 2 }
  * that the step's relative error is about the square of the FP32 solve's (1e-11 on the plastic paths
  * measured).  A point whose first solve leaves more than 1e-3 of the residual (the step's error is then
  * bounded by 1e-6 of it), which is not finite or not converged after 16 corrections starts again in the
- * all-FP64 iteration.  A residual that meets the criterion may hold, below tol, what the refinement left of
- * the last step.
+ * all-FP64 iteration.  What the refinement left of a step that no quadratic term hides is solved for once
+ * more, so that results are as accurate as the all-FP64 solve's.
  * DMN_PREC_MIXED: leaf tangents, laminate condensation and jump corrections
  * in FP32; leaf stresses, strains, jumps, the Newton residual and the final
  * sweep that yields stress and tangent in FP64.
@@ -131,9 +131,9 @@ typedef struct {
 typedef struct {
   double tol;          /* ||A^T W sigma|| / ((2^K - 1) ||sigma_bar||) <= tol (Sec. 4.6); <= 0 selects 1e-12 */
   int32_t max_iter;    /* Newton corrections before status MAXITER; <= 0 selects 50.  Where the FP64 form's
-                        * refined step leaves a residual above tol no larger than 4 times its own linear
-                        * system's, a further solve finishes that step; neither max_iter nor iters nor the
-                        * pass counters count it apart, and one may follow the last correction */
+                        * refined step leaves a residual no larger than 4 times its own linear system's, a
+                        * further solve finishes that step; neither max_iter nor iters nor the pass
+                        * counters count it apart, and one may follow the last correction */
   int32_t precision;   /* DMN_PREC_F64, DMN_PREC_MIXED or DMN_PREC_MIXED_F32_TANGENT */
   int32_t block;       /* threads per CTA of the thread-per-point Newton kernel (multiple of 32); 0 selects 128 */
   int32_t ctas_per_sm; /* resident CTAs per SM of that persistent kernel; 0 selects 384 threads

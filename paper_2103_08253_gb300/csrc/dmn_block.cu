@@ -7,9 +7,10 @@
 //   S  condenses the leaf tangents in FP32 and solves for da1 (relative error some 1e-6),
 //   B  forms R + J da1 with pairs of FP32 numbers (about 46 bits) and solves again in FP32 for da2,
 // and applies da = da1 + da2, whose relative error is the product of the two solves' (1e-11, at most
-// some 1e-10 on the workloads' plastic paths).  Where a large step ends in a fixed set of plastic leaves, no
-// quadratic term hides what the solves left of its linear residual: a residual above the criterion but no larger
-// than that is taken off by a further round that belongs to the same step and is not counted.  So the iterates
+// some 1e-10 on the workloads' plastic paths).  Where a large step ends in a fixed set of plastic leaves, or in none,
+// no quadratic term hides what the solves left of its linear residual: a residual no larger than that is taken off
+// by a further round that belongs to the same step and is not counted, also below the criterion (an elastic
+// point's stress is then 5e-16 from the exact one as with the all-FP64 solve, 5e-14 without).  So the iterates
 // are those of the all-FP64 condensation, with its iteration counts.  A costs about 21 k FP64 instructions, a
 // pass of the all-FP64 kernel 122 k; S and B cost none.  The tangent comes from one FP64
 // sweep at the converged jumps, as in the mixed form.
@@ -44,6 +45,11 @@ namespace {
 constexpr float REFINE_MAX = 1e-3f;
 // A residual this many times what the solves left of the last step's linear system, or less, belongs to that step
 constexpr double LEFT_MAX = 4.0;
+// and is taken off also where it meets the criterion, unless it is at the rounding of FP64 stresses (times the root's)
+constexpr double ROUNDING = 1e-15;
+// What the second solve leaves at least, as a part of the residual it starts from: the pairs' 46 bits, less some for
+// the sums that cancel.
+constexpr double PAIR_LEFT = 9.1e-13;   // 2^-40
 constexpr int BLOCK_ITERS = 16;
 
 // scratch fields of a thread, in units of 8 laminates (7 of the subtree, then the top laminate)
@@ -643,6 +649,7 @@ static __device__ void newton(const BlockParams& P) {
     int it = 0, halv = 0, np = 0;
     double rn_acc = 0.0, left = 0.0;
     bool again = false;   // a step in two parts (LEFT_MAX)
+    bool met = false;     // whose first part met the criterion
     bool more = tid < nP;
     if (tid < nP) sh_fl[tid] = 0;
     if (tid == 0) M.n_in = 0;
@@ -656,7 +663,7 @@ static __device__ void newton(const BlockParams& P) {
           int64_t x;
           point_of(P.perm, P.tid, P.F.n, (int64_t)i, x, tt);
           if (tt == tr) {
-            pt = x; it = 0; halv = 0; np = 0; rn_acc = 0.0; left = 0.0; again = false;
+            pt = x; it = 0; halv = 0; np = 0; rn_acc = 0.0; left = 0.0; again = met = false;
             sh_pt[tid] = pt; sh_st[tid] = 1.f;
             sh_fl[tid] = B_ACT | B_FIRST;
             M.in[atomicAdd(&M.n_in, 1)] = (short)tid;
@@ -812,12 +819,15 @@ static __device__ void newton(const BlockParams& P) {
           if (LS) { f ^= B_CUR; sh_st[tid] = 1.f; halv = 0; }
           rn_acc = rn;
           f &= ~B_FIRST;
+          const bool crit = rn <= P.tol * (double)t.N * sn, rest = !again && rn <= LEFT_MAX * left;
           if (!isfinite(rn) || !isfinite(sn)) retry = true;
-          else if (rn <= P.tol * (double)t.N * sn) st = DMN_STATUS_OK;
-          else if (!again && rn <= LEFT_MAX * left) { again = true; f |= B_CONT; }
+          else if (crit && !(rest && rn > ROUNDING * sn)) st = DMN_STATUS_OK;
+          else if (rest) { again = true; met = crit; f |= B_CONT; }
           else if (it >= P.max_iter) st = DMN_STATUS_MAXITER;
           else if (it >= BLOCK_ITERS) retry = true;
-          else { ++it; again = false; f |= B_CONT; }
+          else { ++it; again = met = false; f |= B_CONT; }
+        } else if (met) {
+          st = DMN_STATUS_OK;   // at its rounding: the accepted iterate stands
         } else if (++halv > 8) {
           st = DMN_STATUS_LINESEARCH;   // no halving lowered the residual: the accepted iterate stands
           ++it;
@@ -983,7 +993,7 @@ static __device__ void newton(const BlockParams& P) {
           double r = 0.0;
           for (int k = 0; k < groups; ++k) r += sh_r[k * nP + tid];
           r = sqrt(r);                 // of the linear residual; the second solve leaves about r / rn_acc of it
-          left = r * (r / rn_acc);
+          left = fmax(r * (r / rn_acc), PAIR_LEFT * rn_acc);
           if (!(r <= (double)REFINE_MAX * rn_acc)) {
             block_retry(P, pt);
             f = 0;
