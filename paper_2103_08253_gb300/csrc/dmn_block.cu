@@ -9,8 +9,10 @@
 // and applies da = da1 + da2, whose relative error is the product of the two solves' (1e-11, at most
 // some 1e-10 on the workloads' plastic paths).  Where a large step ends in a fixed set of plastic leaves, or in none,
 // no quadratic term hides what the solves left of its linear residual: a residual no larger than that is taken off
-// by a further round that belongs to the same step and is not counted, also below the criterion (an elastic
-// point's stress is then 5e-16 from the exact one as with the all-FP64 solve, 5e-14 without).  So the iterates
+// by a second part of the same step, which is not counted, also below the criterion (an elastic point's stress is
+// then 5e-16 from the exact one as with the all-FP64 solve, 5e-14 without).  Below the criterion and with all leaves
+// elastic it keeps the condensed tangents, solves once, R alone, and ends with the jumps, without S and another A
+// (155000 elastic points of depth 8: 62.4 -> 54.7 ms, 52.2 without the second part).  So the iterates
 // are those of the all-FP64 condensation, with its iteration counts.  A costs about 21 k FP64 instructions, a
 // pass of the all-FP64 kernel 122 k; S and B cost none.  The tangent comes from one FP64
 // sweep at the converged jumps, as in the mixed form.
@@ -90,7 +92,7 @@ __device__ __forceinline__ pair split(double x) {
 }  // namespace
 
 // flags of a slot
-enum { B_ACT = 1, B_FIRST = 4, B_CONT = 8, B_CONV = 16, B_CUR = 32 };
+enum { B_ACT = 1, B_FIRST = 4, B_CONT = 8, B_CONV = 16, B_CUR = 32, B_LAST = 64 };
 
 // The Newton kernel for CTAs of BT threads.  A point's results do not depend on BT, bit for bit.
 template <int BT>
@@ -173,14 +175,40 @@ static __device__ __forceinline__ void down_a(const TreeDev& t, const Ctx& c, in
   for (int I = 0; I < 6; ++I) { eL[I] = e[I] - q.c2 * Na[I]; eR[I] = e[I] + q.c1 * Na[I]; }
 }
 
+// The last solve's correction of laminate j's jumps (at f), and its strains in the children (as in down_a).
+template <bool CMP>
+static __device__ __forceinline__ void down_last(const TreeDev& t, const Ctx& c, int h, int j, int f, const float de[6],
+                                          float* dL, float* dR) {
+  const Lam<CMP> q(t, h);
+  if (CMP && q.mode) {
+    if (dL) {
+#pragma unroll
+      for (int I = 0; I < 6; ++I) dL[I] = dR[I] = de[I];
+    }
+    return;
+  }
+  float da[3];
+  step32(c, j, de, da);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) c.d(f + k, j) += widen(da[k]);
+  if (!dL) return;
+  const float c1 = __ldg(t.c1f + q.id), c2 = __ldg(t.c2f + q.id);
+  float n[3], Nd[6];
+  normal32(c, j, n);
+  N_apply<float>(n, n, da, Nd);
+#pragma unroll
+  for (int I = 0; I < 6; ++I) { dL[I] = de[I] - c2 * Nd[I]; dR[I] = de[I] + c1 * Nd[I]; }
+}
+
 static __device__ __forceinline__ void pair_normal(const Ctx& c, int j, pair n[3]) {
 #pragma unroll
   for (int k = 0; k < 3; ++k) n[k] = split(c.d(D_N + k, j));
 }
 
-// B, downwards: the step da1 of laminate j stored, and its strains in the children.
+// B, downwards: the step da1 of laminate j stored, and its strains in the children.  Without `first` there is no
+// first solve: da1 = 0.
 template <bool CMP>
-static __device__ __forceinline__ void down_b(const TreeDev& t, const Ctx& c, int h, int j, const pair e[6],
+static __device__ __forceinline__ void down_b(const TreeDev& t, const Ctx& c, int h, int j, bool first, const pair e[6],
                                        pair eL[6], pair eR[6]) {
   const Lam<CMP> q(t, h);
   if (CMP && q.mode) {
@@ -188,10 +216,10 @@ static __device__ __forceinline__ void down_b(const TreeDev& t, const Ctx& c, in
     for (int I = 0; I < 6; ++I) eL[I] = eR[I] = e[I];
     return;
   }
-  float de[6], x[3];
+  float de[6], x[3] = {0.f, 0.f, 0.f};
 #pragma unroll
   for (int I = 0; I < 6; ++I) de[I] = e[I].h;
-  step32(c, j, de, x);
+  if (first) step32(c, j, de, x);
 #pragma unroll
   for (int k = 0; k < 3; ++k) c.f(F_D + k, j) = x[k];
   pair n[3];
@@ -446,14 +474,14 @@ static __device__ __forceinline__ void condense32_bottom(const TreeDev& t, const
 
 // A, the leaf: stress from the strain e and the state z (shear entries times 1 / sqrt 2), the law of leaf_iso in
 // Voigt components; the tangent mu, c, m for S and B goes to T as pairs, formed in pairs from FP64 xi, 1 / |xi| and
-// k2.  An elastic leaf's tangent is its phase's.
-static __device__ __forceinline__ void leaf_a(const PhaseDev& ph, const double e[6], const double* zp, double sig[6], float* T) {
+// k2.  An elastic leaf's tangent is its phase's.  Returns whether the leaf is plastic.
+static __device__ __forceinline__ bool leaf_a(const PhaseDev& ph, const double e[6], const double* zp, double sig[6], float* T) {
   const double tr = e[0] + e[1] + e[2];
   if (ph.kind == 0) {
     const double lt = ph.lam * tr, g2 = 2.0 * ph.G;
 #pragma unroll
     for (int I = 0; I < 6; ++I) sig[I] = I < 3 ? g2 * e[I] + lt : ph.G * e[I];
-    return;
+    return false;
   }
   double z[6];
 #pragma unroll
@@ -500,6 +528,7 @@ static __device__ __forceinline__ void leaf_a(const PhaseDev& ph, const double e
     v = mul(split(xi[k]), ix);
     T[(2 + k) * BT] = v.h; T[(10 + k) * BT] = v.l;
   }
+  return plastic;
 }
 
 // D e of a leaf in pairs (B): the phase's constants or the stored mu, c, m
@@ -569,6 +598,7 @@ struct BlockShared {
   long long pt[BT];
   int fl[BT];
   float st[BT];
+  int pl[BT];            // the point has a plastic leaf in this round
   int n_in, n_out;       // slots that take a point in / hand one out in this round
   short in[BT], out[BT];
 };
@@ -612,6 +642,7 @@ static __device__ void newton(const BlockParams& P) {
   long long* const sh_pt = M.pt;
   int* const sh_fl = M.fl;
   float* const sh_st = M.st;
+  int* const sh_pl = M.pl;
   const int tid = threadIdx.x;
   const size_t n = (size_t)P.n;
   unsigned long long* const tok = token(P);
@@ -650,6 +681,27 @@ static __device__ void newton(const BlockParams& P) {
     double rn_acc = 0.0, left = 0.0;
     bool again = false;   // a step in two parts (LEFT_MAX)
     bool met = false;     // whose first part met the criterion
+    bool linear = false;  // all leaves elastic in the step's condensation
+    // a point that is done: its counts, and its jumps in the state's order (by the CTA)
+    auto done = [&](int st) {
+      P.iters[pt] = it;
+      P.status[pt] = st;
+      if (P.passes) atomicAdd(P.passes, (unsigned long long)np);
+      M.out[atomicAdd(&M.n_out, 1)] = (short)tid;
+    };
+    auto write_out = [&]() {
+      for (int i = tid; i < M.n_out << K; i += BT) {
+        const int x = M.out[i >> K], h = i & (t.L - 1);
+        const int row = h == t.L - 1 ? -1 : CMP ? __ldg(t.hcid + h) : (1 << K) - 3 * (1 << (31 - __clz(h + 1))) + h + 1;
+        if (row < 0) continue;
+        int os, oj;
+        owner(h, Kt, os, oj);
+        const double* w = D0 + 8 * (LS && (sh_fl[x] & B_CUR) ? D_A2 : D_A) * BT + oj * BT + os * nP + x;
+        double* st = P.state_out + (nzf + 3 * row) * n + (size_t)sh_pt[x];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) st[k * n] = w[8 * k * BT];
+      }
+    };
     bool more = tid < nP;
     if (tid < nP) sh_fl[tid] = 0;
     if (tid == 0) M.n_in = 0;
@@ -672,6 +724,7 @@ static __device__ void newton(const BlockParams& P) {
           block_bad_tree(P, x);
         }
       }
+      if (tid < nP) sh_pl[tid] = 0;
       const bool any = tid < nP && (sh_fl[tid] & B_ACT);
       if (!__syncthreads_or(any)) break;
       int fl = sh_fl[p];
@@ -758,7 +811,7 @@ static __device__ void newton(const BlockParams& P) {
 #pragma unroll
           for (int side = 0; side < 2; ++side) {
             const int ls = both ? 2 * q + side : q;
-            leaf_a(t.ph[side], side ? eR : eL, c.z + 6 * ls * BT, side ? s1 : s0, c.tan + 16 * ls * BT);
+            if (leaf_a(t.ph[side], side ? eR : eL, c.z + 6 * ls * BT, side ? s1 : s0, c.tan + 16 * ls * BT)) sh_pl[p] = 1;
           }
           up_a<CMP>(t, c, heap(3 + q), 3 + q, s0, s1, sb, r2);
           if (!(q & 1)) {
@@ -822,10 +875,11 @@ static __device__ void newton(const BlockParams& P) {
           const bool crit = rn <= P.tol * (double)t.N * sn, rest = !again && rn <= LEFT_MAX * left;
           if (!isfinite(rn) || !isfinite(sn)) retry = true;
           else if (crit && !(rest && rn > ROUNDING * sn)) st = DMN_STATUS_OK;
-          else if (rest) { again = true; met = crit; f |= B_CONT; }
+          else if (rest) { again = true; met = crit; f |= crit && linear && !sh_pl[tid] ? B_CONT | B_LAST : B_CONT; }
           else if (it >= P.max_iter) st = DMN_STATUS_MAXITER;
           else if (it >= BLOCK_ITERS) retry = true;
           else { ++it; again = met = false; f |= B_CONT; }
+          linear = !sh_pl[tid];
         } else if (met) {
           st = DMN_STATUS_OK;   // at its rounding: the accepted iterate stands
         } else if (++halv > 8) {
@@ -837,10 +891,7 @@ static __device__ void newton(const BlockParams& P) {
         if (retry) { block_retry(P, pt); f = 0; }
         if (st >= 0) {
           f |= B_CONV;
-          P.iters[pt] = it;
-          P.status[pt] = st;
-          if (P.passes) atomicAdd(P.passes, (unsigned long long)np);
-          M.out[atomicAdd(&M.n_out, 1)] = (short)tid;
+          done(st);
           f &= ~B_ACT;
         }
         sh_fl[tid] = f;
@@ -848,24 +899,14 @@ static __device__ void newton(const BlockParams& P) {
       __syncthreads();
       fl = sh_fl[p];
       if (tid == 0) M.n_in = 0;
-      for (int i = tid; i < M.n_out << K; i += BT) {   // the converged jumps, in the state's order
-        const int x = M.out[i >> K], h = i & (t.L - 1);
-        const int row = h == t.L - 1 ? -1 : CMP ? __ldg(t.hcid + h) : (1 << K) - 3 * (1 << (31 - __clz(h + 1))) + h + 1;
-        if (row < 0) continue;
-        int os, oj;
-        owner(h, Kt, os, oj);
-        const double* w = D0 + 8 * (LS && (sh_fl[x] & B_CUR) ? D_A2 : D_A) * BT + oj * BT + os * nP + x;
-        double* st = P.state_out + (nzf + 3 * row) * n + (size_t)sh_pt[x];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) st[k * n] = w[8 * k * BT];
-      }
-      const bool cont = fl & B_CONT;
+      write_out();
+      const bool cont = fl & B_CONT, last = fl & B_LAST, solve = cont && !last;
       if (!__syncthreads_or(cont)) {
         if (tid < nP) sh_fl[tid] &= ~B_CONV;
         continue;
       }
       // ---- S: FP32 condensation up
-      if (cont && !dead) {
+      if (solve && !dead) {
         Sub32 res, sib, o;
 #pragma unroll 1
         for (int q = 0; q < 4; ++q) {
@@ -885,13 +926,13 @@ static __device__ void newton(const BlockParams& P) {
         get27(sh_c, tid, sib);
         condense32<CMP>(t, c, heap(0), 0, sib, o, res);
         put27(sh_c, tid, res);
-      } else if (cont) {
+      } else if (solve) {
 #pragma unroll
         for (int k = 0; k < 27; ++k) sh_c[k][tid] = 0.f;
       }
       __syncthreads();
       for (int l = Kt - 1; l >= 0; --l) {
-        if (cont && lev == l) {
+        if (solve && lev == l) {
           Sub32 L, R, o;
           get27(sh_c, pos, L);
           get27(sh_c, pos + half, R);
@@ -910,7 +951,7 @@ static __device__ void newton(const BlockParams& P) {
         if (cont && lev == l) {
           pair e[6], eL[6], eR[6];
           get6(sh_p, pos, e);
-          down_b<CMP>(t, c, s - 1, 7, e, eL, eR);
+          down_b<CMP>(t, c, s - 1, 7, solve, e, eL, eR);
           put6(sh_p, pos, eL); put6(sh_p, pos + half, eR);
         }
         __syncthreads();
@@ -920,7 +961,7 @@ static __device__ void newton(const BlockParams& P) {
         pair e[6], eL[6], eR[6], t0[6], t1[6];
         float x0[6], x1[6];
         get6(sh_p, tid, e);
-        down_b<CMP>(t, c, heap(0), 0, e, eL, eR);
+        down_b<CMP>(t, c, heap(0), 0, solve, e, eL, eR);
         put6(sh_p, tid, eR);
 #pragma unroll
         for (int I = 0; I < 6; ++I) e[I] = eL[I];
@@ -928,12 +969,12 @@ static __device__ void newton(const BlockParams& P) {
         for (int q = 0; q < 4; ++q) {
           const int mid = 1 + (q >> 1);
           if (!(q & 1)) {
-            down_b<CMP>(t, c, heap(mid), mid, e, eL, eR);
+            down_b<CMP>(t, c, heap(mid), mid, solve, e, eL, eR);
             put6(M.s, tid, eR);
 #pragma unroll
             for (int I = 0; I < 6; ++I) e[I] = eL[I];
           }
-          down_b<CMP>(t, c, heap(3 + q), 3 + q, e, eL, eR);
+          down_b<CMP>(t, c, heap(3 + q), 3 + q, solve, e, eL, eR);
           leaf_apply(t.ph[0], c.tan + 16 * (both ? 2 * q : q) * BT, eL, t0);
           leaf_apply(t.ph[1], c.tan + 16 * (both ? 2 * q + 1 : q) * BT, eR, t1);
           up_b<CMP, true>(t, c, heap(3 + q), 3 + q, t0, t1, nullptr, nullptr, eL, x1, q2);
@@ -989,7 +1030,7 @@ static __device__ void newton(const BlockParams& P) {
       __syncthreads();
       if (tid < nP) {
         int f = sh_fl[tid] & ~B_CONV;
-        if (f & B_CONT) {
+        if ((f & B_CONT) && !last) {
           double r = 0.0;
           for (int k = 0; k < groups; ++k) r += sh_r[k * nP + tid];
           r = sqrt(r);                 // of the linear residual; the second solve leaves about r / rn_acc of it
@@ -1001,6 +1042,52 @@ static __device__ void newton(const BlockParams& P) {
         }
         sh_fl[tid] = f;
       }
+      // ---- an elastic point's second part ends with the jumps: no more A
+      if (!__syncthreads_or(last)) continue;
+      const int buf = LS && (fl & B_CUR) ? D_A2 : D_A;
+      if (tid == 0) M.n_out = 0;
+      if (last && s == 0) {
+#pragma unroll
+        for (int I = 0; I < 6; ++I) sd[I][p] = 0.f;
+      }
+      __syncthreads();
+      for (int l = 0; l < Kt; ++l) {
+        if (last && lev == l) {
+          float de[6], dL[6], dR[6];
+          get6(sd, pos, de);
+          down_last<CMP>(t, c, s - 1, 7, buf, de, dL, dR);
+          put6(sd, pos, dL); put6(sd, pos + half, dR);
+        }
+        __syncthreads();
+      }
+      if (last && !dead) {
+        float de[6], dL[6], dR[6];
+        get6(sd, tid, de);
+        down_last<CMP>(t, c, heap(0), 0, buf, de, dL, dR);
+        put6(sd, tid, dR);
+#pragma unroll
+        for (int I = 0; I < 6; ++I) de[I] = dL[I];
+#pragma unroll 1
+        for (int q = 0; q < 4; ++q) {
+          const int mid = 1 + (q >> 1);
+          if (!(q & 1)) {
+            down_last<CMP>(t, c, heap(mid), mid, buf, de, dL, dR);
+            put6(sh_x, tid, dR);
+#pragma unroll
+            for (int I = 0; I < 6; ++I) de[I] = dL[I];
+          }
+          down_last<CMP>(t, c, heap(3 + q), 3 + q, buf, de, nullptr, nullptr);
+          if (!(q & 1)) get6(sh_x, tid, de);
+          else if (q == 1) get6(sd, tid, de);
+        }
+      }
+      if (tid < nP && last) {
+        done(DMN_STATUS_OK);
+        sh_fl[tid] &= B_CUR;
+      }
+      __syncthreads();
+      write_out();
+      __syncthreads();
     }
     __syncthreads();
   }
