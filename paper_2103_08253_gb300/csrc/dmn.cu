@@ -6,16 +6,16 @@
 //              interpolated angles, spherical normal; Sec. 2.3) and the macro
 //              strain in the principal frame;
 //   the Newton iteration of Sec. 3.2.  FP64 form, depth 3 and more: k_newton_block
-//              (csrc/dmn_block.cu), then k_newton or k_newton_warp on the points it hands back.
+//              (csrc/dmn_block.cu), then k_newton_list (csrc/dmn_warp.cu) on the points it hands back.
 //              Otherwise k_newton, persistent, one thread per point slot -- a lane that converges
 //              takes the next point from a global counter at once, so lanes stay busy
 //              although points need different numbers of Newton steps -- or, for small calls,
 //              k_newton_warp (csrc/dmn_warp.cu);
-//   k_sweep_block  (FP64 and mixed form, depth 3 and more) stress and tangent by one FP64
-//              condensation at the converged jumps, rotated back to the global frame;
+//   k_sweep_block  (FP64 form after k_newton_block; mixed form where sweep_block_on says) stress and tangent
+//              by one FP64 condensation at the converged jumps, rotated back to the global frame;
 //   k_final    one thread per point (small calls: several), for what the sweep does not write: the
 //              return mapping at the converged jumps gives z^{n+1}, and stress and tangent are rotated back
-//              to the global frame; below depth 3 the mixed form's FP64 sweep runs here.
+//              to the global frame; where k_sweep_block does not run, the mixed form's FP64 sweep runs here.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -1275,8 +1275,8 @@ int warp_lanes_for(const dmn_handle* h, int64_t n) {
   return h->opt.precision == DMN_PREC_F64 ? 8 : 16;
 }
 
-// The CTA organisation (csrc/dmn_block.cu) takes trees of depth 3 or more (its subtrees), whatever the call's
-// size: the FP64 form's Newton iteration from the paper's start, and every FP64 sweep.
+// The CTA organisation (csrc/dmn_block.cu) takes trees of depth 3 or more (its subtrees): the FP64 form's Newton
+// iteration from the paper's start (block_on) and its sweep, the mixed form's sweep (sweep_block_on), the adjoints.
 bool block_trees(const dmn_handle* h) {
   for (const Tree& t : h->trees)
     if (t.K < 3 || t.N < 1) return false;
@@ -1398,7 +1398,10 @@ bool sweep_block_on(const dmn_handle* h, int64_t n) {
 // condensation after the first stage, depth 8, 16 warps per SM (77824 lanes): 50001 points 11.5 ms with all, 8.6
 // ms with 11 warps (a point per lane); 100003 points 19.4 with all, 18.5, 17.8, 15.9, 17.4 ms with 10 .. 13 (two
 // points per lane and a margin of 15 % for uneven iteration counts: 12); 262144 points 39.0 with all, 40 to 41
-// with fewer.  The first stage waits on memory more than it issues: 5.7 -> 5.4 ms at a point per lane, but 12.0
+// with fewer.  Whole calls of the FP32-tangent variant, all lanes against the rule: 45000 points of depth 8 21.3 and
+// 18.6 ms, depth 5 2.39 and 2.08, depth 3 0.69 and 0.59; 60000 points 23.5 and 22.0, 2.68 and 2.46, 0.78 and 0.71;
+// 85000 points, the worst place of the rule, 33.2 and 32.6, 3.79 and 3.83, 1.03 and 1.04; 120000 points 39.7 and
+// 39.2, 4.75 and 4.69, 1.30 and 1.30.  The first stage waits on memory more than it issues: 5.7 -> 5.4 ms at a point per lane, but 12.0
 // instead of 11.0 ms at two (`waves`: the largest number of points per lane that gains).
 unsigned even_warps_per_sm(int64_t n, int n_sm, int warps, int waves) {
   const int64_t per_warp_row = (int64_t)32 * n_sm, lanes = per_warp_row * warps;

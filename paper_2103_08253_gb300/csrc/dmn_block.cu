@@ -50,7 +50,8 @@ constexpr double LEFT_MAX = 4.0;
 // and is taken off also where it meets the criterion, unless it is at the rounding of FP64 stresses (times the root's)
 constexpr double ROUNDING = 1e-15;
 // What the second solve leaves at least, as a part of the residual it starts from: the pairs' 46 bits, less some for
-// the sums that cancel.
+// the sums that cancel.  (Without it elastic points at criteria of 1e-15 took a counted correction more than with
+// the all-FP64 solve.)
 constexpr double PAIR_LEFT = 9.1e-13;   // 2^-40
 constexpr int BLOCK_ITERS = 16;
 
@@ -1027,7 +1028,7 @@ static __device__ void newton(const BlockParams& P) {
       }
       for (int b = nb - 1; b >= 0; --b) q2 += __shfl_xor_sync(0xffffffffu, q2, nP << b);
       if (!(s & ((1 << nb) - 1))) sh_r[(s >> nb) * nP + p] = (double)q2;
-      __syncthreads();
+      const bool ends = __syncthreads_or(last);
       if (tid < nP) {
         int f = sh_fl[tid] & ~B_CONV;
         if ((f & B_CONT) && !last) {
@@ -1043,7 +1044,7 @@ static __device__ void newton(const BlockParams& P) {
         sh_fl[tid] = f;
       }
       // ---- an elastic point's second part ends with the jumps: no more A
-      if (!__syncthreads_or(last)) continue;
+      if (!ends) continue;
       const int buf = LS && (fl & B_CUR) ? D_A2 : D_A;
       if (tid == 0) M.n_out = 0;
       if (last && s == 0) {

@@ -1126,7 +1126,7 @@ __device__ inline void write_leaf_states(const TreeDev& t, const double Eloc[6],
 }
 
 // The part of write_leaf_states (heap trees) or write_leaf_states_c (compressed ones) below position
-// `part` of level s + 1, s = 1 .. K - 1: the strain is carried from the root to that position (the same
+// `part` of level s + 1, s = 0 .. K - 1: the strain is carried from the root to that position (the same
 // operations as in the whole walk, so the states are the same), then depth first through the subtree.
 // Compressed trees are walked by heap positions: one that holds no laminate hands its strain on.
 __device__ inline void write_leaf_states_part(const TreeDev& t, const double Eloc[6], const PointArrays& P,
