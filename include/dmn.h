@@ -274,7 +274,7 @@ int dmn_update(dmn_handle* h, int64_t n, const int32_t* tree_id, const double* l
  * Unlike dmn_update, state_out may be state_in itself (each point's state is
  * read before it is written), and a point of an unknown tree (status
  * BAD_TREE) gets its state_in as state_out.  The points are processed in chunks of `chunk`
- * points (<= 0: twice the resident lanes of the Newton kernel) through two
+ * points (<= 0: twice the resident lanes of the thread-per-point kernel's shape) through two
  * stages of device buffers owned by the handle, on streams of the handle: the
  * copy-in of chunk j+1 and the copy-out of chunk j-1 overlap the update of
  * chunk j, and the updates of consecutive chunks may overlap (the two stages
